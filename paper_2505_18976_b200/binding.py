@@ -1,9 +1,14 @@
-"""Thin ctypes binding of ``libgrass_b200.so`` (declared in ``include/grass.h``).
+"""Thin binding of ``libgrass_b200.so`` (declared in ``include/grass.h``).
 
 Argument marshalling only: every step of the compression path runs in the CUDA
 kernels behind the C ABI.  Functions take torch CUDA tensors (or raw integer
 device pointers) and enqueue on torch's current stream.  There is no CPU
 fallback: if the shared library is missing, loading raises.
+
+The calls that a training or attribution loop makes go through the ``_native``
+extension first (``csrc/binding_native.cpp``): it marshals ordinary CUDA tensors
+and returns None for anything else, which the ctypes code here then takes, with
+its checks and exceptions.
 """
 from __future__ import annotations
 
@@ -56,11 +61,19 @@ class FactgrassLayer(ctypes.Structure):
 
 
 _lib = None
+_native = None
+
+
+def _fast():
+    """The compiled marshalling of the ordinary calls, bound to the loaded library."""
+    if _lib is None:
+        lib()
+    return _native
 
 
 def lib() -> ctypes.CDLL:
     """Load the CUDA library; raises if it has not been built (no fallback exists)."""
-    global _lib
+    global _lib, _native
     if _lib is None:
         if not os.path.exists(SO_PATH):
             raise ImportError(f"{SO_PATH} is missing: build it with `python -m paper_2505_18976_b200.build` "
@@ -120,6 +133,11 @@ def lib() -> ctypes.CDLL:
         L.grass_set_tuning.argtypes = [ctypes.c_int, i64]
         L.grass_status_string.restype = ctypes.c_char_p
         L.grass_status_string.argtypes = [st]
+        from . import _native as native     # built beside the library; missing = not built, no fallback
+        native.bind(GrassError, *(ctypes.cast(getattr(L, f), vp).value for f in (
+            "grass_compress_out", "factgrass_compress", "factgrass_compress_varlen", "factgrass_compress_grouped_out",
+            "factgrass_compress_grouped_varlen", "grass_score", "grass_score_bf16")))
+        _native = native
         _lib = L
     return _lib
 
@@ -205,6 +223,9 @@ def grass_compress(g: torch.Tensor, idx: Optional[torch.Tensor], k: int, s: int,
     idx: uint32/int32 CUDA tensor of ascending coordinates, or None for the identity mask.
     g may be a pinned host tensor: the kernel then reads the masked elements in place, across the bus.
     The rows are written as fp32, or as bf16 (rounded once, at the final store) when `out` / `out_dtype` is bf16."""
+    r = _fast().grass_compress(g, idx, k, s, seed, out, p, dev_status, out_dtype)
+    if r is not None:
+        return r
     _need_device_readable(g)
     _need_cuda(idx, out, dev_status)
     _need_mask(idx)
@@ -226,6 +247,9 @@ def factgrass_compress(A: torch.Tensor, G: torch.Tensor, mask_in: torch.Tensor, 
                        k: int, s: int, seed: int, out: Optional[torch.Tensor] = None,
                        dev_status: Optional[torch.Tensor] = None) -> torch.Tensor:
     """One linear layer: out[b] = SJLT(vec(sum_t A[b,t,mask_in] (x) G[b,t,mask_out]))."""
+    r = _fast().factgrass_compress(A, G, mask_in, mask_out, k, s, seed, out, dev_status)
+    if r is not None:
+        return r
     _need_device_readable(A, G)
     _need_cuda(mask_in, mask_out, out, dev_status)
     _need_mask(mask_in, mask_out)
@@ -259,6 +283,10 @@ def factgrass_compress_varlen(A: torch.Tensor, G: torch.Tensor, mask_in: torch.T
     """One linear layer, samples with their own sequence lengths.  A, G: token-major (rows, d) matrices
     (or (B, T_max, d) for a padded batch); sample b owns rows tok_begin[b] .. + tok_count[b] (int64 /
     int32 CUDA tensors; None = b * T_max / T_max)."""
+    r = _fast().factgrass_compress_varlen(A, G, mask_in, mask_out, k, s, seed, B, T_max, tok_begin, tok_count, out,
+                                          dev_status)
+    if r is not None:
+        return r
     _need_device_readable(A, G)
     _need_cuda(mask_in, mask_out, out, dev_status)
     _need_mask(mask_in, mask_out)
@@ -287,6 +315,11 @@ class GroupedLayers:
         self.keep = list(layers)
         self.L = len(layers)
         self.array = (FactgrassLayer * max(self.L, 1))()
+        self.addr = ctypes.addressof(self.array)
+        r = _fast().fill_layers(self.keep, self.addr)
+        if r is not None:
+            self.dtype, self.B, self.T = r
+            return
         for i, l in enumerate(layers):
             _need_device_readable(l["A"], l["G"])
             _need_cuda(l["mask_in"], l["mask_out"])
@@ -321,6 +354,9 @@ def factgrass_compress_grouped(group: GroupedLayers, out: torch.Tensor, workspac
                                dev_status: Optional[torch.Tensor] = None) -> torch.Tensor:
     """All layers of ``group`` in one launch; layer l fills out[:, off_l : off_l + k_l].  `out` is fp32, or bf16
     (every output rounded once, at the final store; see factgrass_compress_grouped_out in include/grass.h)."""
+    r = _fast().factgrass_compress_grouped(group.addr, group.L, group.dtype, group.B, group.T, out, workspace, dev_status)
+    if r is not None:
+        return r
     _need_cuda(out, workspace, dev_status)
     assert out.dtype in (torch.float32, torch.bfloat16) and out.stride(1) == 1
     _check(lib().factgrass_compress_grouped_out(group.array, group.L, group.dtype, group.B, group.T, _ptr(out),
@@ -336,6 +372,10 @@ def factgrass_compress_grouped_varlen(group: GroupedLayers, out: torch.Tensor, w
                                       dev_status: Optional[torch.Tensor] = None) -> torch.Tensor:
     """All layers of ``group`` in one launch for a batch whose samples have their own lengths; the layers'
     A and G are token-major (rows, d) matrices that share one token layout (tok_begin, tok_count)."""
+    r = _fast().factgrass_compress_grouped_varlen(group.addr, group.L, group.dtype, B, T_max, out, workspace, tok_begin,
+                                                  tok_count, dev_status)
+    if r is not None:
+        return r
     _need_cuda(out, workspace, dev_status)
     _check_token_arrays(tok_begin, tok_count, B)
     assert out.dtype == torch.float32 and out.stride(1) == 1 and out.shape[0] == B
@@ -366,6 +406,9 @@ def factgrass_compress_grouped_static(group: GroupedLayers, out: torch.Tensor,
 
 def grass_score(train: torch.Tensor, test: torch.Tensor, out: Optional[torch.Tensor] = None) -> torch.Tensor:
     """scores[i, m] = <train[i], test[m]> (fp32)."""
+    r = _fast().grass_score(train, test, out)
+    if r is not None:
+        return r
     _need_cuda(train, test, out)
     assert train.dtype == torch.float32 and test.dtype == torch.float32
     assert train.stride(1) == 1 and test.stride(1) == 1
@@ -397,6 +440,9 @@ def grass_to_bf16(x: torch.Tensor, out: Optional[torch.Tensor] = None) -> torch.
 
 def grass_score_bf16(train: torch.Tensor, test: torch.Tensor, out: Optional[torch.Tensor] = None) -> torch.Tensor:
     """scores[i, m] = <train[i], test[m]> for bf16 vectors (fp32 scores)."""
+    r = _fast().grass_score_bf16(train, test, out)
+    if r is not None:
+        return r
     _need_cuda(train, test, out)
     assert train.dtype == torch.bfloat16 and test.dtype == torch.bfloat16
     assert train.stride(1) == 1 and test.stride(1) == 1
