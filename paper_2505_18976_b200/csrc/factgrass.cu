@@ -25,9 +25,7 @@ namespace grass {
 
 // What happens to the finished k'_in x k'_out block.
 constexpr int kEpiSjlt = 0;   // FactGraSS stage 3: hash every entry into the k-bin accumulator
-constexpr int kEpiBlock = 2;  // factorised Mask alone (Section 3.2): add the block itself into out[b, off + a*kout + c]
-constexpr int kEpiRaw = 1;    // add scale * block into a dense symmetric matrix (projected FIM, see grass_fim.cu):
-                              // only tiles on or above the diagonal are computed, the others are mirrored
+constexpr int kEpiBlock = 1;  // factorised Mask alone (Section 3.2): add the block itself into out[b, off + a*kout + c]
 
 // TM x TN block tile of C per CTA (TM = MMA M: masked input coordinates, TN = MMA N: masked output
 // coordinates, contraction over tokens).  F32: fp32 inputs, split exactly into three bf16 pieces.
@@ -69,7 +67,6 @@ factgrass_kernel(const LayerDesc* __restrict__ descs, const __grid_constant__ La
     if (L.tiles_m <= 0 || L.tiles_n <= 0) return;
     const int tm = tile % L.tiles_m, tn = tile / L.tiles_m;
     if (tn >= L.tiles_n) return;
-    if (EPI == kEpiRaw && tn < tm) return;
     const int kin = L.kin, kout = L.kout;
     const int64_t d_in = L.d_in, d_out = L.d_out;
     const uint32_t k = L.k;
@@ -224,13 +221,6 @@ factgrass_kernel(const LayerDesc* __restrict__ descs, const __grid_constant__ La
     auto project = [&](int a, int c, float val) {
         if constexpr (EPI == kEpiBlock) {
             if (a < kin && c < kout && val != 0.0f) atomicAdd(orow + (int64_t)a * kout + c, val);
-        } else if constexpr (EPI == kEpiRaw) {
-            // tiles above the diagonal fill their mirror image too; a diagonal tile uses its upper half
-            if (a < kin && c < kout && (tm != tn || a <= c)) {
-                const float sv = val * L.scale;
-                atomicAdd(out + (int64_t)a * ld_out + c, sv);
-                if (a != c) atomicAdd(out + (int64_t)c * ld_out + a, sv);
-            }
         } else if (a < kin && c < kout && val != 0.0f) {
             const uint64_t q = (uint64_t)a * (uint64_t)kout + (uint64_t)c;
             for (uint32_t r = 0; r < s; ++r) {
@@ -337,7 +327,6 @@ static grass_status fill_desc(LayerDesc& d, const factgrass_layer& l, int tile, 
     d.tiles_m = (l.kin + tile - 1) / tile;
     d.tiles_n = (l.kout + tile - 1) / tile;
     d.use_smem_bins = (size_t)l.spec.k * sizeof(float) <= kMaxSmemBins;
-    d.scale = 1.0f;
     return GRASS_OK;
 }
 
@@ -364,7 +353,7 @@ static grass_status run_factgrass(const factgrass_layer* layers, int32_t L, gras
             return GRASS_ERR_INVALID_ARG;
     }
     // 64 x 64 block tiles; larger blocks are covered by several tiles whose shared rows come from L2.
-    // The 128 x 128 variant serves the projected FIM and comparison runs (GRASS_TUNE_FACTGRASS_TILE = 128).
+    // The 128 x 128 variant serves comparison runs (GRASS_TUNE_FACTGRASS_TILE = 128).
     const int tile = tuning(GRASS_TUNE_FACTGRASS_TILE, 64) == 128 && max_kk > 64 ? 128 : 64;
 
     if (!workspace && L != 1) return GRASS_ERR_INVALID_ARG;
@@ -548,51 +537,6 @@ static grass_status run_factmask(const factgrass_layer* layers, int32_t L, grass
     }
     return run_factgrass(tmp.data(), L, dt, B, T, nullptr, nullptr, out, ld_out, workspace, workspace_bytes, dev_status,
                          st, kEpiBlock);
-}
-
-// Projected Fisher information matrix F = scale * X^T X of the n rows of X (n x k fp32, row stride ld):
-// the Kronecker-sum contraction of the FactGraSS kernel with both factors = X, identity masks and the
-// raw-block epilogue.  F (k x k, row stride ld_f) must have been zeroed on the stream.
-grass_status launch_fim(const float* X, int64_t n, int64_t k, int64_t ld, float scale, float* F, int64_t ld_f,
-                        cudaStream_t st)
-{
-    constexpr int tile = 128;
-    LayerDesc d;
-    std::memset(&d, 0, sizeof d);
-    d.A = X;
-    d.G = X;
-    d.d_in = d.d_out = (int32_t)ld;
-    d.kin = d.kout = (int32_t)k;
-    d.tiles_m = d.tiles_n = (int32_t)((k + tile - 1) / tile);
-    d.scale = scale;
-    int dev = 0, sms = 148;
-    if (cudaGetDevice(&dev) != cudaSuccess) return GRASS_ERR_CUDA;
-    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return GRASS_ERR_CUDA;
-    auto kern = factgrass_kernel<tile, tile, true, kEpiRaw>;
-    const size_t smem = kFgBufs * 3 * (size_t)tile * tc::ROW_BYTES * 2;
-    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
-        return GRASS_ERR_CUDA;
-    const int per_sm = 2;   // 97 KB of shared memory and 256 tensor-memory columns per CTA; 196 KB carve-out
-    if (cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, 85) != cudaSuccess)
-        return GRASS_ERR_CUDA;
-    // sample chunks: enough CTAs for ~4 waves of the tiles on or above the diagonal, at least 256 samples each
-    const int64_t tiles = (int64_t)d.tiles_m * (d.tiles_m + 1) / 2;
-    int64_t want = (4 * (int64_t)sms * per_sm + tiles - 1) / tiles;
-    const int64_t max_chunks = (n + 255) / 256;
-    want = std::max<int64_t>(want, (n + 8191) / 8192);   // bounded accumulation runs, as for the token chunks
-    if (want > max_chunks) want = max_chunks;
-    if (want < 1) want = 1;
-    int64_t chunk_len = (n + want - 1) / want;
-    chunk_len = (chunk_len + kTokTile - 1) / kTokTile * kTokTile;
-    const int64_t nchunks = (n + chunk_len - 1) / chunk_len;
-    const int64_t gx = nchunks * d.tiles_m * d.tiles_n;
-    if (gx > 0x7FFFFFFFLL || chunk_len > 0x7FFFFFFFLL) return GRASS_ERR_UNSUPPORTED;
-    dim3 grid((unsigned)gx, 1, 1);
-    int nprod = (int)tuning(GRASS_TUNE_SPLIT_PRODUCTS, tc::kSplitProductsDefault);
-    if (nprod != 3 && nprod != 4) nprod = 6;
-    kern<<<grid, kFgThreads, smem, st>>>(nullptr, d, 1, (int32_t)n, nullptr, nullptr, d.tiles_m * d.tiles_n,
-                                         (int32_t)chunk_len, F, ld_f, nullptr, nprod, 0);
-    return launch_status();
 }
 
 }  // namespace grass

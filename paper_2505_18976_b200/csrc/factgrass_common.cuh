@@ -24,7 +24,7 @@ struct LayerDesc {
     int64_t out_offset;
     int32_t tiles_m, tiles_n;
     int32_t use_smem_bins;
-    float scale;   // raw-block epilogue: factor applied to every entry
+    int32_t pad;
 };
 static_assert(sizeof(LayerDesc) == 88, "descriptor layout");
 
