@@ -90,3 +90,47 @@ def test_preconditioned_score(G, oracle_mod):
     cond = np.linalg.cond(oracle_mod.fim(th)[0] + lam * np.eye(k))
     scale = np.linalg.norm(ref, axis=0, keepdims=True) / np.sqrt(n)
     assert (np.abs(sc - ref) / scale).max() <= 64 * cond * 2.0 ** -23
+
+
+# Sizes at which the one-launch kernels change shape: one block, one block and a row, a last block of one row; the first
+# trailing update just within / beyond one thread block per tile (k = 1,088 / 1,152); clusters of 1, 2, 4, 8 and
+# 2 .. 32 right-hand sides each; row strides that rule out 16-byte loads.
+@pytest.mark.parametrize("k,M,pad", [(1, 1, 0), (63, 2, 1), (64, 40, 0), (65, 5, 3), (128, 600, 4), (129, 33, 1), (320, 1, 0),
+                                     (576, 130, 2), (1088, 260, 0), (1152, 300, 1), (1345, 37, 4), (256, 5000, 0)])
+def test_factor_and_apply_shapes(G, k, M, pad):
+    n = 2 * k + 3
+    X = _compressed(n, k, 40 + k)
+    wide = torch.full((k, k + pad), float("nan"), device="cuda")
+    F = wide[:, :k]
+    G.grass_fim(X, out=F)
+    A = torch.tril(F).double()
+    A = A + torch.tril(A, -1).T + 0.05 * torch.eye(k, device="cuda", dtype=torch.float64)
+    st = torch.zeros(1, dtype=torch.int32, device="cuda")
+    G.grass_fim_factor(F, 0.05, dev_status=st)
+    wide_b = torch.full((M, k + pad), float("nan"), device="cuda")
+    Bm = wide_b[:, :k]
+    Bm.copy_(_compressed(M, k, 41 + k))
+    b = Bm.double()
+    G.grass_fim_apply(F, Bm)
+    assert int(st.item()) == 0
+    assert pad == 0 or (torch.isnan(wide[:, k:]).all() and torch.isnan(wide_b[:, k:]).all())
+    # backward error of a factorisation and two substitutions with k-term fp32 sums: rounding errors of independent
+    # sign add like sqrt(k) 2^-24, three passes, two standard deviations
+    u = 6.0 * k ** 0.5 * 2.0 ** -24
+    L = torch.tril(F).double()
+    assert (L @ L.T - A).norm() <= u * A.norm()
+    x = Bm.double()
+    assert (x @ A - b).norm() <= u * A.norm() * x.norm()
+
+
+# one sample, fewer samples than a step, a chunk boundary at 8,192; tiles on the diagonal alone, a ragged second tile, many
+# tiles (pairs instead of clusters of eight); columns that start off a 16-byte boundary
+@pytest.mark.parametrize("n,k,off", [(1, 128, 0), (31, 129, 0), (33, 127, 1), (8_192, 64, 0), (8_200, 200, 3), (700, 900, 0)])
+def test_fim_shapes(G, n, k, off):
+    X = _compressed(n, k + off + 3, 60 + k)[:, off:off + k]
+    F = G.grass_fim(X).double()
+    Xd = X.double()
+    ref, absum = Xd.T @ Xd / n, Xd.abs().T @ Xd.abs() / n
+    # six bf16 products keep each product to 2^-23; accumulators are truncated once per 16 samples
+    assert ((F - ref).abs() <= 2.0 ** -22 * absum + 2.0 * (n / 16 + 64) ** 0.5 * 2.0 ** -23 * absum).all()
+    assert (F - F.T).abs().max() <= 2.0 ** -21 * absum.max()
