@@ -16,6 +16,8 @@
 
 #include <cooperative_groups.h>
 
+#include <algorithm>
+
 namespace cg = cooperative_groups;
 
 namespace grass {
@@ -368,24 +370,40 @@ static CompressPlan plan_compress(int64_t n, int64_t kprime, uint32_t k, int sm_
     if (S == 1 && !dense && tuning(GRASS_TUNE_COMPRESS_LOADS, 8) == 16) U = 16;
     pl.U = U;
     const int64_t groups = (n + S - 1) / S;
+    // With a row for every SM, a thread block of up to 1,024 threads takes a whole row in one round of loads: no
+    // position split, so no cluster, no exchange of bins and no thread blocks left waiting for a slot
+    // (256 x 65,536, k' = 8,192: 25.2 -> 22.9 us).  Everything else runs 512 threads: the loads in flight per SM come
+    // from resident threads, and a few long rows then keep the machine busy (61 rows of k' = 32,768: 55 us with
+    // 256 threads, 33 us with 512).
     pl.threads = kThreads;
+    bool whole = false;
     if (!dense) {
-        // With a row for every SM, a thread block of up to 1,024 threads takes a whole row in one round of loads:
-        // no position split, so no cluster, no exchange of bins and no thread blocks left waiting for a slot
-        // (config 1: 25.2 -> 22.9 us).  Longer masks and fewer rows keep 256 threads and split the positions.
-        int t = kThreads;
-        if (S == 1 && groups >= sm_count && kprime <= (int64_t)4 * kThreads * U)
+        whole = S == 1 && groups >= sm_count && kprime <= (int64_t)4 * kThreads * U;
+        int t = whole ? kThreads : 2 * kThreads;
+        if (whole)
             while ((int64_t)t * U < kprime) t *= 2;
         t = (int)tuning(GRASS_TUNE_COMPRESS_THREADS, t);
-        if (t == 2 * kThreads || t == 4 * kThreads) pl.threads = t;
+        pl.threads = (t == 2 * kThreads || t == 4 * kThreads) ? t : kThreads;
     }
-    // split positions until there are ~4 CTAs per SM, but keep one full round of loads per CTA
+    // Split of the positions over a cluster of up to 8 thread blocks.  A block's share has to be worth its k bins (zeroed,
+    // exchanged and stored): at least k positions, or k / 2 while there are fewer blocks than SMs, and at least 1,024
+    // (one row of k' = 8,192, k = 2,048: 8.2 us over 4 blocks, 6.2 us over 8; 512 rows of k' = 65,536: 345 us
+    // over 2 blocks, 332 us over 8).  Streamed rows keep one full round of loads per block.
     const int64_t round = (int64_t)pl.threads * U;
-    const int64_t max_js = kprime / round > 0 ? kprime / round : 1;
     int64_t js = 1;
-    while (js < 8 && groups * js < (int64_t)sm_count * 4 && js * 2 <= max_js) js *= 2;
+    if (dense) {
+        const int64_t max_js = std::max<int64_t>(1, kprime / round);
+        while (js < 8 && groups * js < (int64_t)sm_count * 4 && js * 2 <= max_js) js *= 2;
+    } else if (!whole) {
+        while (js < 8) {
+            const int64_t share = kprime / (js * 2);
+            if (share < 1024 || share < (int64_t)(groups * js < sm_count ? k / 2 : k)) break;
+            js *= 2;
+        }
+    }
     pl.cluster = 1;
-    if (groups * js < sm_count && js * 2 <= max_js) {
+    const int64_t max_js = std::max<int64_t>(1, kprime / ((int64_t)kThreads * U));
+    if (groups * js < sm_count && js * 2 <= max_js && js == 8) {
         // very few samples: split wider than a cluster allows and reduce with global atomics
         js = ((int64_t)sm_count * 2 + groups - 1) / groups;
         if (js > max_js) js = max_js;
