@@ -28,13 +28,10 @@
 // adds its partial products into the zeroed output (see launch_score_tc).
 // The TMA path needs 16-byte aligned bases and row strides; other inputs take the plain FMA kernel
 // (grass_score.cu).
-#include <cuda.h>
-
 #include <algorithm>
 #include <cstdlib>
 
-#include "grass_common.cuh"
-#include "tcgen05_util.cuh"
+#include "score_common.cuh"
 
 namespace grass {
 namespace tc {
@@ -66,74 +63,6 @@ constexpr int RAW_BYTES = 2 * RAW_HALF;          // train tile + this CTA's test
 constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + RING * RAW_BYTES;
 static_assert(BM == BNH, "both raw tiles use the same TMA box");
 static_assert(SMEM_BYTES <= 224 * 1024 && STAGE_BYTES % 1024 == 0 && RAW_HALF % 1024 == 0, "shared memory layout");
-
-__device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes)
-{
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
-}
-// 2-D tiled TMA load into this CTA's shared memory; x = first k-value (a multiple of 32: 128 bytes), y = first row
-__device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map, int32_t x, int32_t y, uint32_t bar)
-{
-    asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
-                 ::"r"(dst), "l"(map), "r"(x), "r"(y), "r"(bar)
-                 : "memory");
-}
-
-__device__ __forceinline__ uint32_t cluster_ctarank()
-{
-    uint32_t r;
-    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-    return r;
-}
-// address of the same shared-memory location in CTA `rank` of the cluster
-__device__ __forceinline__ uint32_t map_to_cta(uint32_t local_addr, uint32_t rank)
-{
-    uint32_t ra;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(ra) : "r"(local_addr), "r"(rank));
-    return ra;
-}
-__device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_addr)
-{
-    asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
-}
-// bounded wait with cluster-scope acquire (the arrivals come from both CTAs)
-__device__ __forceinline__ bool mbar_wait_cluster(uint32_t bar, uint32_t parity)
-{
-    for (uint32_t it = 0; it < SPIN_LIMIT; ++it) {
-        uint32_t done;
-        asm volatile(
-            "{\n\t.reg .pred P;\n\t"
-            "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 P, [%1], %2;\n\t"
-            "selp.u32 %0, 1, 0, P;\n\t}"
-            : "=r"(done)
-            : "r"(bar), "r"(parity)
-            : "memory");
-        if (done) return true;
-    }
-    return false;
-}
-__device__ __forceinline__ void umma_bf16_pair(uint32_t tmem_d, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
-                                               uint32_t accumulate)
-{
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-        ::"r"(tmem_d), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
-        : "memory");
-}
-// arrives on the barrier at this shared-memory offset in both CTAs once all MMAs issued so far are done
-__device__ __forceinline__ void umma_commit_pair(uint32_t bar)
-{
-    const uint16_t mask = 3;
-    asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;"
-                 ::"r"(bar), "h"(mask)
-                 : "memory");
-}
-__device__ __forceinline__ void cluster_sync_all()
-{
-    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
 
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
 grass_score_tc_kernel(const __grid_constant__ CUtensorMap map_train, const __grid_constant__ CUtensorMap map_test,
@@ -329,7 +258,8 @@ grass_score_tc_kernel(const __grid_constant__ CUtensorMap map_train, const __gri
             const uint32_t round = (uint32_t)(kt / STAGES);
             ok = mbar_wait_cluster(full0 + 8 * s, round & 1) && !abort_flag;
             if (!ok) break;
-            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            // (the only thing other threads hand over here are operand stores, made visible to the tensor core by their
+            // fence.proxy.async and the barrier; no tensor-memory access of another thread has to be ordered)
             const uint32_t a0 = smem_base + s * STAGE_BYTES, b0 = a0 + 3 * A_SPLIT_BYTES;
             // hi*hi goes to the first accumulator, the correction terms (2^-8 and 2^-16 of it) to the second:
             // the tensor core truncates after every accumulation, so the large sum should see as few of
@@ -360,416 +290,7 @@ grass_score_tc_kernel(const __grid_constant__ CUtensorMap map_train, const __gri
     }
 }
 
-
-// ---------------------------------------------------------------------------------------------------------
-// The same contraction for vectors already stored as bf16 (a cache of compressed gradients at half the size):
-// no split is needed, so there are no producer warps at all.  TMA writes the bf16 tiles (128 rows x 64 k-values,
-// 128-byte rows, 128-byte swizzle) straight into the K-major operand layout the tensor core reads; per CTA one warp issues the
-// loads, one forwards "my tiles have landed" to the leader CTA's barriers, one thread of the leader issues the
-// MMAs (one product per 16 k-values), four warps drain the accumulator.
-constexpr int H_STAGES = 7;
-constexpr int H_BK = 64;                                 // k-values per stage: 128-byte rows, 128-byte swizzle
-constexpr int H_ROW_BYTES = H_BK * 2;
-constexpr int H_A_BYTES = BM * H_ROW_BYTES;              // this CTA's 128 train rows x 64 k-values of bf16: 16 KB
-constexpr int H_B_BYTES = BNH * H_ROW_BYTES;             // this CTA's half of the test rows: 16 KB
-constexpr int H_STAGE_BYTES = H_A_BYTES + H_B_BYTES;
-constexpr int H_BOX_ROWS = 128;                          // rows per TMA box
-constexpr int H_BOXES = BM / H_BOX_ROWS;                 // boxes per operand tile
-constexpr int H_EPI_WARPS = 4;
-constexpr int H_THREADS = (H_EPI_WARPS + 3) * 32;        // + MMA / tensor-memory warp, TMA warp, forwarding warp
-constexpr uint32_t H_TMEM_COLS = 256;                    // one fp32 accumulator of BN columns
-static_assert(H_STAGE_BYTES % 1024 == 0 && H_A_BYTES % 1024 == 0, "operand tiles stay 1024-byte aligned");
-static_assert(H_STAGES <= 32 && 2 * H_BOXES <= 32 && BM == BNH && (H_BOX_ROWS * H_ROW_BYTES) % 1024 == 0,
-              "one stage and one box per lane");
-static_assert(H_STAGES * H_STAGE_BYTES <= 224 * 1024, "shared memory");
-
-// shared-memory matrix descriptor for K-major tiles with 128-byte rows and the 128-byte swizzle (8-row groups
-// 1,024 bytes apart; 16-byte chunk c of row r stored at chunk c ^ (r & 7)); a descriptor that starts 32 * i bytes
-// into the tile addresses k-values 16 i .. 16 i + 15
-__device__ __forceinline__ uint64_t make_smem_desc_sw128(uint32_t addr)
-{
-    return (uint64_t)((addr >> 4) & 0x3FFF) | (1ull << 16) | ((uint64_t)(1024 >> 4) << 32) | (1ull << 46) |
-           (2ull << 61);
-}
-
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(H_THREADS, 1)
-grass_score_bf16_kernel(const __grid_constant__ CUtensorMap map_train, const __grid_constant__ CUtensorMap map_test,
-                        int64_t N, int64_t M, int64_t D, int64_t kt_split, float* __restrict__ scores, int64_t ld_s,
-                        int out_vec_ok)
-{
-    extern __shared__ __align__(1024) unsigned char smem[];
-    __shared__ __align__(8) unsigned long long bars[3 * H_STAGES + 1];
-    __shared__ uint32_t tmem_base_slot;
-    __shared__ volatile int abort_flag;
-
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const uint32_t rank = cluster_ctarank();
-    const int64_t n0 = (int64_t)blockIdx.x * BM;
-    const int64_t m0 = (int64_t)blockIdx.y * BN;
-    const int64_t m_rows = (M - m0) < BN ? (M - m0) : BN;
-    const uint32_t n_mma = (uint32_t)((m_rows + 15) / 16 * 16);
-    const int n_half = (int)(n_mma / 2);
-    const int64_t kt0 = (int64_t)blockIdx.z * kt_split;
-    const int64_t kt_left = (D + H_BK - 1) / H_BK - kt0;
-    const int64_t ktiles = kt_left < kt_split ? (kt_left > 0 ? kt_left : 0) : kt_split;
-    const bool add_out = gridDim.z > 1;
-
-    // landed[s]: this CTA's two tiles of stage s have arrived; full[s] (used in the leader): both CTAs' tiles have;
-    // empty[s]: the MMAs that read stage s are done (both CTAs); accum: the accumulators are complete
-    const uint32_t landed0 = smem_u32(&bars[0]), full0 = smem_u32(&bars[H_STAGES]), empty0 = smem_u32(&bars[2 * H_STAGES]);
-    const uint32_t accum = smem_u32(&bars[3 * H_STAGES]);
-    if (tid == 0) {
-        for (int s = 0; s < H_STAGES; ++s) {
-            mbar_init(landed0 + 8 * s, 1);
-            mbar_init(full0 + 8 * s, 2);
-            mbar_init(empty0 + 8 * s, 1);
-        }
-        mbar_init(accum, 1);
-        abort_flag = 0;
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    }
-    if (warp == H_EPI_WARPS) {
-        asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base_slot)),
-                     "r"(H_TMEM_COLS)
-                     : "memory");
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
-    }
-    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-    __syncthreads();
-    cluster_sync_all();
-    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    const uint32_t tmem_d = tmem_base_slot;
-    const uint32_t smem_base = smem_u32(smem);
-
-    if (warp < H_EPI_WARPS) {
-        // ---------------- epilogue: this CTA's 128 rows of the accumulator ----------------
-        bool ok = true;
-        if (ktiles > 0) ok = mbar_wait(accum, 0) && !abort_flag;
-        if (!ok) abort_flag = 1;
-        ok = __all_sync(0xFFFFFFFFu, ok);
-        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        const int64_t row = n0 + warp * 32 + lane;
-        for (uint32_t c0 = 0; c0 < n_mma; c0 += 32) {
-            uint32_t v[32];
-            if (ok && ktiles > 0) {
-                tmem_ld32(tmem_d + ((uint32_t)(warp * 32) << 16) + c0, v);
-                asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-            } else {
-#pragma unroll
-                for (int e = 0; e < 32; ++e) v[e] = (ktiles > 0) ? 0x7FC00000u : 0u;   // NaN marks an aborted tile
-            }
-            if (row < N) {
-                float* dst = scores + row * ld_s + m0 + c0;
-                const bool vec = out_vec_ok && (int64_t)(c0 + 32) <= m_rows;
-                if (add_out) {
-                    if (vec) {
-#pragma unroll
-                        for (int e = 0; e < 32; e += 4)
-                            asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(dst + e),
-                                         "f"(__uint_as_float(v[e])), "f"(__uint_as_float(v[e + 1])),
-                                         "f"(__uint_as_float(v[e + 2])), "f"(__uint_as_float(v[e + 3]))
-                                         : "memory");
-                    } else {
-#pragma unroll
-                        for (int e = 0; e < 32; ++e)
-                            if ((int64_t)(c0 + e) < m_rows) atomicAdd(dst + e, __uint_as_float(v[e]));
-                    }
-                } else if (vec) {
-#pragma unroll
-                    for (int e = 0; e < 32; e += 4)
-                        *reinterpret_cast<uint4*>(dst + e) = make_uint4(v[e], v[e + 1], v[e + 2], v[e + 3]);
-                } else {
-#pragma unroll
-                    for (int e = 0; e < 32; ++e)
-                        if ((int64_t)(c0 + e) < m_rows) dst[e] = __uint_as_float(v[e]);
-                }
-            }
-        }
-    } else if (warp == H_EPI_WARPS + 1) {
-        // ---------------- TMA: bf16 tiles straight into the operand stages ----------------
-        // A tile arrives as H_BOXES boxes of H_BOX_ROWS rows, one box per lane.
-        const int32_t row_a = (int32_t)n0, row_b = (int32_t)(m0 + (int64_t)rank * n_half);
-        int64_t issued = 0;
-        bool ok = true;
-        for (int64_t kt = 0; kt < ktiles; ++kt) {
-            const int s = (int)(kt % H_STAGES);
-            const uint32_t round = (uint32_t)(kt / H_STAGES);
-            if (lane == 0) {
-                if (round > 0) ok = mbar_wait(empty0 + 8 * s, (round - 1) & 1) && !abort_flag;
-                if (ok) mbar_expect_tx(landed0 + 8 * s, H_STAGE_BYTES);
-            }
-            ok = __shfl_sync(0xFFFFFFFFu, ok ? 1 : 0, 0) != 0;
-            if (!ok) break;
-            if (lane < 2 * H_BOXES) {
-                const bool is_b = lane >= H_BOXES;
-                const int bx = is_b ? lane - H_BOXES : lane;
-                const uint32_t dst = smem_base + s * H_STAGE_BYTES + (is_b ? H_A_BYTES : 0) + bx * H_BOX_ROWS * H_ROW_BYTES;
-                tma_load_2d(dst, is_b ? &map_test : &map_train, (int32_t)((kt0 + kt) * H_BK),
-                            (is_b ? row_b : row_a) + bx * H_BOX_ROWS, landed0 + 8 * s);
-            }
-            issued = kt + 1;
-        }
-        if (!ok) abort_flag = 1;
-        // no copy of this CTA may still be in flight when it leaves
-        if (lane == 0)
-            for (int64_t kt = issued > H_STAGES ? issued - H_STAGES : 0; kt < issued; ++kt)
-                if (!mbar_wait(landed0 + 8 * (int)(kt % H_STAGES), (uint32_t)(kt / H_STAGES) & 1)) abort_flag = 1;
-    } else if (warp == H_EPI_WARPS + 2) {
-        // ---------------- forward "landed" to the leader CTA ----------------
-        // An arrival on another CTA's barrier takes about a microsecond to return, so one thread forwarding
-        // stage after stage would set the pace of the whole kernel.  Lane s looks after stage s instead: the
-        // arrivals of several stages are in flight together; every lane polls once per turn of the common loop.
-        const uint32_t leader_full0 = map_to_cta(full0, 0);
-        int64_t kt = lane;
-        bool active = lane < H_STAGES;
-        uint32_t spins = 0;
-        while (__any_sync(0xFFFFFFFFu, active && kt < ktiles)) {
-            if (active && kt < ktiles) {
-                uint32_t done;
-                asm volatile(
-                    "{\n\t.reg .pred P;\n\t"
-                    "mbarrier.try_wait.parity.shared::cta.b64 P, [%1], %2;\n\t"
-                    "selp.u32 %0, 1, 0, P;\n\t}"
-                    : "=r"(done)
-                    : "r"(landed0 + 8 * lane), "r"((uint32_t)(kt / H_STAGES) & 1)
-                    : "memory");
-                if (done) {
-                    mbar_arrive_cluster(leader_full0 + 8 * lane);
-                    kt += H_STAGES;
-                    spins = 0;
-                } else if (++spins > SPIN_LIMIT || abort_flag) {
-                    abort_flag = 1;
-                    active = false;
-                }
-            }
-        }
-    } else if (lane == 0 && rank == 0) {
-        // ---------------- MMA issuer (leader CTA only) ----------------
-        const uint32_t idesc = make_idesc(2 * BM, n_mma);
-        bool ok = true;
-        for (int64_t kt = 0; kt < ktiles && ok; ++kt) {
-            const int s = (int)(kt % H_STAGES);
-            ok = mbar_wait_cluster(full0 + 8 * s, (uint32_t)(kt / H_STAGES) & 1) && !abort_flag;
-            if (!ok) break;
-            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            const uint32_t a0 = smem_base + s * H_STAGE_BYTES, b0 = a0 + H_A_BYTES;
-#pragma unroll
-            for (int ks = 0; ks < H_BK / 16; ++ks)
-                umma_bf16_pair(tmem_d, make_smem_desc_sw128(a0 + ks * 32), make_smem_desc_sw128(b0 + ks * 32), idesc,
-                               (kt > 0 || ks > 0) ? 1u : 0u);
-            umma_commit_pair(empty0 + 8 * s);
-        }
-        if (!ok) abort_flag = 1;
-        if (ok && ktiles > 0) umma_commit_pair(accum);
-    }
-
-    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-    __syncthreads();
-    cluster_sync_all();
-    if (warp == H_EPI_WARPS) {
-        __syncwarp();
-        asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_d), "r"(H_TMEM_COLS) : "memory");
-    }
-}
-
-
-// ---------------------------------------------------------------------------------------------------------
-// bf16 scores with one thread block per 128 x (<= 256) output tile (tcgen05.mma.cta_group::1): for a test set that
-// fits one column tile (M <= 256, the usual attribute-stage shape) the pair kernel above gains nothing from sharing
-// the test tile between two SMs and pays a remote barrier arrival per stage.  Here every thread block brings in its
-// own 128 train rows and ALL test rows of a k tile (the test rows come from L2 after the first block has read
-// them), one warp issues the loads, one thread the MMAs, four warps drain the accumulator; all barriers are local.
-constexpr int S_STAGES = 4;
-constexpr int S_A_BYTES = BM * H_ROW_BYTES;              // 128 train rows x 64 k-values: 16 KB
-constexpr int S_B_BYTES = BN * H_ROW_BYTES;              // up to 256 test rows x 64 k-values: 32 KB
-constexpr int S_STAGE_BYTES = S_A_BYTES + S_B_BYTES;
-constexpr int S_THREADS = (H_EPI_WARPS + 2) * 32;        // + MMA / tensor-memory warp, TMA warp
-static_assert(S_STAGES * S_STAGE_BYTES <= 224 * 1024 && S_STAGE_BYTES % 1024 == 0, "shared memory");
-
-__global__ void __launch_bounds__(S_THREADS, 1)
-grass_score_bf16_solo_kernel(const __grid_constant__ CUtensorMap map_train, const __grid_constant__ CUtensorMap map_test,
-                             int64_t N, int64_t M, int64_t D, int64_t kt_split, float* __restrict__ scores,
-                             int64_t ld_s, int out_vec_ok)
-{
-    extern __shared__ __align__(1024) unsigned char smem[];
-    __shared__ __align__(8) unsigned long long bars[2 * S_STAGES + 1];
-    __shared__ uint32_t tmem_base_slot;
-    __shared__ volatile int abort_flag;
-
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int64_t n0 = (int64_t)blockIdx.x * BM;
-    const int64_t m0 = (int64_t)blockIdx.y * BN;
-    const int64_t m_rows = (M - m0) < BN ? (M - m0) : BN;
-    const uint32_t n_mma = (uint32_t)((m_rows + 15) / 16 * 16);    // MMA N (a multiple of 16 for M = 128)
-    const int b_boxes = n_mma > (uint32_t)H_BOX_ROWS ? 2 : 1;      // boxes of 128 test rows per stage
-    const int64_t kt0 = (int64_t)blockIdx.z * kt_split;
-    const int64_t kt_left = (D + H_BK - 1) / H_BK - kt0;
-    const int64_t ktiles = kt_left < kt_split ? (kt_left > 0 ? kt_left : 0) : kt_split;
-    const bool add_out = gridDim.z > 1;
-
-    // full[s]: the tiles of stage s have landed; empty[s]: the MMAs that read stage s are done; accum: all MMAs are
-    const uint32_t full0 = smem_u32(&bars[0]), empty0 = smem_u32(&bars[S_STAGES]), accum = smem_u32(&bars[2 * S_STAGES]);
-    if (tid == 0) {
-        for (int s = 0; s < S_STAGES; ++s) {
-            mbar_init(full0 + 8 * s, 1);
-            mbar_init(empty0 + 8 * s, 1);
-        }
-        mbar_init(accum, 1);
-        abort_flag = 0;
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    }
-    if (warp == H_EPI_WARPS) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base_slot)),
-                     "r"(H_TMEM_COLS)
-                     : "memory");
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-    }
-    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-    __syncthreads();
-    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    const uint32_t tmem_d = tmem_base_slot;
-    const uint32_t smem_base = smem_u32(smem);
-
-    if (warp < H_EPI_WARPS) {
-        // ---------------- epilogue: the 128 rows of the accumulator ----------------
-        bool ok = true;
-        if (ktiles > 0) ok = mbar_wait(accum, 0) && !abort_flag;
-        if (!ok) abort_flag = 1;
-        ok = __all_sync(0xFFFFFFFFu, ok);
-        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        const int64_t row = n0 + warp * 32 + lane;
-        for (uint32_t c0 = 0; c0 < n_mma; c0 += 32) {
-            uint32_t v[32];
-            if (ok && ktiles > 0) {
-                tmem_ld32(tmem_d + ((uint32_t)(warp * 32) << 16) + c0, v);
-                asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-            } else {
-#pragma unroll
-                for (int e = 0; e < 32; ++e) v[e] = (ktiles > 0) ? 0x7FC00000u : 0u;   // NaN marks an aborted tile
-            }
-            if (row < N) {
-                float* dst = scores + row * ld_s + m0 + c0;
-                const bool vec = out_vec_ok && (int64_t)(c0 + 32) <= m_rows;
-                if (add_out) {
-                    if (vec) {
-#pragma unroll
-                        for (int e = 0; e < 32; e += 4)
-                            asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(dst + e),
-                                         "f"(__uint_as_float(v[e])), "f"(__uint_as_float(v[e + 1])),
-                                         "f"(__uint_as_float(v[e + 2])), "f"(__uint_as_float(v[e + 3]))
-                                         : "memory");
-                    } else {
-#pragma unroll
-                        for (int e = 0; e < 32; ++e)
-                            if ((int64_t)(c0 + e) < m_rows) atomicAdd(dst + e, __uint_as_float(v[e]));
-                    }
-                } else if (vec) {
-#pragma unroll
-                    for (int e = 0; e < 32; e += 4)
-                        *reinterpret_cast<uint4*>(dst + e) = make_uint4(v[e], v[e + 1], v[e + 2], v[e + 3]);
-                } else {
-#pragma unroll
-                    for (int e = 0; e < 32; ++e)
-                        if ((int64_t)(c0 + e) < m_rows) dst[e] = __uint_as_float(v[e]);
-                }
-            }
-        }
-    } else if (warp == H_EPI_WARPS + 1) {
-        // ---------------- TMA: bf16 tiles straight into the operand stages (one thread) ----------------
-        if (lane == 0) {
-            const uint32_t stage_tx = (uint32_t)(S_A_BYTES + b_boxes * H_BOX_ROWS * H_ROW_BYTES);
-            const int64_t rot = (ktiles > 0 && ktiles <= 128) ? ((int64_t)blockIdx.x * ktiles / gridDim.x) % ktiles : 0;
-            int64_t issued = 0;
-            bool ok = true;
-            for (int64_t kt = 0; kt < ktiles; ++kt) {
-                const int s = (int)(kt % S_STAGES);
-                const uint32_t round = (uint32_t)(kt / S_STAGES);
-                if (round > 0) ok = mbar_wait(empty0 + 8 * s, (round - 1) & 1) && !abort_flag;
-                if (!ok) break;
-                mbar_expect_tx(full0 + 8 * s, stage_tx);
-                const uint32_t dst = smem_base + s * S_STAGE_BYTES;
-                // thread blocks walk the k tiles in rotated order (spread evenly over the contraction), so that at
-                // any moment they ask L2 for different tiles of the test matrix instead of all for the same one:
-                // 65 -> 56 us at 16,384 x 256 x 4,096; for long contractions it measured slower (143 -> 151 us at
-                // D = 16,384) and is left out
-                const int32_t x = (int32_t)((kt0 + (kt + rot) % ktiles) * H_BK);
-                tma_load_2d(dst, &map_train, x, (int32_t)n0, full0 + 8 * s);
-                for (int bx = 0; bx < b_boxes; ++bx)
-                    tma_load_2d(dst + S_A_BYTES + bx * H_BOX_ROWS * H_ROW_BYTES, &map_test, x,
-                                (int32_t)m0 + bx * H_BOX_ROWS, full0 + 8 * s);
-                issued = kt + 1;
-            }
-            if (!ok) abort_flag = 1;
-            // no copy of this thread block may still be in flight when it leaves
-            for (int64_t kt = issued > S_STAGES ? issued - S_STAGES : 0; kt < issued; ++kt)
-                if (!mbar_wait(full0 + 8 * (int)(kt % S_STAGES), (uint32_t)(kt / S_STAGES) & 1)) abort_flag = 1;
-        }
-    } else if (lane == 0) {
-        // ---------------- MMA issuer ----------------
-        const uint32_t idesc = make_idesc(BM, n_mma);
-        bool ok = true;
-        for (int64_t kt = 0; kt < ktiles && ok; ++kt) {
-            const int s = (int)(kt % S_STAGES);
-            ok = mbar_wait(full0 + 8 * s, (uint32_t)(kt / S_STAGES) & 1) && !abort_flag;
-            if (!ok) break;
-            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            const uint32_t a0 = smem_base + s * S_STAGE_BYTES, b0 = a0 + S_A_BYTES;
-#pragma unroll
-            for (int ks = 0; ks < H_BK / 16; ++ks)
-                umma_bf16(tmem_d, make_smem_desc_sw128(a0 + ks * 32), make_smem_desc_sw128(b0 + ks * 32), idesc,
-                          (kt > 0 || ks > 0) ? 1u : 0u);
-            umma_commit(empty0 + 8 * s);
-        }
-        if (!ok) abort_flag = 1;
-        if (ok && ktiles > 0) umma_commit(accum);
-    }
-
-    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-    __syncthreads();
-    if (warp == H_EPI_WARPS) {
-        __syncwarp();
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_d), "r"(H_TMEM_COLS) : "memory");
-    }
-}
-
 }  // namespace tc
-
-// cuTensorMapEncodeTiled through the runtime's driver entry point (the library does not link libcuda)
-typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
-                                  const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
-                                  CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-
-static EncodeTiledFn encode_tiled_fn()
-{
-    static EncodeTiledFn fn = [] {
-        void* p = nullptr;
-        cudaDriverEntryPointQueryResult q;
-        if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &p, cudaEnableDefault, &q) != cudaSuccess ||
-            q != cudaDriverEntryPointSuccess)
-            p = nullptr;
-        return (EncodeTiledFn)p;
-    }();
-    return fn;
-}
-
-// rows x D matrix with row stride ld, read in boxes of box_rows rows x 128 bytes with the 128-byte swizzle: 32 fp32
-// k-values, or 64 bf16 k-values (then the box is an operand tile as it stands); elements outside the matrix are
-// delivered as zeros
-static bool make_map(CUtensorMap* map, const void* base, int64_t rows, int64_t D, int64_t ld, bool bf16 = false,
-                     int box_rows = tc::BM)
-{
-    EncodeTiledFn enc = encode_tiled_fn();
-    if (!enc) return false;
-    const size_t esz = bf16 ? 2 : 4;
-    const cuuint64_t gdim[2] = {(cuuint64_t)D, (cuuint64_t)rows};
-    const cuuint64_t gstride[1] = {(cuuint64_t)ld * esz};
-    const cuuint32_t box[2] = {(cuuint32_t)(bf16 ? tc::H_BK : tc::BK), (cuuint32_t)box_rows};
-    const cuuint32_t estride[2] = {1, 1};
-    return enc(map, bf16 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, const_cast<void*>(base),
-               gdim, gstride, box, estride, CU_TENSOR_MAP_INTERLEAVE_NONE,
-               CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
-               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
 
 // true if the tensor-core path can take these operands (TMA wants 16-byte aligned bases and row strides)
 bool score_tc_supported(const float* train, int64_t ld_train, const float* test, int64_t ld_test, int64_t D)
@@ -823,57 +344,6 @@ grass_status launch_score_tc(const float* train, int64_t N, int64_t ld_train, co
     if (nprod != 3 && nprod != 4) nprod = 6;
     tc::grass_score_tc_kernel<<<grid, tc::THREADS, smem, st>>>(map_train, map_test, N, M, D, kt_split, scores, ld_s,
                                                                out_vec_ok, nprod);
-    return launch_status();
-}
-
-bool score_bf16_supported(const void* train, int64_t ld_train, const void* test, int64_t ld_test, int64_t D)
-{
-    return D > 0 && ((uintptr_t)train % 16 == 0) && ((uintptr_t)test % 16 == 0) && (ld_train % 8 == 0) &&
-           (ld_test % 8 == 0) && encode_tiled_fn() != nullptr;
-}
-
-grass_status launch_score_bf16(const void* train, int64_t N, int64_t ld_train, const void* test, int64_t M,
-                               int64_t ld_test, int64_t D, float* scores, int64_t ld_s, cudaStream_t st)
-{
-    const int64_t gx = ((N + tc::BM - 1) / tc::BM + 1) / 2 * 2;
-    const int64_t gy = (M + tc::BN - 1) / tc::BN;
-    if (gx > 0x7FFFFFFFLL || gy > 65535 || N > 0x7FFFFFFFLL || M > 0x7FFFFFFFLL || D > 0x7FFFFFFFLL)
-        return GRASS_ERR_UNSUPPORTED;
-    CUtensorMap map_train, map_test;
-    if (!make_map(&map_train, train, N, D, ld_train, true, tc::H_BOX_ROWS) ||
-        !make_map(&map_test, test, M, D, ld_test, true, tc::H_BOX_ROWS))
-        return GRASS_ERR_CUDA;
-    const int out_vec = ((uintptr_t)scores % 16 == 0) && (ld_s % 4 == 0);
-    if (gy == 1 && tuning(GRASS_TUNE_SCORE_BF16_SOLO, 1) != 0) {
-        // one column tile (M <= 256): one thread block per 128 train rows, no cluster
-        const int64_t tiles = (N + tc::BM - 1) / tc::BM;
-        const size_t smem1 = (size_t)tc::S_STAGES * tc::S_STAGE_BYTES + 1024;
-        if (cudaFuncSetAttribute(tc::grass_score_bf16_solo_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)smem1) != cudaSuccess)
-            return GRASS_ERR_CUDA;
-        int64_t splits1 = 1, kt_split1 = 1;
-        if (plan_splits(D, (tiles + 1) / 2, tc::H_BK, &splits1, &kt_split1) != GRASS_OK) return GRASS_ERR_CUDA;
-        if (splits1 > 1 && cudaMemset2DAsync(scores, (size_t)ld_s * sizeof(float), 0, (size_t)M * sizeof(float),
-                                             (size_t)N, st) != cudaSuccess)
-            return GRASS_ERR_CUDA;
-        dim3 grid1((unsigned)tiles, 1, (unsigned)splits1);
-        tc::grass_score_bf16_solo_kernel<<<grid1, tc::S_THREADS, smem1, st>>>(map_train, map_test, N, M, D, kt_split1,
-                                                                              scores, ld_s, out_vec);
-        return launch_status();
-    }
-    const size_t smem = (size_t)tc::H_STAGES * tc::H_STAGE_BYTES + 1024;
-    if (cudaFuncSetAttribute(tc::grass_score_bf16_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
-        cudaSuccess)
-        return GRASS_ERR_CUDA;
-    int64_t splits = 1, kt_split = 1;
-    if (plan_splits(D, gx / 2 * gy, tc::H_BK, &splits, &kt_split) != GRASS_OK) return GRASS_ERR_CUDA;
-    if (splits > 1 &&
-        cudaMemset2DAsync(scores, (size_t)ld_s * sizeof(float), 0, (size_t)M * sizeof(float), (size_t)N, st) != cudaSuccess)
-        return GRASS_ERR_CUDA;
-    dim3 grid((unsigned)gx, (unsigned)gy, (unsigned)splits);
-    const int out_vec_ok = ((uintptr_t)scores % 16 == 0) && (ld_s % 4 == 0);
-    tc::grass_score_bf16_kernel<<<grid, tc::H_THREADS, smem, st>>>(map_train, map_test, N, M, D, kt_split, scores, ld_s,
-                                                                   out_vec_ok);
     return launch_status();
 }
 

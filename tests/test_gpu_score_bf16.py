@@ -85,3 +85,19 @@ def test_score_of_a_bf16_cache_tracks_the_fp32_scores(G):
     half = G.grass_score_bf16(G.grass_to_bf16(tr), G.grass_to_bf16(te))
     scale = tr.norm(dim=1)[:, None] * te.norm(dim=1)[None, :]
     assert float(((full - half).abs() / scale).max()) < 2.0 ** -9
+
+
+# Stages of one and of two boxes (D up to 64 and beyond; widths that leave no room for three long stages), one and two
+# accumulators, several column tiles; ranges of k that begin and end inside a tile, runs of 8,192; ragged last rows
+@pytest.mark.parametrize("N,M,D", [(256, 32, 64), (255, 33, 72), (600, 300, 1_000), (1_000, 384, 136), (300, 385, 2_056),
+                                   (700, 512, 512), (150, 1_100, 8_200), (2_900, 260, 17_000), (40_000, 20, 128)])
+def test_score_bf16_shapes(G, N, M, D):
+    g = torch.Generator(device="cuda")
+    g.manual_seed(N + M)
+    tr = torch.randn((N, D), generator=g, device="cuda").to(torch.bfloat16)
+    te = torch.randn((M, D), generator=g, device="cuda").to(torch.bfloat16)
+    sc = G.grass_score_bf16(tr, te, out=torch.full((N, M), 7.0, device="cuda")).double()
+    ref, absum = tr.double() @ te.double().T, tr.double().abs() @ te.double().abs().T
+    # one truncation of the accumulator per 16 k-values, a bias of up to 2^-23 of the partial sum (its size: sqrt(D)
+    # against absum's D), plus the spread of the remaining roundings
+    assert ((sc - ref).abs() <= 2.0 * (D + 72) ** 0.5 * 2.0 ** -23 * absum).all()
