@@ -35,34 +35,18 @@ constexpr int A_BYTES = ROWS * ROW;            // 16 KB
 constexpr int MAX_STAGES = 12;
 constexpr int EPI_WARPS = 4;
 constexpr int THREADS_H = (EPI_WARPS + 2) * 32;
-constexpr int SMEM_BUDGET = 224 * 1024;
+constexpr int SMEM_BUDGET = 216 * 1024;        // for the stages
 constexpr uint32_t COLS = 512;                 // all of tensor memory: two accumulators of up to 256 columns
 constexpr int64_t MAX_RUN = 8192;              // k-values per accumulator run when D > 16,384
 
+constexpr int SCRATCH_BYTES = EPI_WARPS * 32 * 16 * 4;         // the epilogue warps' transposition buffers, behind the stages
+
 struct Plan {
+    WorkPlan work;         // k tiles of KW * 64 k-values, one stage each
     int64_t tiles_n;       // row tiles of 256
-    int64_t ktiles;        // of KW * 64 k-values, one stage each
-    int64_t units;         // tiles * ktiles
-    int64_t per_pair;      // units per pair
-    int64_t run;           // longest accumulator run in k-tiles; runs start at multiples of it within a tile
     int width;             // test rows per tile (a multiple of 32; of 64 above 256)
     int stages;
 };
-
-// a contiguous piece of one tile: k-tiles [k0, k1)
-struct Segment { int64_t tile, k0, k1; };
-__device__ __forceinline__ bool next_segment(const Plan& p, int64_t& u, int64_t end, Segment& s)
-{
-    if (u >= end) return false;
-    s.tile = u / p.ktiles;
-    s.k0 = u - s.tile * p.ktiles;
-    int64_t k1 = (s.k0 / p.run + 1) * p.run;
-    k1 = k1 < p.ktiles ? k1 : p.ktiles;
-    k1 = k1 < s.k0 + (end - u) ? k1 : s.k0 + (end - u);
-    s.k1 = k1;
-    u += k1 - s.k0;
-    return true;
-}
 
 // K-major tiles with 128-byte rows and the 128-byte swizzle (8-row groups 1,024 bytes apart; 16-byte chunk c of row r at
 // chunk c ^ (r & 7)); 32 * i bytes into the tile are k-values 16 i .. 16 i + 15
@@ -92,10 +76,10 @@ score_bf16_kernel(const __grid_constant__ CUtensorMap map_train, const __grid_co
     __shared__ uint32_t tmem_base_slot;
     __shared__ volatile int abort_flag;
 
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = __shfl_sync(0xFFFFFFFFu, tid >> 5, 0), lane = tid & 31;
     const uint32_t rank = cluster_ctarank();
-    const int64_t u0 = (int64_t)(blockIdx.x >> 1) * plan.per_pair;
-    const int64_t u1 = u0 + plan.per_pair < plan.units ? u0 + plan.per_pair : plan.units;
+    int64_t u0, u1;
+    pair_range(plan.work, blockIdx.x >> 1, u0, u1);
     const int S = plan.stages;
     const int n_sub = plan.width / SUBS, n_half = n_sub / 2;      // columns per accumulator; test rows of it staged here
     const int b_bytes = n_half * ROW;                             // one box of them
@@ -134,18 +118,20 @@ score_bf16_kernel(const __grid_constant__ CUtensorMap map_train, const __grid_co
     if (warp < EPI_WARPS) {
         // ---------------- epilogue: this block's 128 rows of every segment ----------------
         const uint32_t leader_empty = map_to_cta(acc_empty0, 0);
+        float* scratch = reinterpret_cast<float*>(smem + S * stage_bytes) + warp * (32 * 16);
         bool ok = true;
         int64_t u = u0;
         Segment seg;
-        for (int i = 0; next_segment(plan, u, u1, seg); ++i) {
+        for (int i = 0; next_segment(plan.work, u, u1, seg); ++i) {
             const int b = i % nbuf;
             if (ok) ok = mbar_wait(acc_full0 + 8 * b, (uint32_t)(i / nbuf) & 1) && !abort_flag;
             if (!ok) abort_flag = 1;
             ok = __all_sync(0xFFFFFFFFu, ok);
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             const int64_t tn = seg.tile % plan.tiles_n, tm = seg.tile / plan.tiles_n;
-            const int64_t row = tn * (2 * ROWS) + rank * ROWS + warp * 32 + lane, m0 = tm * plan.width;
-            const bool whole = seg.k0 == 0 && seg.k1 == plan.ktiles;
+            const int64_t row = tn * (2 * ROWS) + rank * ROWS + warp * 32, m0 = tm * plan.width;
+            const int rows = (int)((N - row) < 32 ? (N - row) : 32);
+            const bool whole = seg.k0 == 0 && seg.k1 == plan.work.ktiles;
             const int cols = (int)((M - m0) < plan.width ? (M - m0) : plan.width);
             for (int c0 = 0; c0 < cols; c0 += 32) {
                 uint32_t v[32];
@@ -158,107 +144,90 @@ score_bf16_kernel(const __grid_constant__ CUtensorMap map_train, const __grid_co
 #pragma unroll
                     for (int e = 0; e < 32; ++e) v[e] = 0x7FC00000u;        // NaN marks an aborted tile
                 }
-                if (row >= N) continue;
-                float* dst = scores + row * ld_s + m0 + c0;
-                const bool vec = out_vec_ok && c0 + 32 <= cols;
-                if (!whole) {
-                    if (vec) {
-#pragma unroll
-                        for (int e = 0; e < 32; e += 4)
-                            asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(dst + e),
-                                         "f"(__uint_as_float(v[e])), "f"(__uint_as_float(v[e + 1])),
-                                         "f"(__uint_as_float(v[e + 2])), "f"(__uint_as_float(v[e + 3]))
-                                         : "memory");
-                    } else {
-#pragma unroll
-                        for (int e = 0; e < 32; ++e)
-                            if (c0 + e < cols) atomicAdd(dst + e, __uint_as_float(v[e]));
-                    }
-                } else if (vec) {
-#pragma unroll
-                    for (int e = 0; e < 32; e += 4)
-                        *reinterpret_cast<uint4*>(dst + e) = make_uint4(v[e], v[e + 1], v[e + 2], v[e + 3]);
-                } else {
-#pragma unroll
-                    for (int e = 0; e < 32; ++e)
-                        if (c0 + e < cols) dst[e] = __uint_as_float(v[e]);
-                }
+                emit_block<16>(scratch, v, scores + row * ld_s + m0 + c0, ld_s, rows, cols - c0, out_vec_ok != 0, !whole);
             }
             asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
             __syncwarp();
             if (lane == 0) mbar_arrive_cluster(leader_empty + 8 * b);
         }
     } else if (warp == EPI_WARPS + 1) {
-        // ---------------- loads (one thread per block) ----------------
-        if (lane == 0) {
-            const uint32_t leader_full0 = map_to_cta(full0, 0);
-            const uint32_t both = 2u * (uint32_t)stage_bytes;
-            int s = 0, wrapped = 0;                        // stage to fill next; how often the ring has come round
-            bool ok = true;
-            int64_t u = u0;
-            Segment seg;
-            while (ok && next_segment(plan, u, u1, seg)) {
-                const int64_t tn = seg.tile % plan.tiles_n, tm = seg.tile / plan.tiles_n;
-                const int32_t row_a = (int32_t)(tn * (2 * ROWS) + rank * ROWS);
-                const int32_t row_b = (int32_t)(tm * plan.width + rank * n_half);
-                // pairs that cover whole tiles walk them in rotated order, so that at any moment they ask L2 for
-                // different parts of the test matrix (pieces of tiles start at different k-values anyway)
-                const int64_t len = seg.k1 - seg.k0;
-                const int64_t rot = len == plan.ktiles && len <= 128 ? (int64_t)(blockIdx.x >> 1) * len / (gridDim.x >> 1) : 0;
-                int32_t x = (int32_t)((seg.k0 + rot) * (KW * BKH));
-                for (int64_t kt = 0; kt < len; ++kt) {
-                    if (wrapped > 0) ok = mbar_wait(empty0 + 8 * s, (uint32_t)(wrapped - 1) & 1) && !abort_flag;
-                    if (!ok) break;
+        // ---------------- loads (one warp per block) ----------------
+        const uint32_t leader_full0 = map_to_cta(full0, 0);
+        const uint32_t both = 2u * (uint32_t)stage_bytes;
+        int s = 0;                                         // stage to fill next
+        uint32_t wrapped = 0;                              // how often the ring has come round
+        bool ok = true;
+        int64_t u = u0;
+        Segment seg;
+        while (ok && next_segment(plan.work, u, u1, seg)) {
+            const int64_t tn = seg.tile % plan.tiles_n, tm = seg.tile / plan.tiles_n;
+            const int32_t row_a = (int32_t)(tn * (2 * ROWS) + rank * ROWS);
+            const int32_t row_b = (int32_t)(tm * plan.width + rank * n_half);
+            // pairs that cover whole tiles walk them in rotated order, so that at any moment they ask L2 for
+            // different parts of the test matrix (pieces of tiles start at different k-values anyway)
+            const int len = (int)(seg.k1 - seg.k0);
+            const int rot = len == plan.work.ktiles && len <= 128 ? (int)((int64_t)(blockIdx.x >> 1) * len / (gridDim.x >> 1)) : 0;
+            int32_t x = (int32_t)((seg.k0 + rot) * (KW * BKH));
+            for (int kt = 0; kt < len; ++kt) {
+                if (wrapped > 0) ok = mbar_wait(empty0 + 8 * s, (wrapped - 1) & 1) && !abort_flag;
+                ok = __all_sync(0xFFFFFFFFu, ok);
+                if (!ok) break;
+                if (elect_one()) {
+                    const uint32_t dst = smem_base + (uint32_t)s * stage_bytes, bar = leader_full0 + 8 * s;
                     if (rank == 0) mbar_expect_tx(full0 + 8 * s, both);
-                    const uint32_t dst = smem_base + (uint32_t)s * stage_bytes;
 #pragma unroll
-                    for (int w = 0; w < KW; ++w)
-                        load_pair(dst + w * A_BYTES, &map_train, x + w * BKH, row_a, leader_full0 + 8 * s);
+                    for (int w = 0; w < KW; ++w) load_pair(dst + w * A_BYTES, &map_train, x + w * BKH, row_a, bar);
 #pragma unroll
                     for (int q = 0; q < SUBS; ++q)
 #pragma unroll
                         for (int w = 0; w < KW; ++w)
-                            load_pair(dst + KW * A_BYTES + (q * KW + w) * b_bytes, &map_test, x + w * BKH, row_b + q * n_sub,
-                                      leader_full0 + 8 * s);
-                    x = kt + rot + 1 == len ? (int32_t)(seg.k0 * (KW * BKH)) : x + KW * BKH;
-                    if (++s == S) { s = 0; ++wrapped; }
+                            load_pair(dst + KW * A_BYTES + (q * KW + w) * b_bytes, &map_test, x + w * BKH, row_b + q * n_sub, bar);
                 }
+                __syncwarp();
+                x = kt + rot + 1 == len ? (int32_t)(seg.k0 * (KW * BKH)) : x + KW * BKH;
+                if (++s == S) { s = 0; ++wrapped; }
             }
-            if (!ok) abort_flag = 1;
-            // no copy may still be in flight when the pair leaves: the leader's barriers count both blocks' bytes
-            if (rank == 0)
-                for (int q = 0; q < S; ++q)                // stage q was last filled in round wrapped (q < s) or the one before
-                    if ((q < s || wrapped > 0) && !mbar_wait(full0 + 8 * q, (uint32_t)(q < s ? wrapped : wrapped - 1) & 1)) abort_flag = 1;
         }
-    } else if (lane == 0 && rank == 0) {
+        if (!ok) abort_flag = 1;
+        // no copy may still be in flight when the pair leaves: the leader's barriers count both blocks' bytes
+        if (rank == 0)
+            for (int q = 0; q < S; ++q)                    // stage q was last filled in round wrapped (q < s) or the one before
+                if ((q < s || wrapped > 0) && !mbar_wait(full0 + 8 * q, (q < s ? wrapped : wrapped - 1) & 1)) abort_flag = 1;
+    } else if (warp == EPI_WARPS && rank == 0) {
         // ---------------- MMA issuer (leader only) ----------------
         const uint32_t idesc = make_idesc(2 * ROWS, (uint32_t)n_sub);
+        const uint64_t desc0 = desc128(smem_base);             // addresses below are 16-byte units added to it
         bool ok = true;
         int s = 0;
         uint32_t phase = 0;
         int64_t u = u0;
         Segment seg;
-        for (int i = 0; ok && next_segment(plan, u, u1, seg); ++i) {
+        for (int i = 0; ok && next_segment(plan.work, u, u1, seg); ++i) {
             const int b = i % nbuf;
             if (i >= nbuf) ok = mbar_wait_cluster(acc_empty0 + 8 * b, (uint32_t)(i / nbuf - 1) & 1) && !abort_flag;
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            for (int64_t kt = seg.k0; ok && kt < seg.k1; ++kt) {
+            const int len = (int)(seg.k1 - seg.k0);
+            for (int kt = 0; ok && kt < len; ++kt) {
                 ok = mbar_wait(full0 + 8 * s, phase) && !abort_flag;
+                ok = __all_sync(0xFFFFFFFFu, ok);
                 if (!ok) break;
-                const uint32_t a0 = smem_base + (uint32_t)s * stage_bytes, b0 = a0 + KW * A_BYTES;
+                if (elect_one()) {
+                    const uint64_t a0 = desc0 + (uint32_t)(s * stage_bytes >> 4), b0 = a0 + (KW * A_BYTES >> 4);
 #pragma unroll
-                for (int w = 0; w < KW; ++w)
+                    for (int w = 0; w < KW; ++w)
 #pragma unroll
-                    for (int ks = 0; ks < BKH / 16; ++ks)
+                        for (int ks = 0; ks < BKH / 16; ++ks)
 #pragma unroll
-                        for (int q = 0; q < SUBS; ++q)
-                            umma_bf16_pair(tmem_d + (uint32_t)((b + q) * 256), desc128(a0 + w * A_BYTES + ks * 32),
-                                           desc128(b0 + (q * KW + w) * b_bytes + ks * 32), idesc,
-                                           (kt > seg.k0 || w > 0 || ks > 0) ? 1u : 0u);
-                umma_commit_pair(empty0 + 8 * s);
+                            for (int q = 0; q < SUBS; ++q)
+                                umma_bf16_pair(tmem_d + (uint32_t)((b + q) * 256), a0 + ((w * A_BYTES + ks * 32) >> 4),
+                                               b0 + (uint32_t)(((q * KW + w) * b_bytes + ks * 32) >> 4), idesc,
+                                               (kt > 0 || w > 0 || ks > 0) ? 1u : 0u);
+                    umma_commit_pair(empty0 + 8 * s);
+                    if (kt + 1 == len) umma_commit_pair(acc_full0 + 8 * b);
+                }
+                __syncwarp();
                 if (++s == S) { s = 0; phase ^= 1; }
             }
-            if (ok) umma_commit_pair(acc_full0 + 8 * b);
         }
         if (!ok) abort_flag = 1;
     }
@@ -300,20 +269,11 @@ grass_status launch_score_bf16(const void* train, int64_t N, int64_t ld_train, c
     const int stage_bytes = kw * box_bytes;
     p.stages = std::min(MAX_STAGES, SMEM_BUDGET / stage_bytes);
     p.tiles_n = (N + 2 * ROWS - 1) / (2 * ROWS);
-    p.ktiles = (D + kw * BKH - 1) / (kw * BKH);
-    const int64_t tiles = p.tiles_n * tiles_m;
-    p.units = tiles * p.ktiles;
-    p.run = D > 16384 ? MAX_RUN / (kw * BKH) : p.ktiles;
-    const int64_t forced = tuning(GRASS_TUNE_SCORE_SPLITS, -1);
-    if (forced > 0) p.run = std::min<int64_t>(p.run, (p.ktiles + forced - 1) / forced);
-    // Whole tiles per pair cost ceil(tiles / pairs) tiles of time, an even cut by k costs its share plus the zero-fill and
-    // the additions, about what 768 k-values take; fewer than 512 k-values per pair are not worth a pair.
-    const int64_t pairs = sms / 2;
-    const int64_t whole = (tiles + pairs - 1) / pairs * p.ktiles;
-    const int64_t even = std::max<int64_t>(8 / kw, (p.units + pairs - 1) / pairs);
-    p.per_pair = even + 12 / kw < whole ? even : whole;
-    const int64_t used = (p.units + p.per_pair - 1) / p.per_pair;
-    const bool adds = p.per_pair % p.ktiles != 0 || p.run < p.ktiles;
+    const int64_t ktiles = (D + kw * BKH - 1) / (kw * BKH);
+    const int64_t run = D > 16384 ? MAX_RUN / (kw * BKH) : ktiles;
+    // 64 k-values take about 0.3 us
+    bool adds;
+    const int64_t used = plan_work(p.work, p.tiles_n * tiles_m, ktiles, run, sms / 2, 10 / kw, 12 / kw, tuning(GRASS_TUNE_SCORE_SPLITS, -1), &adds);
     CUtensorMap map_train, map_test;
     if (!make_map(&map_train, train, N, D, ld_train, true, ROWS) ||
         !make_map(&map_test, test, M, D, ld_test, true, p.width / subs / 2))
@@ -322,9 +282,9 @@ grass_status launch_score_bf16(const void* train, int64_t N, int64_t ld_train, c
         return GRASS_ERR_CUDA;
     const int out_vec = ((uintptr_t)scores % 16 == 0) && (ld_s % 4 == 0);
     auto launch = [&](auto kern) -> grass_status {
-        if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BUDGET) != cudaSuccess)
+        if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BUDGET + SCRATCH_BYTES) != cudaSuccess)
             return GRASS_ERR_CUDA;
-        kern<<<(unsigned)(2 * used), THREADS_H, (size_t)p.stages * stage_bytes, st>>>(map_train, map_test, p, N, M, scores, ld_s,
+        kern<<<(unsigned)(2 * used), THREADS_H, (size_t)p.stages * stage_bytes + SCRATCH_BYTES, st>>>(map_train, map_test, p, N, M, scores, ld_s,
                                                                                       out_vec);
         return launch_status();
     };

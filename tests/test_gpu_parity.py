@@ -560,3 +560,17 @@ def test_grass_score_long_contraction_keeps_relative_accuracy(G, oracle_mod):
     ref, _ = oracle_mod.score(tr.cpu().numpy(), te.cpu().numpy())
     rel = np.abs(sc - ref) / np.abs(ref)
     assert rel.max() <= 1e-4, rel.max()
+
+
+# The tensor-core score kernel where its work plan changes: whole tiles, pieces of one tile, an even cut with ranges that
+# begin and end inside tiles, accumulator runs of 8,192, a tile narrower than a stage, ragged rows, columns and k
+@pytest.mark.parametrize("N,M,D", [(20_000, 40, 96), (256, 256, 8_192), (4_000, 300, 700), (30_000, 256, 260), (300, 33, 20_004),
+                                   (1_030, 600, 1_000), (257, 1, 36), (19_000, 513, 64)])
+def test_score_work_plans(G, W, N, M, D):
+    tr, te = W.score_vectors(N, M, D, 77 + M, device="cuda")
+    buf = torch.full((N, M + 1), 5.0, device="cuda")
+    sc = G.grass_score(tr, te, out=buf[:, :M]).double()
+    ref, absum = tr.double() @ te.double().T, tr.double().abs() @ te.double().abs().T
+    # six bf16 products hold each product to 2^-23; one truncation of the accumulators per 16 k-values
+    assert ((sc - ref).abs() <= (2.0 ** -22 + 2.0 * (D + 72) ** 0.5 * 2.0 ** -23) * absum).all()
+    assert (buf[:, M] == 5.0).all()
