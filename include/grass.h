@@ -154,6 +154,22 @@ grass_status factgrass_compress_grouped_out(const factgrass_layer* layers /*host
                                             void* stream);
 
 /*
+ * grass_compress_out with device scratch.  The identity mask (plain SJLT) of a large batch is projected through a table
+ * of the projection that the call builds once for all samples; the table lives in the caller's scratch.
+ *   grass_compress_workspace_bytes  what the call with these arguments would use; 0 means it uses none.
+ *   workspace  device scratch of at least that many bytes, 128-byte aligned, in use until the work enqueued by the call
+ *              has finished; NULL or a smaller one is valid and gives grass_compress_out.  With a workspace and
+ *              idx == NULL, g is device memory.
+ * Results are those of grass_compress_out up to the order of additions.
+ */
+size_t grass_compress_workspace_bytes(grass_dtype dt, int64_t n, int64_t p, const uint32_t* idx,
+                                      const grass_sjlt_spec* spec /*host*/);
+grass_status grass_compress_ws(const void* g, grass_dtype dt, int64_t n, int64_t p, int64_t ld,
+                               const uint32_t* idx, int64_t kprime, const grass_sjlt_spec* spec /*host*/,
+                               void* out, grass_dtype out_dt, int64_t ld_out, void* workspace, size_t workspace_bytes,
+                               uint32_t* dev_status, void* stream);
+
+/*
  * Sparsification alone (Section 3.2: Random / Selective Mask used as the whole compressor, which the
  * paper evaluates next to GraSS and FactGraSS).
  *   grass_mask         out[i, j] = g[i, idx[j]],  out n x kprime fp32 (row stride ld_out >= kprime);
@@ -318,7 +334,7 @@ typedef enum {
     GRASS_TUNE_COMPRESS_SAMPLES = 0,   /* grass_compress: samples per thread block (1, 2, 4, 8) */
     GRASS_TUNE_COMPRESS_JSPLIT = 1,    /* grass_compress: thread blocks that share one sample's masked positions */
     GRASS_TUNE_COMPRESS_CLUSTER = 2,   /* grass_compress: 0 = reduce position splits with global reductions */
-    GRASS_TUNE_COMPRESS_DENSE = 3,     /* grass_compress: 0 = no vector-load path for identity masks */
+    GRASS_TUNE_COMPRESS_DENSE = 3,     /* identity masks: 0 = gathers, 1 = streamed rows, 2 = the table wherever it fits (grass_compress_ws) */
     GRASS_TUNE_FACTGRASS_TILE = 4,     /* factgrass: block tile 64 or 128 */
     GRASS_TUNE_FACTGRASS_CHUNK = 5,    /* factgrass: tokens per thread block */
     GRASS_TUNE_FACTGRASS_CARVEOUT = 6, /* factgrass: shared-memory carve-out in percent */

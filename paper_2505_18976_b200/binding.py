@@ -34,7 +34,7 @@ EXPORTS = ("grass_compress", "factgrass_compress", "factgrass_compress_grouped",
            "factmask_compress_grouped",
            "factgrass_grouped_workspace_bytes", "factgrass_compress_grouped_static", "grass_score", "grass_sjlt_table", "grass_validate_mask",
            "grass_random_mask_host", "grass_status_string", "grass_to_bf16", "grass_score_bf16", "grass_set_tuning",
-           "grass_compress_out", "factgrass_compress_grouped_out")
+           "grass_compress_out", "factgrass_compress_grouped_out", "grass_compress_workspace_bytes", "grass_compress_ws")
 
 # grass_tuning_key in include/grass.h
 TUNE = {"compress_samples": 0, "compress_jsplit": 1, "compress_cluster": 2, "compress_dense": 3,
@@ -135,8 +135,8 @@ def lib() -> ctypes.CDLL:
         L.grass_status_string.argtypes = [st]
         from . import _native as native     # built beside the library; missing = not built, no fallback
         native.bind(GrassError, *(ctypes.cast(getattr(L, f), vp).value for f in (
-            "grass_compress_out", "factgrass_compress", "factgrass_compress_varlen", "factgrass_compress_grouped_out",
-            "factgrass_compress_grouped_varlen", "grass_score", "grass_score_bf16")))
+            "grass_compress_ws", "factgrass_compress", "factgrass_compress_varlen", "factgrass_compress_grouped_out",
+            "factgrass_compress_grouped_varlen", "grass_score", "grass_score_bf16", "grass_compress_workspace_bytes")))
         _native = native
         _lib = L
     return _lib

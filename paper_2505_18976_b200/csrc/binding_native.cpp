@@ -21,9 +21,10 @@
 
 namespace {
 
-// entry points of libgrass_b200.so, in the order of kNames
+// entry points of libgrass_b200.so
 struct Api {
-    decltype(&::grass_compress_out) compress_out = nullptr;
+    decltype(&::grass_compress_ws) compress = nullptr;
+    decltype(&::grass_compress_workspace_bytes) compress_bytes = nullptr;
     decltype(&::factgrass_compress) factgrass = nullptr;
     decltype(&::factgrass_compress_varlen) factgrass_varlen = nullptr;
     decltype(&::factgrass_compress_grouped_out) grouped_out = nullptr;
@@ -162,9 +163,18 @@ PyObject* py_grass_compress(PyObject*, PyObject* const* a, Py_ssize_t n)
     void* const st = current_stream();
     const void* gp = g->const_data_ptr();
     void* op = o->data_ptr();
+    // scratch from torch's stream-ordered pool: it may be handed out again as soon as this tensor is gone, to work that
+    // is enqueued behind the kernels that use it
+    at::Tensor scratch;
+    void* wp = nullptr;
+    const size_t wbytes = idx ? 0 : api.compress_bytes((grass_dtype)dt, rows, p, idx, &sp);
+    if (wbytes > 0) {
+        scratch = empty2(1, (int64_t)wbytes, at::kByte, g->device());
+        wp = scratch.data_ptr();
+    }
     grass_status rc;
     Py_BEGIN_ALLOW_THREADS
-    rc = api.compress_out(gp, (grass_dtype)dt, rows, p, ld, idx, kprime, &sp, op, (grass_dtype)odt, ld_out, dev_status, st);
+    rc = api.compress(gp, (grass_dtype)dt, rows, p, ld, idx, kprime, &sp, op, (grass_dtype)odt, ld_out, wp, wbytes, dev_status, st);
     Py_END_ALLOW_THREADS
     return finish(rc, "grass_compress", a[5], made);
     GUARD_END
@@ -403,16 +413,17 @@ PyObject* py_score(PyObject*, PyObject* const* a, Py_ssize_t n)
 // bind(GrassError, addresses...): the library's entry points, in the order of struct Api
 PyObject* py_bind(PyObject*, PyObject* const* a, Py_ssize_t n)
 {
-    void* p[7];
-    if (n != 8) {
-        PyErr_SetString(PyExc_TypeError, "bind(GrassError, 7 addresses)");
+    void* p[8];
+    if (n != 9) {
+        PyErr_SetString(PyExc_TypeError, "bind(GrassError, 8 addresses)");
         return nullptr;
     }
-    for (int i = 0; i < 7; ++i) {
+    for (int i = 0; i < 8; ++i) {
         p[i] = PyLong_AsVoidPtr(a[i + 1]);
         if (PyErr_Occurred()) return nullptr;
     }
-    api.compress_out = (decltype(api.compress_out))p[0];
+    api.compress = (decltype(api.compress))p[0];
+    api.compress_bytes = (decltype(api.compress_bytes))p[7];
     api.factgrass = (decltype(api.factgrass))p[1];
     api.factgrass_varlen = (decltype(api.factgrass_varlen))p[2];
     api.grouped_out = (decltype(api.grouped_out))p[3];

@@ -98,6 +98,12 @@ grass_status launch_compress_rows(const void* g, grass_dtype dt, int64_t n, int6
                                   int64_t kprime, const grass_sjlt_spec& sp, float* out, int64_t ld_out,
                                   uint32_t* dev_status, cudaStream_t st, int out_bf16);
 
+// Plain SJLT through a table of the projection (grass_sjlt_table.cu): bytes of device scratch it wants for this call (0:
+// the call does not take it), and the launches
+size_t sjlt_table_bytes(int64_t n, int64_t p, uint32_t k, uint32_t s, size_t elem_bytes);
+grass_status launch_sjlt_table(const void* g, grass_dtype dt, int64_t n, int64_t p, int64_t ld, const grass_sjlt_spec& sp, float* out,
+                               int64_t ld_out, void* table, uint32_t* dev_status, cudaStream_t st, int out_bf16);
+
 // launch-shape override set through grass_set_tuning, or `dflt` while the key is on automatic
 int64_t tuning(grass_tuning_key key, int64_t dflt);
 

@@ -536,10 +536,16 @@ extern "C" grass_status grass_mask(const void* g, grass_dtype dt, int64_t n, int
     return grass::launch_status();
 }
 
-extern "C" grass_status grass_compress_out(const void* g, grass_dtype dt, int64_t n, int64_t p, int64_t ld,
-                                           const uint32_t* idx, int64_t kprime, const grass_sjlt_spec* spec,
-                                           void* out_v, grass_dtype out_dt, int64_t ld_out, uint32_t* dev_status,
-                                           void* stream)
+extern "C" size_t grass_compress_workspace_bytes(grass_dtype dt, int64_t n, int64_t p, const uint32_t* idx, const grass_sjlt_spec* spec)
+{
+    if (idx || !spec || spec->k == 0 || p >= 0xFFFFFFFFLL || (dt != GRASS_F32 && dt != GRASS_BF16)) return 0;
+    return grass::sjlt_table_bytes(n, p, spec->k, spec->s, dt == GRASS_F32 ? 4 : 2);
+}
+
+extern "C" grass_status grass_compress_ws(const void* g, grass_dtype dt, int64_t n, int64_t p, int64_t ld,
+                                          const uint32_t* idx, int64_t kprime, const grass_sjlt_spec* spec,
+                                          void* out_v, grass_dtype out_dt, int64_t ld_out, void* workspace,
+                                          size_t workspace_bytes, uint32_t* dev_status, void* stream)
 {
     if (!spec || spec->k == 0 || spec->s == 0) return GRASS_ERR_INVALID_ARG;
     if (n < 0 || p < 0 || kprime < 0 || kprime > p || ld < p || ld_out < (int64_t)spec->k) return GRASS_ERR_INVALID_ARG;
@@ -556,6 +562,16 @@ extern "C" grass_status grass_compress_out(const void* g, grass_dtype dt, int64_
     if (kprime == 0) {
         return grass::cuda_ok(cudaMemset2DAsync(out, (size_t)ld_out * osz, 0, (size_t)spec->k * osz, (size_t)n, st));
     }
+    if (!idx && workspace) {
+        // Short fp32 rows that the streamed path can read with vector loads stay there: emptying the bins after every two
+        // rows costs the table's kernel what it saves (2,048 x 20,000, k = 4,096: 76 against 85 us dense, 41 against 45 at
+        // 99 % zeros; at 50,000 positions 158 against 137 and 74 against 63).
+        const bool streamed = dt == GRASS_F32 && (uintptr_t)g % 16 == 0 && ld % 4 == 0 && p < 32768 && spec->k <= 8192 &&
+                              grass::tuning(GRASS_TUNE_COMPRESS_DENSE, -1) != 2;
+        const size_t need = streamed ? 0 : grass_compress_workspace_bytes(dt, n, p, idx, spec);
+        if (need > 0 && workspace_bytes >= need && (uintptr_t)workspace % 128 == 0)
+            return grass::launch_sjlt_table(g, dt, n, p, ld, *spec, out, ld_out, workspace, dev_status, st, out_bf16);
+    }
     // Row staging for dense masks (grass_compress_rows.cu): whole rows through shared memory, window by window,
     // the masked elements picked from there.  It is built and parity-tested but not chosen automatically: on B200
     // it is slower than the gathers below even where the mask touches nine pieces in ten (config 1: 28.6 against
@@ -570,6 +586,14 @@ extern "C" grass_status grass_compress_out(const void* g, grass_dtype dt, int64_
                                                dev_status, st, out_bf16);
     return grass::dispatch_compress<__nv_bfloat16>((const __nv_bfloat16*)g, n, p, ld, idx, kprime, *spec, out,
                                                    ld_out, dev_status, st, out_bf16);
+}
+
+extern "C" grass_status grass_compress_out(const void* g, grass_dtype dt, int64_t n, int64_t p, int64_t ld,
+                                           const uint32_t* idx, int64_t kprime, const grass_sjlt_spec* spec,
+                                           void* out, grass_dtype out_dt, int64_t ld_out, uint32_t* dev_status,
+                                           void* stream)
+{
+    return grass_compress_ws(g, dt, n, p, ld, idx, kprime, spec, out, out_dt, ld_out, nullptr, 0, dev_status, stream);
 }
 
 extern "C" grass_status grass_compress(const void* g, grass_dtype dt, int64_t n, int64_t p, int64_t ld,
