@@ -398,6 +398,19 @@ static grass_status run_factgrass(const factgrass_layer* layers, int32_t L, gras
         cluster_chunk = (int)chunk;
     };
 
+    // The persistent kernel takes what is left of one-tile blocks (factgrass_persistent.cu).
+    bool persistent = false;
+    auto plan_persistent = [&](const LayerDesc* hd) {
+        const int64_t forced = tuning(GRASS_TUNE_FACTGRASS_PATH, -1);
+        if (epi != kEpiSjlt || out_bf16 || T <= 0 || forced == 0 || cluster_nc > 0) return;
+        if (!persistent_fits(hd, L, B, tok_count)) return;
+        persistent = forced == 2;
+    };
+    // the table of every layer's projection sits behind the descriptors where the workspace has room for it
+    const size_t table_off = ((size_t)L * sizeof(LayerDesc) + 255) / 256 * 256;
+    void* const table = workspace && workspace_bytes >= table_off + persistent_table_bytes(L) && (uintptr_t)workspace % 16 == 0
+                            ? (char*)workspace + table_off : nullptr;
+
     // a single layer travels as a kernel parameter: no descriptor copy, whoever provided a workspace
     const bool grouped = workspace != nullptr && L > 1;
     LayerDesc single;
@@ -416,16 +429,23 @@ static grass_status run_factgrass(const factgrass_layer* layers, int32_t L, gras
                 max_tiles = host[l].tiles_m * host[l].tiles_n;
         }
         if (rc == GRASS_OK) plan_cluster(host);
+        if (rc == GRASS_OK) plan_persistent(host);
         if (rc == GRASS_OK)
             rc = cuda_ok(cudaMemcpyAsync(workspace, host, (size_t)L * sizeof(LayerDesc), cudaMemcpyHostToDevice, st));
+        if (rc == GRASS_OK && persistent)
+            rc = launch_persistent(host, (LayerDesc*)workspace, single, f32, L, B, T, tok_begin, tok_count, out, ld_out, table,
+                                   dev_status, st);
         if (host != stack_buf) std::free(host);
-        if (rc != GRASS_OK) return rc;
+        if (rc != GRASS_OK || persistent) return rc;
         dev_descs = (LayerDesc*)workspace;
     } else {
         grass_status rc = fill_desc(single, layers[0], tile, T);
         if (rc != GRASS_OK) return rc;
         max_tiles = single.tiles_m * single.tiles_n;
         plan_cluster(&single);
+        plan_persistent(&single);
+        if (persistent)
+            return launch_persistent(&single, nullptr, single, f32, L, B, T, tok_begin, tok_count, out, ld_out, table, dev_status, st);
     }
     if (cluster_nc > 0)
         return launch_factgrass_cluster(dev_descs, single, cplan, L, B, T, tok_begin, tok_count, cluster_nc,
@@ -617,7 +637,9 @@ extern "C" grass_status factmask_compress_grouped(const factgrass_layer* layers,
 extern "C" size_t factgrass_grouped_workspace_bytes(int32_t L)
 {
     if (L <= 0) return 256;
-    return ((size_t)L * sizeof(grass::LayerDesc) + 255) / 256 * 256;
+    // the descriptors, and a table of every layer's projection for the persistent kernel (which hashes where the
+    // workspace has no room for it)
+    return ((size_t)L * sizeof(grass::LayerDesc) + 255) / 256 * 256 + grass::persistent_table_bytes(L);
 }
 
 extern "C" grass_status factgrass_compress_grouped(const factgrass_layer* layers, int32_t L, grass_dtype dt, int32_t B,
