@@ -157,7 +157,7 @@ factgrass_persistent_kernel(const __grid_constant__ Args x, const __grid_constan
     __shared__ int32_t prefix[MAX_VAR_B + 1];
     float* bins = reinterpret_cast<float*>(smem + NBUF * STAGE);
 
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = __shfl_sync(0xFFFFFFFFu, tid >> 5, 0), lane = tid & 31;
     // stage[b]: the MMAs that read operand buffer b are done; full[a]: accumulator a is complete; empty[a]: it was read
     const uint32_t stage0 = tc::smem_u32(&bars[0]), full0 = tc::smem_u32(&bars[NBUF]), empty0 = tc::smem_u32(&bars[NBUF + 2]);
     if (tid == 0) {
@@ -310,7 +310,7 @@ factgrass_persistent_kernel(const __grid_constant__ Args x, const __grid_constan
                 *reinterpret_cast<uint4*>(tile0 + off) = pack8_bf16(v);
             }
         };
-        const uint32_t smem_base = tc::smem_u32(smem);
+        const uint64_t desc0 = tc::make_smem_desc(tc::smem_u32(smem));
         const uint32_t idesc = tc::make_idesc(TILE, TILE);
         bool ok = true;
         int n = 0;
@@ -330,29 +330,34 @@ factgrass_persistent_kernel(const __grid_constant__ Args x, const __grid_constan
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
             fetch(ra, rg);
             asm volatile("bar.sync 1, %0;" ::"n"(GATHER) : "memory");
-            if (tid == 0) {
+            if (warp == 0) {
                 if (first && seg >= 2) ok = ok && tc::mbar_wait(empty0 + 8 * acc, (uint32_t)(seg / 2 - 1) & 1u);
+                __syncwarp();
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                const uint32_t a0 = smem_base + buf * STAGE, g0 = a0 + NP * PIECE, d0 = tmem_d + acc * ACC;
+                if (tc::elect_one()) {
+                    // addresses in 16-byte units on top of the first descriptor
+                    const uint64_t a0 = desc0 + (uint32_t)(buf * (STAGE >> 4)), g0 = a0 + (NP * PIECE >> 4);
+                    const uint32_t d0 = tmem_d + acc * ACC;
 #pragma unroll
-                for (int ks = 0; ks < kTokTile / 16; ++ks) {
-                    if constexpr (F32) {
-                        // hi*hi goes to the first accumulator, the correction terms to the second (the tensor core
-                        // truncates after every accumulation, so the large sum sees as few of them as possible)
+                    for (int ks = 0; ks < kTokTile / 16; ++ks) {
+                        if constexpr (F32) {
+                            // hi*hi goes to the first accumulator, the correction terms to the second (the tensor core
+                            // truncates after every accumulation, so the large sum sees as few of them as possible)
 #pragma unroll
-                        for (int q = 0; q < 6; ++q) {
-                            if (q >= x.nprod) break;
-                            const uint64_t ad = tc::make_smem_desc(a0 + tc::split_piece_a(q) * PIECE + ks * 32);
-                            const uint64_t gd = tc::make_smem_desc(g0 + tc::split_piece_b(q) * PIECE + ks * 32);
-                            tc::umma_bf16(q == 0 ? d0 : d0 + TILE, ad, gd, idesc, (!first || ks > 0 || q > 1) ? 1u : 0u);
+                            for (int q = 0; q < 6; ++q) {
+                                if (q >= x.nprod) break;
+                                tc::umma_bf16(q == 0 ? d0 : d0 + TILE, a0 + ((tc::split_piece_a(q) * PIECE + ks * 32) >> 4),
+                                              g0 + ((tc::split_piece_b(q) * PIECE + ks * 32) >> 4), idesc,
+                                              (!first || ks > 0 || q > 1) ? 1u : 0u);
+                            }
+                        } else {
+                            tc::umma_bf16(d0, a0 + (ks * 32 >> 4), g0 + (ks * 32 >> 4), idesc, (!first || ks > 0) ? 1u : 0u);
                         }
-                    } else {
-                        tc::umma_bf16(d0, tc::make_smem_desc(a0 + ks * 32), tc::make_smem_desc(g0 + ks * 32), idesc,
-                                      (!first || ks > 0) ? 1u : 0u);
                     }
+                    tc::umma_commit(stage0 + 8 * buf);             // buffer free once these MMAs have read it
+                    if (last) tc::umma_commit(full0 + 8 * acc);    // accumulator complete
                 }
-                tc::umma_commit(stage0 + 8 * buf);             // buffer free once these MMAs have read it
-                if (last) tc::umma_commit(full0 + 8 * acc);    // accumulator complete
+                __syncwarp();
             }
             ++n;
         };
@@ -408,15 +413,12 @@ factgrass_persistent_kernel(const __grid_constant__ Args x, const __grid_constan
                         for (int q = 0; q < 4; ++q) t4[q] = *reinterpret_cast<const uint4*>(tab + a * TILE + c0 + 8 * q);
                     uint32_t v[32];
                     if (ok) {
-                        tc::tmem_ld32(d0 + (uint32_t)c0, v);
+                        tc::tmem_ld32_wait(d0 + (uint32_t)c0, v);
                         if constexpr (F32) {
                             uint32_t w[32];
-                            tc::tmem_ld32(d0 + (uint32_t)(TILE + c0), w);
-                            asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+                            tc::tmem_ld32_wait(d0 + (uint32_t)(TILE + c0), w);
 #pragma unroll
                             for (int e = 0; e < 32; ++e) v[e] = __float_as_uint(__uint_as_float(v[e]) + __uint_as_float(w[e]));
-                        } else {
-                            asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
                         }
                     } else {
 #pragma unroll
@@ -438,13 +440,8 @@ factgrass_persistent_kernel(const __grid_constant__ Args x, const __grid_constan
                             }
                         }
                     } else {
-#pragma unroll 1
-                        for (int e = 0; e < 32; ++e) {
-                            uint32_t pick = v[0];
 #pragma unroll
-                            for (int q = 1; q < 32; ++q) pick = q == e ? v[q] : pick;
-                            hash(a, c0 + e, pick);
-                        }
+                        for (int e = 0; e < 32; ++e) hash(a, c0 + e, v[e]);
                     }
                 } else {
                     // accumulator row a sits in lane (a % 16) + 32 (a / 16): register e of a lane holds row
@@ -457,15 +454,12 @@ factgrass_persistent_kernel(const __grid_constant__ Args x, const __grid_constan
                             t2[e] = *reinterpret_cast<const uint32_t*>(tab + (a0 + 8 * (e & 1)) * TILE + cc + 8 * (e >> 1));
                     uint32_t v[16];
                     if (ok) {
-                        tc::tmem_ld_16x256b_x4(d0 + (uint32_t)c0, v);
+                        tc::tmem_ld_16x256b_x4_wait(d0 + (uint32_t)c0, v);
                         if constexpr (F32) {
                             uint32_t w[16];
-                            tc::tmem_ld_16x256b_x4(d0 + (uint32_t)(TILE + c0), w);
-                            asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+                            tc::tmem_ld_16x256b_x4_wait(d0 + (uint32_t)(TILE + c0), w);
 #pragma unroll
                             for (int e = 0; e < 16; ++e) v[e] = __float_as_uint(__uint_as_float(v[e]) + __uint_as_float(w[e]));
-                        } else {
-                            asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
                         }
                     } else {
 #pragma unroll

@@ -23,16 +23,6 @@ __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map
                  : "memory");
 }
 
-// One lane of a converged warp.  The issuing warps run their loops as a whole and let one elected lane execute each
-// tcgen05 / TMA instruction: their operands live in uniform registers, and in code that only one lane runs the compiler
-// has to move every one of them there anew (70 cycles per MMA instead of about 20).
-__device__ __forceinline__ bool elect_one()
-{
-    uint32_t p;
-    asm volatile("{\n\t.reg .pred P;\n\telect.sync _|P, 0xFFFFFFFF;\n\tselp.u32 %0, 1, 0, P;\n\t}" : "=r"(p));
-    return p != 0;
-}
-
 __device__ __forceinline__ uint32_t cluster_ctarank()
 {
     uint32_t r;
