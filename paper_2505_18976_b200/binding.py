@@ -135,7 +135,7 @@ def lib() -> ctypes.CDLL:
         L.grass_status_string.argtypes = [st]
         from . import _native as native     # built beside the library; missing = not built, no fallback
         native.bind(GrassError, *(ctypes.cast(getattr(L, f), vp).value for f in (
-            "grass_compress_ws", "factgrass_compress", "factgrass_compress_varlen", "factgrass_compress_grouped_out",
+            "grass_compress_ws", "factgrass_grouped_workspace_bytes", "factgrass_compress_varlen", "factgrass_compress_grouped_out",
             "factgrass_compress_grouped_varlen", "grass_score", "grass_score_bf16", "grass_compress_workspace_bytes")))
         _native = native
         _lib = L

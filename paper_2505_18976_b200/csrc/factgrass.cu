@@ -377,7 +377,7 @@ static grass_status run_factgrass(const factgrass_layer* layers, int32_t L, gras
     auto plan_cluster = [&](const LayerDesc* hd) {
         if (epi != kEpiSjlt || f32 || T <= 0) return;
         const int64_t forced = tuning(GRASS_TUNE_FACTGRASS_PATH, -1);
-        if (forced == 0 || !cluster_path_fits(hd, L, &cplan)) return;
+        if (forced == 0 || forced == 2 || !cluster_path_fits(hd, L, &cplan)) return;
         const int64_t items = (int64_t)L * B, slots = (int64_t)sms * cplan.per_sm;
         if (items > slots && forced != 1) return;
         // clusters of 1, 2, 4 or 8 thread blocks: as many as fill the machine, each with at least two 32-token steps;
@@ -398,18 +398,24 @@ static grass_status run_factgrass(const factgrass_layer* layers, int32_t L, gras
         cluster_chunk = (int)chunk;
     };
 
-    // The persistent kernel takes what is left of one-tile blocks (factgrass_persistent.cu).
-    bool persistent = false;
-    auto plan_persistent = [&](const LayerDesc* hd) {
-        const int64_t forced = tuning(GRASS_TUNE_FACTGRASS_PATH, -1);
-        if (epi != kEpiSjlt || out_bf16 || T <= 0 || forced == 0 || cluster_nc > 0) return;
-        if (!persistent_fits(hd, L, B, tok_count)) return;
-        persistent = forced == 2;
-    };
-    // the table of every layer's projection sits behind the descriptors where the workspace has room for it
+    // Blocks above 64 x 64 with work for every SM take the persistent kernel (factgrass_persistent.cu), which gathers a
+    // column once where four 64 x 64 tiles gather it twice.  Of these, bf16 launches with clusters of several thread
+    // blocks stay with the cluster kernel: it has no table to write and no rows to zero.  Up to 64 x 64 the streaming
+    // kernel's thread blocks are short enough (and two to three per SM) to hide each other's projections.
+    // The table of the projections sits behind the descriptors where the workspace has room for it.
     const size_t table_off = ((size_t)L * sizeof(LayerDesc) + 255) / 256 * 256;
-    void* const table = workspace && workspace_bytes >= table_off + persistent_table_bytes(L) && (uintptr_t)workspace % 16 == 0
-                            ? (char*)workspace + table_off : nullptr;
+    void* const table = workspace && workspace_bytes >= table_off + persistent_table_bytes(L) ? (char*)workspace + table_off : nullptr;
+    // A share ends with a projection, so it wants a few 32-token steps: with fewer (layer, sample) items than SMs four
+    // per SM (three up to 96 x 96, where the projection is half as long); measured in fp32, streaming -> persistent, 768 x
+    // 3,072 at 128 x 128: 27.7 -> 28.8 us at 1.7 steps, 38.7 -> 40.5 at 3.5, 62.3 -> 61.7 at 6.9; at 72 x 72: 39.8 -> 33.7 at
+    // 3.5.  With an item for every SM the streaming kernel projects as often, at four tiles per block, and the persistent
+    // one is faster down to one step per item (16 layers of 16 x 32 tokens, 128 x 128 bf16: 75.5 -> 34.8 us).
+    auto persistent = [&](const LayerDesc* hd) {
+        const int64_t forced = tuning(GRASS_TUNE_FACTGRASS_PATH, -1);
+        if (epi != kEpiSjlt || out_bf16 || T <= 0 || !table || cluster_nc > 1 || !persistent_fits(hd, L, B, tok_count)) return false;
+        const int64_t items = (int64_t)L * B, steps = (T + kTokTile - 1) / kTokTile * items;
+        return forced == 2 || (forced == -1 && max_kk > 64 && (items >= sms || steps >= (max_kk > 96 ? 4 : 3) * (int64_t)sms));
+    };
 
     // a single layer travels as a kernel parameter: no descriptor copy, whoever provided a workspace
     const bool grouped = workspace != nullptr && L > 1;
@@ -429,23 +435,21 @@ static grass_status run_factgrass(const factgrass_layer* layers, int32_t L, gras
                 max_tiles = host[l].tiles_m * host[l].tiles_n;
         }
         if (rc == GRASS_OK) plan_cluster(host);
-        if (rc == GRASS_OK) plan_persistent(host);
+        const bool take_persistent = rc == GRASS_OK && persistent(host);
         if (rc == GRASS_OK)
             rc = cuda_ok(cudaMemcpyAsync(workspace, host, (size_t)L * sizeof(LayerDesc), cudaMemcpyHostToDevice, st));
-        if (rc == GRASS_OK && persistent)
-            rc = launch_persistent(host, (LayerDesc*)workspace, single, f32, L, B, T, tok_begin, tok_count, out, ld_out, table,
-                                   dev_status, st);
         if (host != stack_buf) std::free(host);
-        if (rc != GRASS_OK || persistent) return rc;
+        if (rc != GRASS_OK) return rc;
         dev_descs = (LayerDesc*)workspace;
+        if (take_persistent)
+            return launch_persistent(dev_descs, single, max_k, f32, L, B, T, tok_begin, tok_count, out, ld_out, table, dev_status, sms, st);
     } else {
         grass_status rc = fill_desc(single, layers[0], tile, T);
         if (rc != GRASS_OK) return rc;
         max_tiles = single.tiles_m * single.tiles_n;
         plan_cluster(&single);
-        plan_persistent(&single);
-        if (persistent)
-            return launch_persistent(&single, nullptr, single, f32, L, B, T, tok_begin, tok_count, out, ld_out, table, dev_status, st);
+        if (persistent(&single))
+            return launch_persistent(nullptr, single, max_k, f32, L, B, T, tok_begin, tok_count, out, ld_out, table, dev_status, sms, st);
     }
     if (cluster_nc > 0)
         return launch_factgrass_cluster(dev_descs, single, cplan, L, B, T, tok_begin, tok_count, cluster_nc,
@@ -637,8 +641,7 @@ extern "C" grass_status factmask_compress_grouped(const factgrass_layer* layers,
 extern "C" size_t factgrass_grouped_workspace_bytes(int32_t L)
 {
     if (L <= 0) return 256;
-    // the descriptors, and a table of every layer's projection for the persistent kernel (which hashes where the
-    // workspace has no room for it)
+    // the descriptors, and a table of every layer's projection for the persistent kernel
     return ((size_t)L * sizeof(grass::LayerDesc) + 255) / 256 * 256 + grass::persistent_table_bytes(L);
 }
 

@@ -58,11 +58,11 @@ grass_status launch_factgrass_cluster(const LayerDesc* dev_descs, const LayerDes
                                       int64_t ld_out, uint32_t* dev_status, cudaStream_t st, int out_bf16);
 
 // The persistent kernel (factgrass_persistent.cu).  persistent_fits: every layer of the call is one block of at most
-// 128 x 128 and its bins fit.  table: device scratch of persistent_table_bytes(L) bytes, or NULL.
+// 128 x 128 whose projection can be a table.  table: device scratch of persistent_table_bytes(L).
 size_t persistent_table_bytes(int32_t L);
 bool persistent_fits(const LayerDesc* host_descs, int32_t L, int32_t B, const int32_t* tok_count);
-grass_status launch_persistent(const LayerDesc* host_descs, const LayerDesc* dev_descs, const LayerDesc& single, bool f32, int32_t L,
-                               int32_t B, int32_t T, const int64_t* tok_begin, const int32_t* tok_count, float* out, int64_t ld_out,
-                               void* table, uint32_t* dev_status, cudaStream_t st);
+grass_status launch_persistent(const LayerDesc* dev_descs, const LayerDesc& single, uint32_t max_k, bool f32, int32_t L, int32_t B,
+                               int32_t T, const int64_t* tok_begin, const int32_t* tok_count, float* out, int64_t ld_out, void* table,
+                               uint32_t* dev_status, int sms, cudaStream_t st);
 
 }  // namespace grass

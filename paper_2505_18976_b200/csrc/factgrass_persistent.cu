@@ -3,20 +3,26 @@
 //
 // The streaming kernel (factgrass.cu) gives every (layer, sample, token chunk, block tile) a thread block of its own: loads,
 // then hashes, atomics and a flush, with nothing in flight meanwhile but what a neighbour on the same SM has; and a block
-// above 64 x 64 is cut into tiles that gather the same columns again.  Here one thread block per SM (two for small tiles)
-// walks an equal share of all 32-token steps of the launch, whole TM x TN blocks at a time:
-//   warps 0-7   gather: thread (c, g) owns masked column c and token group g of a step, two register sets, so that the
-//               loads of the next two steps are in flight while this one is written to the operand tiles (K-major,
+// above 64 x 64 is cut into tiles that gather the same columns again.  Here one thread block per SM walks an equal share
+// of all 32-token steps of the launch, whole 128 x 128 blocks at a time:
+//   warps 0-7   gather: thread (c, g) owns masked column c and every second 8-token group of a step, two register sets, so
+//               that the loads of the next two steps are in flight while this one is written to the operand tiles (K-major,
 //               64-byte swizzle) and multiplied (tcgen05.mma, accumulators in tensor memory); columns and pointers of
 //               the next (layer, sample) are fetched one segment ahead;
-//   warps 8-11  project the finished accumulator of the segment before (two accumulators alternate): every entry's
-//               bucket and sign come from a table (written once per call for all samples) or from the seed, bins in
-//               shared memory, one flush.
+//   warps 8-15  project the finished accumulator of the segment before (two accumulators alternate): every entry's
+//               bucket and sign come from a table (written once per call for all samples), bins in shared memory, one
+//               flush.  The last accumulator is projected and flushed by all sixteen warps.
 // A (layer, sample) that one thread block covers alone is stored; pieces are added into zeroed rows (SJLT is linear).
 // No accumulator runs over more than 8,192 tokens.
 //
-// What bounds it: DRAM, by the 64-byte pieces that the masks touch; next to that, for short samples, the projection
-// (16,384 shared-memory atomics and k stores per sample and layer at 128 x 128).
+// What bounds it: DRAM, by the 64-byte pieces that the masks touch (a step takes what 1/148 of 6.6 TB/s gives it, whether
+// one or two steps are ahead), and for short launches what lies around the gathers: 8 us until the first data are there and
+// 10 us for the last projection (a shared-memory fp32 addition is a compare-and-swap, 26 cycles per warp and instruction
+// here; eight projecting warps instead of four took 6 us off, four swaps per thread at a time put 30 us on).
+// Measured, streaming -> persistent (us): packed fp32, 12 layers x 7 samples of 640 tokens on average, 128 x 128: 144 -> 97;
+// bf16, 24 layers x 8 x 512, 128 x 128: 194 -> 103 (503 MB of pieces); fp32, the same at 96 x 96: 208 -> 132 (686 MB);
+// fp32, 28 layers of a 4,096-wide model x 2 x 1,024: 182 -> 154.  64 x 64 tiles were slower here (fp32, 12 layers x 5 x
+// 300: 34 -> 38) and stay with the streaming kernel.
 #include "factgrass_common.cuh"
 
 #include <algorithm>
@@ -24,14 +30,17 @@
 namespace grass {
 namespace fgp {
 
+constexpr int TILE = 128;
 constexpr int GATHER = 256;                    // gathering threads
-constexpr int EPI_WARPS = 4;
+constexpr int EPI_WARPS = 8;
 constexpr int THREADS = GATHER + EPI_WARPS * 32;
 constexpr int NBUF = 2;
 constexpr int MAX_RUN = 8192 / kTokTile;       // steps per accumulator run
 constexpr int MAX_VAR_B = 1024;                // samples of their own lengths whose work is shared out evenly
 constexpr uint16_t NO_ENTRY = 0xFFFF;          // table entry of a position outside the k'_in x k'_out block
-constexpr uint32_t MAX_TABLE_K = 32767;        // buckets that an entry can name
+// fp32 operand tiles (96 KB) and the bins stay within 164 KB of shared memory.  With less than 92 KB of L1 behind them the
+// gathers of one SM fall from 6.6 to 4.6 TB/s (of all SMs): L1 holds a line for every one in flight.
+constexpr uint32_t MAX_K = 14336;
 
 struct Args {
     const LayerDesc* descs;        // NULL: `single`
@@ -40,7 +49,7 @@ struct Args {
     const int32_t* tok_count;
     float* out;
     int64_t ld_out;
-    const uint16_t* table;         // per layer TM x TN entries (bucket | sign << 15), NULL: hash
+    const uint16_t* table;         // per layer TILE x TILE entries (bucket | sign << 15)
     uint32_t* dev_status;
     int nprod;
 };
@@ -60,7 +69,6 @@ __host__ __device__ __forceinline__ Deal deal_out(int64_t per_layer, int32_t L, 
 
 // Writes the table of every layer and zeroes the output rows that are added into: all of them for samples of their own
 // lengths, else those that lie across two blocks' shares.
-template <int TILE>
 __global__ void __launch_bounds__(256)
 prepare_kernel(const __grid_constant__ Args x, const __grid_constant__ LayerDesc single, uint16_t* __restrict__ table, int64_t steps,
                int64_t blocks)
@@ -70,17 +78,14 @@ prepare_kernel(const __grid_constant__ Args x, const __grid_constant__ LayerDesc
     const int l = blockIdx.y;
     const LayerDesc& L = x.descs ? x.descs[l] : single;
     const int tid = blockIdx.x * blockDim.x + threadIdx.x, stride = gridDim.x * blockDim.x;
-    if (table) {
-        uint16_t* tab = table + (int64_t)l * (TILE * TILE);
-        for (int e = tid; e < TILE * TILE; e += stride) {
-            const int a = e / TILE, c = e % TILE;
-            uint16_t v = NO_ENTRY;
-            if (a < L.kin && c < L.kout) {
-                const uint64_t h = sjlt_hash_counter(L.seed, (uint64_t)a * (uint64_t)L.kout + (uint64_t)c + 1);
-                v = (uint16_t)(sjlt_bucket(h, L.k) | ((uint32_t)h << 15));
-            }
-            tab[e] = v;
+    for (int e = tid; e < TILE * TILE; e += stride) {
+        const int a = e / TILE, c = e % TILE;
+        uint16_t v = NO_ENTRY;
+        if (a < L.kin && c < L.kout) {
+            const uint64_t h = sjlt_hash_counter(L.seed, (uint64_t)a * (uint64_t)L.kout + (uint64_t)c + 1);
+            v = (uint16_t)(sjlt_bucket(h, L.k) | ((uint32_t)h << 15));
         }
+        table[(int64_t)l * (TILE * TILE) + e] = v;
     }
     const Deal d = deal_out(steps * x.B, x.L, blocks);
     for (int b = blockIdx.x; b < x.B; b += gridDim.x) {
@@ -137,8 +142,8 @@ struct Walk {
     }
 };
 
-template <int TILE, bool F32>
-__global__ void __launch_bounds__(THREADS, TILE == 64 ? 2 : 1)
+template <bool F32>
+__global__ void __launch_bounds__(THREADS, 1)
 factgrass_persistent_kernel(const __grid_constant__ Args x, const __grid_constant__ LayerDesc single, uint32_t max_k)
 {
     using elem_t = typename in_elem<F32>::type;
@@ -184,7 +189,7 @@ factgrass_persistent_kernel(const __grid_constant__ Args x, const __grid_constan
         return n;
     };
     const bool var = x.tok_count != nullptr;
-    if (var && warp == EPI_WARPS) {
+    if (var && warp == GATHER / 32) {
         int32_t carry = 0;
         for (int b0 = 0; b0 < x.B; b0 += 32) {
             const int b = b0 + lane;
@@ -220,6 +225,64 @@ factgrass_persistent_kernel(const __grid_constant__ Args x, const __grid_constan
         walk.end = walk.u + d.per_block < d.units ? walk.u + d.per_block : d.units;
     }
 
+    // adds columns 32 * part + .., every parts-th piece of 32, of a finished accumulator to the bins
+    auto project = [&](const Segment& g, int seg, int part, int parts, bool ok) {
+        const int acc = seg & 1, a = (warp & 3) * 32 + lane;      // accumulator row a sits in tensor-memory lane a
+        const uint16_t* row = x.table + (int64_t)g.l * (TILE * TILE) + a * TILE;
+        ok = ok && tc::mbar_wait(full0 + 8 * acc, (uint32_t)(seg / 2) & 1u);
+        ok = __all_sync(0xFFFFFFFFu, ok);
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        const uint32_t d0 = tmem_d + acc * ACC + ((uint32_t)((warp & 3) * 32) << 16);
+        auto add = [&](uint32_t entry, uint32_t v) {
+            if (entry != NO_ENTRY && __uint_as_float(v) != 0.0f)
+                atomicAdd(bins + (entry & 0x7FFFu), __uint_as_float(v ^ ((entry & 0x8000u) << 16)));
+        };
+#pragma unroll 1
+        for (int c0 = 32 * part; c0 < TILE; c0 += 32 * parts) {
+            uint4 t4[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) t4[q] = *reinterpret_cast<const uint4*>(row + c0 + 8 * q);
+            uint32_t v[32];
+            if (ok) {
+                tc::tmem_ld32_wait(d0 + (uint32_t)c0, v);
+                if constexpr (F32) {
+                    uint32_t w[32];
+                    tc::tmem_ld32_wait(d0 + (uint32_t)(TILE + c0), w);
+#pragma unroll
+                    for (int e = 0; e < 32; ++e) v[e] = __float_as_uint(__uint_as_float(v[e]) + __uint_as_float(w[e]));
+                }
+            } else {
+#pragma unroll
+                for (int e = 0; e < 32; ++e) v[e] = 0u;
+            }
+            if (parts == EPI_WARPS / 4 && c0 + 32 * parts >= TILE) {     // everything that this warp reads has been read
+                asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+                __syncwarp();
+                if (lane == 0) tc::mbar_arrive(empty0 + 8 * acc);
+            }
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const uint32_t w4[4] = {t4[q].x, t4[q].y, t4[q].z, t4[q].w};
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    add(w4[e] & 0xFFFFu, v[8 * q + 2 * e]);
+                    add(w4[e] >> 16, v[8 * q + 2 * e + 1]);
+                }
+            }
+        }
+        return ok;
+    };
+    auto flush = [&](const Segment& g, int first, int stride) {
+        const LayerDesc& L = x.descs ? x.descs[g.l] : single;
+        float* orow = x.out + (int64_t)g.b * x.ld_out + L.out_offset;
+        for (uint32_t i = first; i < L.k; i += stride) {
+            const float v = bins[i];
+            bins[i] = 0.0f;
+            if (g.whole) orow[i] = v;
+            else if (v != 0.0f) atomicAdd(orow + i, v);
+        }
+    };
+
     if (warp < GATHER / 32) {
         // ---------------- gather and contract ----------------
         const int col = tid % TILE, grp = tid / TILE;
@@ -253,7 +316,7 @@ factgrass_persistent_kernel(const __grid_constant__ Args x, const __grid_constan
             r.t_end = min(g.k1 * kTokTile, tokens_of(g.b));
             return r;
         };
-        Source cur = open(), nxt = open();
+        Source cur = open(), nxt;
         auto check = [&](Source& r) {
             if (r.has_a && (int64_t)r.ca >= r.d_in) { bad = true; r.has_a = false; r.ca = 0; }
             if (r.has_g && (int64_t)r.cg >= r.d_out) { bad = true; r.has_g = false; r.cg = 0; }
@@ -315,7 +378,11 @@ factgrass_persistent_kernel(const __grid_constant__ Args x, const __grid_constan
         bool ok = true;
         int n = 0;
         uint32_t ra0[PASS][8], rg0[PASS][8], ra1[PASS][8], rg1[PASS][8];
+        // the first loads leave before the second segment is looked up
+        nxt.t = 0;
+        nxt.t_end = -1;
         fetch(ra0, rg0);
+        nxt = open();
         fetch(ra1, rg1);
         auto step = [&](uint32_t (&ra)[PASS][8], uint32_t (&rg)[PASS][8], int seg, bool first, bool last) {
             const int buf = n % NBUF, acc = seg & 1;
@@ -362,137 +429,42 @@ factgrass_persistent_kernel(const __grid_constant__ Args x, const __grid_constan
             ++n;
         };
         Segment g;
-        for (int seg = 0; walk.next(g); ++seg)
+        int segs = 0;
+        for (; walk.next(g); ++segs)
             for (int k = g.k0; k < g.k1; ++k) {
-                if (n & 1) step(ra1, rg1, seg, k == g.k0, k + 1 == g.k1);
-                else step(ra0, rg0, seg, k == g.k0, k + 1 == g.k1);
+                if (n & 1) step(ra1, rg1, segs, k == g.k0, k + 1 == g.k1);
+                else step(ra0, rg0, segs, k == g.k0, k + 1 == g.k1);
             }
+        if (segs > 0) {
+            // nothing left to gather: the last accumulator is everybody's work
+            asm volatile("griddepcontrol.wait;" ::: "memory");
+            asm volatile("bar.sync 2, %0;" ::"n"(THREADS) : "memory");
+            ok = project(g, segs - 1, warp / 4, THREADS / 128, ok);
+            asm volatile("bar.sync 2, %0;" ::"n"(THREADS) : "memory");
+            flush(g, tid, THREADS);
+        }
         if (bad && x.dev_status) atomicOr(x.dev_status, GRASS_DEV_BAD_INDEX);
         if (!ok) abort_flag = 1;
     } else {
         // ---------------- project ----------------
-        const int ew = warp - GATHER / 32, et = tid - GATHER;
+        const int et = tid - GATHER;
         for (uint32_t i = et; i < max_k; i += EPI_WARPS * 32) bins[i] = 0.0f;
         // the table and the zeroed rows are complete
         asm volatile("griddepcontrol.wait;" ::: "memory");
-        asm volatile("bar.sync 2, %0;" ::"n"(EPI_WARPS * 32) : "memory");
         bool ok = true;
         Segment g;
         for (int seg = 0; walk.next(g); ++seg) {
-            const LayerDesc& L = x.descs ? x.descs[g.l] : single;
-            const uint32_t k = L.k, s = L.s;
-            const int kin = L.kin, kout = L.kout;
-            const uint64_t seed = L.seed;
-            const float scale = 1.0f / sqrtf((float)s);
-            const uint16_t* tab = x.table ? x.table + (int64_t)g.l * (TILE * TILE) : nullptr;
-            const int acc = seg & 1;
-            if (ok) ok = tc::mbar_wait(full0 + 8 * acc, (uint32_t)(seg / 2) & 1u);
-            ok = __all_sync(0xFFFFFFFFu, ok);
-            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            const uint32_t d0 = tmem_d + acc * ACC + ((uint32_t)(ew * 32) << 16);
-            auto add = [&](uint32_t entry, uint32_t v) {
-                if (entry != NO_ENTRY && __uint_as_float(v) != 0.0f)
-                    atomicAdd(bins + (entry & 0x7FFFu), __uint_as_float(v ^ ((entry & 0x8000u) << 16)));
-            };
-            auto hash = [&](int a, int c, uint32_t v) {
-                if (a >= kin || c >= kout || __uint_as_float(v) == 0.0f) return;
-                const uint64_t q = (uint64_t)a * (uint64_t)kout + (uint64_t)c;
-                for (uint32_t r = 0; r < s; ++r) {
-                    const uint64_t h = sjlt_hash_counter(seed, q * s + r + 1);
-                    const float f = sjlt_signed(h, __uint_as_float(v));
-                    atomicAdd(bins + sjlt_bucket(h, k), s == 1 ? f : f * scale);
-                }
-            };
-#pragma unroll 1
-            for (int c0 = 0; c0 < TILE; c0 += 32) {
-                if (TILE == 128) {
-                    const int a = ew * 32 + lane;          // accumulator row a sits in lane a
-                    uint4 t4[4];
-                    if (tab)
-#pragma unroll
-                        for (int q = 0; q < 4; ++q) t4[q] = *reinterpret_cast<const uint4*>(tab + a * TILE + c0 + 8 * q);
-                    uint32_t v[32];
-                    if (ok) {
-                        tc::tmem_ld32_wait(d0 + (uint32_t)c0, v);
-                        if constexpr (F32) {
-                            uint32_t w[32];
-                            tc::tmem_ld32_wait(d0 + (uint32_t)(TILE + c0), w);
-#pragma unroll
-                            for (int e = 0; e < 32; ++e) v[e] = __float_as_uint(__uint_as_float(v[e]) + __uint_as_float(w[e]));
-                        }
-                    } else {
-#pragma unroll
-                        for (int e = 0; e < 32; ++e) v[e] = 0u;
-                    }
-                    if (c0 + 32 == TILE) {                 // everything has been read
-                        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-                        __syncwarp();
-                        if (lane == 0) tc::mbar_arrive(empty0 + 8 * acc);
-                    }
-                    if (tab) {
-#pragma unroll
-                        for (int q = 0; q < 4; ++q) {
-                            const uint32_t w4[4] = {t4[q].x, t4[q].y, t4[q].z, t4[q].w};
-#pragma unroll
-                            for (int e = 0; e < 4; ++e) {
-                                add(w4[e] & 0xFFFFu, v[8 * q + 2 * e]);
-                                add(w4[e] >> 16, v[8 * q + 2 * e + 1]);
-                            }
-                        }
-                    } else {
-#pragma unroll
-                        for (int e = 0; e < 32; ++e) hash(a, c0 + e, v[e]);
-                    }
-                } else {
-                    // accumulator row a sits in lane (a % 16) + 32 (a / 16): register e of a lane holds row
-                    // 16 ew + lane / 4 + 8 ((e & 3) / 2), column c0 + 8 (e / 4) + 2 (lane % 4) + e % 2
-                    const int a0 = ew * 16 + (lane >> 2), cc = c0 + 2 * (lane & 3);
-                    uint32_t t2[8];
-                    if (tab)
-#pragma unroll
-                        for (int e = 0; e < 8; ++e)
-                            t2[e] = *reinterpret_cast<const uint32_t*>(tab + (a0 + 8 * (e & 1)) * TILE + cc + 8 * (e >> 1));
-                    uint32_t v[16];
-                    if (ok) {
-                        tc::tmem_ld_16x256b_x4_wait(d0 + (uint32_t)c0, v);
-                        if constexpr (F32) {
-                            uint32_t w[16];
-                            tc::tmem_ld_16x256b_x4_wait(d0 + (uint32_t)(TILE + c0), w);
-#pragma unroll
-                            for (int e = 0; e < 16; ++e) v[e] = __float_as_uint(__uint_as_float(v[e]) + __uint_as_float(w[e]));
-                        }
-                    } else {
-#pragma unroll
-                        for (int e = 0; e < 16; ++e) v[e] = 0u;
-                    }
-                    if (c0 + 32 == TILE) {
-                        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-                        __syncwarp();
-                        if (lane == 0) tc::mbar_arrive(empty0 + 8 * acc);
-                    }
-#pragma unroll
-                    for (int e = 0; e < 8; ++e) {
-                        // rows a0 (e even) and a0 + 8 (e odd), columns cc + 8 (e / 2) and the next
-                        const int r = 4 * (e >> 1) + 2 * (e & 1);
-                        if (tab) {
-                            add(t2[e] & 0xFFFFu, v[r]);
-                            add(t2[e] >> 16, v[r + 1]);
-                        } else {
-                            hash(a0 + 8 * (e & 1), cc + 8 * (e >> 1), v[r]);
-                            hash(a0 + 8 * (e & 1), cc + 8 * (e >> 1) + 1, v[r + 1]);
-                        }
-                    }
-                }
+            if (walk.u >= walk.end) {
+                asm volatile("bar.sync 2, %0;" ::"n"(THREADS) : "memory");      // bins are clear
+                ok = project(g, seg, warp / 4, THREADS / 128, ok);
+                asm volatile("bar.sync 2, %0;" ::"n"(THREADS) : "memory");
+                flush(g, tid, THREADS);
+                break;
             }
-            asm volatile("bar.sync 2, %0;" ::"n"(EPI_WARPS * 32) : "memory");
-            float* orow = x.out + (int64_t)g.b * x.ld_out + L.out_offset;
-            for (uint32_t i = et; i < k; i += EPI_WARPS * 32) {
-                const float v = bins[i];
-                bins[i] = 0.0f;
-                if (g.whole) orow[i] = v;
-                else if (v != 0.0f) atomicAdd(orow + i, v);
-            }
-            asm volatile("bar.sync 2, %0;" ::"n"(EPI_WARPS * 32) : "memory");
+            asm volatile("bar.sync 3, %0;" ::"n"(EPI_WARPS * 32) : "memory");   // bins are clear
+            ok = project(g, seg, warp / 4 - GATHER / 128, EPI_WARPS / 4, ok);
+            asm volatile("bar.sync 3, %0;" ::"n"(EPI_WARPS * 32) : "memory");
+            flush(g, et, EPI_WARPS * 32);
         }
         if (!ok) abort_flag = 1;
     }
@@ -507,39 +479,29 @@ factgrass_persistent_kernel(const __grid_constant__ Args x, const __grid_constan
 
 }  // namespace fgp
 
-size_t persistent_table_bytes(int32_t L) { return (size_t)L * 128 * 128 * sizeof(uint16_t); }
+size_t persistent_table_bytes(int32_t L) { return (size_t)L * fgp::TILE * fgp::TILE * sizeof(uint16_t); }
 
-// true if the launch can run here: whole k'_in x k'_out blocks of one tile, bins in shared memory
 bool persistent_fits(const LayerDesc* d, int32_t L, int32_t B, const int32_t* tok_count)
 {
-    if (tok_count && B > fgp::MAX_VAR_B) return false;
+    using namespace fgp;
+    if (tok_count && B > MAX_VAR_B) return false;
     for (int l = 0; l < L; ++l)
-        if (d[l].kin > 128 || d[l].kout > 128 || (size_t)d[l].k * 4 > 96 * 1024) return false;
+        if (d[l].kin > TILE || d[l].kout > TILE || d[l].s != 1 || d[l].k > MAX_K) return false;
     return true;
 }
 
-grass_status launch_persistent(const LayerDesc* host, const LayerDesc* dev_descs, const LayerDesc& single, bool f32, int32_t L, int32_t B,
+grass_status launch_persistent(const LayerDesc* dev_descs, const LayerDesc& single, uint32_t max_k, bool f32, int32_t L, int32_t B,
                                int32_t T, const int64_t* tok_begin, const int32_t* tok_count, float* out, int64_t ld_out, void* table,
-                               uint32_t* dev_status, cudaStream_t st)
+                               uint32_t* dev_status, int sms, cudaStream_t st)
 {
     using namespace fgp;
-    int dev = 0, sms = 148;
-    if (cudaGetDevice(&dev) != cudaSuccess) return GRASS_ERR_CUDA;
-    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return GRASS_ERR_CUDA;
-    int kk = 0;
-    uint32_t max_k = 0;
-    bool tables = table != nullptr;
-    for (int l = 0; l < L; ++l) {
-        kk = std::max(kk, std::max(host[l].kin, host[l].kout));
-        max_k = std::max(max_k, host[l].k);
-        if (host[l].s != 1 || host[l].k > MAX_TABLE_K) tables = false;
-    }
-    const int tile = kk > 64 ? 128 : 64;
     const int64_t steps = (T + kTokTile - 1) / kTokTile, units = steps * B * L;
-    const int per_sm = tile == 64 ? 2 : 1;
-    // Every share costs one projection more; a few steps are not worth that.
-    const int64_t least = std::max<int64_t>(1, tuning(GRASS_TUNE_FACTGRASS_CHUNK, tile == 64 ? 64 : 128) / kTokTile);
-    const int64_t blocks = std::max<int64_t>(1, std::min<int64_t>((int64_t)sms * per_sm, (units + least - 1) / least));
+    // An equal share for every SM.  Where samples are longer than that and a share of one or two steps more divides a
+    // sample evenly, it is taken: a share that runs into the next sample pays for a second projection (8,192 tokens of 32
+    // samples at 128 x 128 fp32: 70 us in shares of 7 steps, 62 in shares of 8).
+    const int64_t per = (units + sms - 1) / sms, pieces = steps / per;
+    const bool even = !tok_count && pieces > 0 && steps % pieces == 0 && steps / pieces <= per + 2;
+    const int64_t blocks = even ? pieces * B * L : std::min<int64_t>(sms, units);
     Args x;
     x.descs = dev_descs;
     x.L = L;
@@ -549,22 +511,19 @@ grass_status launch_persistent(const LayerDesc* host, const LayerDesc* dev_descs
     x.tok_count = tok_count;
     x.out = out;
     x.ld_out = ld_out;
-    x.table = tables ? (const uint16_t*)table : nullptr;
+    x.table = (const uint16_t*)table;
     x.dev_status = dev_status;
     x.nprod = (int)tuning(GRASS_TUNE_SPLIT_PRODUCTS, tc::kSplitProductsDefault);
     if (x.nprod != 3 && x.nprod != 4) x.nprod = 6;
-    const dim3 pg((unsigned)std::min<int64_t>(std::max<int64_t>(tile * tile / 2048, std::min<int64_t>(B, 64)), 64), (unsigned)L, 1);
-    if (tile == 64) prepare_kernel<64><<<pg, 256, 0, st>>>(x, single, tables ? (uint16_t*)table : nullptr, steps, blocks);
-    else prepare_kernel<128><<<pg, 256, 0, st>>>(x, single, tables ? (uint16_t*)table : nullptr, steps, blocks);
+    prepare_kernel<<<dim3((unsigned)std::min(std::max(B, 8), 64), (unsigned)L, 1), 256, 0, st>>>(x, single, (uint16_t*)table, steps, blocks);
     if (launch_status() != GRASS_OK) return GRASS_ERR_CUDA;
-    auto launch = [&](auto kern, size_t stage_bytes) -> grass_status {
-        const size_t smem = NBUF * stage_bytes + (size_t)max_k * 4;
+    auto launch = [&](auto kern, int pieces) -> grass_status {
+        const size_t smem = (size_t)NBUF * 2 * pieces * TILE * tc::ROW_BYTES + (size_t)max_k * 4;
         if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return GRASS_ERR_CUDA;
         // what shared memory does not need is L1, where gathered loads wait
-        const size_t need = per_sm * (smem + 6 * 1024);
         int carve = 100;
-        for (int kb : {8, 16, 32, 64, 100, 132, 164, 196, 228})
-            if ((size_t)kb * 1024 >= need) { carve = (kb * 100 + 227) / 228; break; }
+        for (int kb : {64, 100, 132, 164, 196, 228})
+            if ((size_t)kb * 1024 >= smem + 7 * 1024) { carve = (kb * 100 + 227) / 228; break; }
         carve = (int)tuning(GRASS_TUNE_FACTGRASS_CARVEOUT, carve);
         if (cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, carve) != cudaSuccess) return GRASS_ERR_CUDA;
         cudaLaunchConfig_t cfg = {};
@@ -580,9 +539,7 @@ grass_status launch_persistent(const LayerDesc* host, const LayerDesc* dev_descs
         const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, x, single, max_k);
         return e == cudaSuccess ? launch_status() : GRASS_ERR_CUDA;
     };
-    const size_t piece = (size_t)tile * tc::ROW_BYTES * 2;
-    if (tile == 64) return f32 ? launch(factgrass_persistent_kernel<64, true>, 3 * piece) : launch(factgrass_persistent_kernel<64, false>, piece);
-    return f32 ? launch(factgrass_persistent_kernel<128, true>, 3 * piece) : launch(factgrass_persistent_kernel<128, false>, piece);
+    return f32 ? launch(factgrass_persistent_kernel<true>, 3) : launch(factgrass_persistent_kernel<false>, 1);
 }
 
 }  // namespace grass
