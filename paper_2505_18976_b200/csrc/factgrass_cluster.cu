@@ -7,17 +7,22 @@
 //   stages 1-2  every block gathers its own token range into K-major operand tiles and contracts it on the
 //               tensor core (tcgen05.mma, bf16 in / fp32 in tensor memory) into a PARTIAL k'_in x k'_out block;
 //   exchange    block r of the cluster owns rows [r TM/NC, (r+1) TM/NC) of the sample's block: every block writes
-//               those rows of its partial block from tensor memory straight into a receive area in the owner's
-//               shared memory (distributed shared memory stores, posted: nobody waits for a remote load);
-//   stage 3     after a cluster barrier the owner adds the NC partial slices it received, so that every entry of
-//               Eq. 2's block is complete in exactly one thread block, hashes it from the seed (once per sample,
-//               not once per token chunk) and adds it into its own k-bin accumulator;
+//               the others' rows of its partial block from tensor memory into its operand tiles, which are free by then,
+//               and sends each owner its slice with one bulk copy that counts on the owner's barrier (16-byte stores
+//               into the owners' memory plus a cluster barrier, 4.2 us at 128 x 128 over four blocks, took 0.6 us more);
+//   stage 3     the owner adds the NC partial slices it received, so that every entry of Eq. 2's block is complete in
+//               exactly one thread block, hashes it from the seed (once per sample, not once per token chunk) and adds
+//               it into its own k-bin accumulator;
 //   reduce      slice r of the output row belongs to block r: every block writes the r-th slice of its
 //               accumulator into the owner's second receive area, and after one more cluster barrier the owner
 //               adds the NC slices and writes its part of the row with plain stores: no zero-fill, no global
 //               atomics, and no thread block touches another's memory after the last barrier.
 // The block must fit one TM x TN tile (k'_in, k'_out <= 128) and the accumulators must fit in shared memory;
 // everything else takes the streaming kernel.
+//
+// What bounds it: DRAM for the gathers (32 x 512 tokens, 768 x 3,072, 128 x 128: 14.4 us for 100 MB of 64-byte pieces), and
+// around them 3 us until the first loads are out and 9 us of exchange, projection and reduction, which nothing
+// overlaps in a launch of one wave: 28.3 us in all (28.9 with the exchange by plain stores).
 #include "factgrass_common.cuh"
 
 #include <cooperative_groups.h>
@@ -116,6 +121,7 @@ factgrass_cluster_kernel(const LayerDesc* __restrict__ descs, const __grid_const
 
     extern __shared__ __align__(1024) unsigned char smem[];
     __shared__ __align__(8) unsigned long long bars[NBUF + 1];
+    __shared__ __align__(8) unsigned long long recv_bar;      // every other block's slice has landed in the receive area
     __shared__ uint32_t tmem_slot;
     __shared__ int abort_flag;
     // operand tiles | receive area for partial blocks | k bins | receive area for bin slices (NC x ceil(k / NC)).
@@ -126,11 +132,19 @@ factgrass_cluster_kernel(const LayerDesc* __restrict__ descs, const __grid_const
 
     cg::cluster_group cluster = cg::this_cluster();
     const uint32_t nc = cluster.num_blocks(), rank = cluster.block_rank();
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const bool nc_ok = nc == 1 || nc == 2 || nc == 4 || nc == 8;    // the launcher forms no other clusters
+    const int rows = TM / (int)(nc_ok ? nc : 1);
+    const uint32_t slice_bytes = (uint32_t)(rows * TN * 4), bar_recv = tc::smem_u32(&recv_bar);
+    if (tid == 0) {
+        tc::mbar_init(bar_recv, 1);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        tc::expect_tx(bar_recv, nc_ok ? (nc - 1) * slice_bytes : 0u);
+    }
     // "I have started": the other half of this barrier is waited for just before the first write into another thread
     // block's shared memory, which is only defined once that thread block is running (by then everyone has arrived)
     asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
     const LayerDesc& L = descs ? descs[blockIdx.z] : single;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int b = blockIdx.y;
     const int kin = L.kin, kout = L.kout;
     const int64_t d_in = L.d_in, d_out = L.d_out;
@@ -254,12 +268,26 @@ factgrass_cluster_kernel(const LayerDesc* __restrict__ descs, const __grid_const
     if (!ok && tid == 0 && dev_status) atomicOr(dev_status, GRASS_DEV_TIMEOUT);
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 
-    // exchange: the rows of the partial block go from tensor memory to their owners (zeros where there was no work).
+    // exchange: the rows of the partial block go from tensor memory to their owners (zeros where there was no work): this
+    // block's own into its receive area, the others' into shared memory that is free here (the operand tiles, then the
+    // second receive area) and on by one bulk copy each.
     // Accumulator row a sits in tensor-memory lane a (TM = 128) or lane (a % 16) + 32 * (a / 16) (TM = 64);
     // warp w may read lanes 32 * (w % 4) .. + 31; the two warps that share a lane quarter split the columns.
+    // Slices for which there is no room (8 x 8 KB, small k) leave as stores that count on the owner's barrier.
+    const int in_tiles = NBUF * STAGE / (int)slice_bytes;       // slices that the operand tiles hold
+    const int in_bins = (int)(k * 4 / slice_bytes);             // and the second receive area
+    auto staged = [&](uint32_t owner) -> float* {
+        if (owner == rank) return recv + (int)rank * (rows * TN);
+        const int i = (int)(owner - (owner > rank ? 1u : 0u));
+        if (i < in_tiles) return reinterpret_cast<float*>(smem) + i * (rows * TN);
+        return i - in_tiles < in_bins ? recv_bins + (i - in_tiles) * (rows * TN) : nullptr;
+    };
+    auto in_cluster = [](const void* p, uint32_t block) {
+        uint32_t a;
+        asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(tc::smem_u32(p)), "r"(block));
+        return a;
+    };
     asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");     // every thread block of the cluster runs
-    const bool nc_ok = nc == 1 || nc == 2 || nc == 4 || nc == 8;    // the launcher forms no other clusters
-    const int rows = TM / (int)(nc_ok ? nc : 1);
     if (nc_ok) {
         const int quarter = warp & 3;
         const uint32_t tq = tmem_d + ((uint32_t)(quarter * 32) << 16);
@@ -278,12 +306,11 @@ factgrass_cluster_kernel(const LayerDesc* __restrict__ descs, const __grid_const
             for (int e = 0; e < 16; e += 2) {
                 const int a = quarter * 16 + (lane >> 2) + 8 * ((e & 3) >> 1);
                 const int c = c0 + 8 * (e >> 2) + 2 * (lane & 3);
-                float* dst = cluster.map_shared_rank(recv, a / rows) + (int)rank * (rows * TN);
-                *reinterpret_cast<uint2*>(dst + recv_offset<TN>(a % rows, c)) = make_uint2(v[e], v[e + 1]);
+                *reinterpret_cast<uint2*>(staged(a / rows) + recv_offset<TN>(a % rows, c)) = make_uint2(v[e], v[e + 1]);
             }
         } else {
             const int a = quarter * 32 + lane;
-            float* dst = cluster.map_shared_rank(recv, a / rows) + (int)rank * (rows * TN);
+            float* dst = staged(a / rows);
 #pragma unroll 1
             for (int c0 = (warp >> 2) * 32; c0 < TN; c0 += 64) {
                 uint32_t v[32];
@@ -294,22 +321,44 @@ factgrass_cluster_kernel(const LayerDesc* __restrict__ descs, const __grid_const
 #pragma unroll
                     for (int e = 0; e < 32; ++e) v[e] = 0u;
                 }
+                if (dst) {
 #pragma unroll
-                for (int e = 0; e < 32; e += 4)
-                    *reinterpret_cast<uint4*>(dst + recv_offset<TN>(a % rows, c0 + e)) =
-                        make_uint4(v[e], v[e + 1], v[e + 2], v[e + 3]);
+                    for (int e = 0; e < 32; e += 4)
+                        *reinterpret_cast<uint4*>(dst + recv_offset<TN>(a % rows, c0 + e)) =
+                            make_uint4(v[e], v[e + 1], v[e + 2], v[e + 3]);
+                } else {
+                    const uint32_t far = in_cluster(recv + (int)rank * (rows * TN), a / rows), bar = in_cluster(&recv_bar, a / rows);
+#pragma unroll
+                    for (int e = 0; e < 32; e += 4)
+                        asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v4.b32 [%0], {%1, %2, %3, %4}, [%5];"
+                                     ::"r"(far + 4 * recv_offset<TN>(a % rows, c0 + e)), "r"(v[e]), "r"(v[e + 1]), "r"(v[e + 2]),
+                                     "r"(v[e + 3]), "r"(bar)
+                                     : "memory");
+                }
             }
         }
     } else if (tid == 0 && dev_status) {
         atomicOr(dev_status, GRASS_DEV_TIMEOUT);
     }
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
+    if (nc_ok && tid < (int)nc && tid != (int)rank) {
+        const float* src = staged((uint32_t)tid);
+        if (src)
+            asm volatile("cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+                         ::"r"(in_cluster(recv + (int)rank * (rows * TN), tid)), "r"(tc::smem_u32(src)), "r"(slice_bytes),
+                           "r"(in_cluster(&recv_bar, tid))
+                         : "memory");
+    }
     if (warp == 0) {
         __syncwarp();
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_d), "r"(ACC_COLS) : "memory");
     }
-    cluster.sync();      // every thread block holds the NC partial slices of its rows
+    if (!tc::mbar_wait(bar_recv, 0) && tid == 0 && dev_status) atomicOr(dev_status, GRASS_DEV_TIMEOUT);
+    __syncwarp();
+    // "I hold every slice": waited for before the bins go out, because they land where others may still copy from
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
 
     // stage 3 in the owner of the rows
     {
@@ -323,6 +372,7 @@ factgrass_cluster_kernel(const LayerDesc* __restrict__ descs, const __grid_const
         }
     }
     __syncthreads();     // this thread block's accumulator is final
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 
     // reduce: slice o of the accumulator goes to thread block o's second receive area ...
     if (nc_ok) {

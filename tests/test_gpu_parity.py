@@ -292,6 +292,19 @@ def test_factgrass_parity(G, W, oracle_mod, kw):
     _fact_case(G, W, oracle_mod, _fact_cfg(W, **kw))
 
 
+@pytest.mark.parametrize("T,k,kin,kout", [
+    (600, 100, 128, 128),       # eight blocks: slices in the operand tiles, the rest as counted stores
+    (600, 2_048, 100, 65),      # one more slice in the second receive area
+    (600, 6_200, 128, 128),     # all slices by bulk copy
+    (260, 100, 128, 128),       # four blocks
+    (260, 4_096, 65, 128),
+    (130, 100, 128, 128),       # two blocks
+    (600, 100, 64, 33),         # eight blocks, 64 x 64 tile
+])
+def test_factgrass_cluster_exchange(G, W, oracle_mod, T, k, kin, kout):
+    _fact_case(G, W, oracle_mod, _fact_cfg(W, layers=(W.LinearLayer("l", 200, 300),), B=2, T=T, k=k, kin=kin, kout=kout))
+
+
 @pytest.mark.parametrize("kw", [
     dict(),
     dict(kin=64, kout=64, k=1024, T=200, B=4),
