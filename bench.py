@@ -246,12 +246,11 @@ class FactJob:
         self.fetch_bytes_per_launch = line
         self.dense_bytes_per_launch = self.dense
         self.launches_per_step = 1
-        nb = (cfg.k + 63) // 64
         # the grouped call is one kernel when it takes the cluster kernel (few (layer, sample) items: config 3), else a
         # zero-fill kernel and the streaming kernel (the library's rule: items <= thread-block slots of one wave)
         items, slots = len(cfg.layers) * cfg.B, 148 * (1 if max(cfg.kin, cfg.kout) > 64 else 2)
         fact_kernels = 1 if (items <= slots and not fp32_inputs and max(cfg.kin, cfg.kout) <= 128) else 2
-        self.kernels_per_step = fact_kernels + (1 if self.score else 0) + ((2 + 3 * nb + 4 * nb) if self.precondition else 0)
+        self.kernels_per_step = fact_kernels + (1 if self.score else 0) + (3 if self.precondition else 0)      # FIM, factor, solve
         self.dominant = "factgrass_kernel"
         self.need_flush = self.dense < 4 * L2_BYTES
         self.l2 = L2_FLUSHED if self.need_flush else "inputs >> L2"
