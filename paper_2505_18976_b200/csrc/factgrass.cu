@@ -380,11 +380,16 @@ static grass_status run_factgrass(const factgrass_layer* layers, int32_t L, gras
         if (forced == 0 || forced == 2 || !cluster_path_fits(hd, L, &cplan)) return;
         const int64_t items = (int64_t)L * B, slots = (int64_t)sms * cplan.per_sm;
         if (items > slots && forced != 1) return;
-        // clusters of 1, 2, 4 or 8 thread blocks: as many as fill the machine, each with at least two 32-token steps;
-        // no accumulator runs over more than 8,192 tokens
-        auto pow2_floor = [](int64_t v) { int64_t p = 1; while (p * 2 <= v) p *= 2; return p; };
-        int64_t nc = pow2_floor(std::max<int64_t>(1, std::min<int64_t>(8, slots / std::max<int64_t>(items, 1))));
-        nc = std::min<int64_t>(nc, pow2_floor(std::max<int64_t>(1, T / (2 * kTokTile))));
+        // Clusters of 8, 4, 2 or 1 thread blocks, as many as are resident at once: a second wave costs more than a larger
+        // cluster saves (128 x 128, 1,000 x 1,000, 16 samples of 700 tokens: 35 us over 8 blocks each, of which 15 clusters
+        // fit, 25 over 4).  Blocks of a short sample that get no tokens still take their part of the projection (32 tokens:
+        // 23 us over one block, 13 over eight).  Two blocks share an SM (64 x 64) only for two 32-token steps or more each
+        // (64 samples of 128 tokens: 18.3 us over four blocks, 17.3 over two).
+        auto fits = [&](int n) {
+            const int64_t one_each = n == 2 ? sms / 2 : cluster_capacity(n);
+            return items <= one_each || (items <= one_each * cplan.per_sm && T >= 2 * kTokTile * n);
+        };
+        int64_t nc = fits(8) ? 8 : fits(4) ? 4 : fits(2) ? 2 : 1;
         int64_t chunk = ((T + nc - 1) / nc + kTokTile - 1) / kTokTile * kTokTile;
         const int64_t forced_chunk = tuning(GRASS_TUNE_FACTGRASS_CHUNK, -1);
         if (forced_chunk > 0) {

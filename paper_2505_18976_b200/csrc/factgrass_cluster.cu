@@ -28,6 +28,7 @@
 #include <cooperative_groups.h>
 
 #include <algorithm>
+#include <atomic>
 
 namespace cg = cooperative_groups;
 
@@ -393,6 +394,8 @@ factgrass_cluster_kernel(const LayerDesc* __restrict__ descs, const __grid_const
     }
 }
 
+constexpr size_t kClusterSmemLimit = 198 * 1024;
+
 static size_t cluster_smem_bytes(int tile, uint32_t max_k)
 {
     const size_t stage = 2 * (size_t)tile * tc::ROW_BYTES;
@@ -414,7 +417,7 @@ bool cluster_path_fits(const LayerDesc* d, int32_t L, ClusterPlan* plan)
     const int tile = max_kk > 64 ? 128 : 64;
     plan->tile_m = plan->tile_n = tile;
     plan->smem = cluster_smem_bytes(tile, max_k);
-    if (plan->smem + 2048 > 200 * 1024) return false;
+    if (plan->smem > kClusterSmemLimit) return false;
     // resident thread blocks per SM: registers, `tile` tensor-memory columns, shared memory; at most 164 KB of
     // the SM go to shared memory, so that the gathered loads in flight keep their L1
     cudaFuncAttributes fa;
@@ -427,13 +430,44 @@ bool cluster_path_fits(const LayerDesc* d, int32_t L, ClusterPlan* plan)
     return per_sm >= 1;
 }
 
+// The SMs of a cluster lie in one part of the chip (a GPC), and these are not all of the same size: 148 SMs hold 15 clusters
+// of 8, not 18.  The runtime knows; a device's answer is kept.
+int cluster_capacity(int nc)
+{
+    constexpr int kDevices = 64;
+    static std::atomic<int> known[kDevices][2];
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kDevices) return 0;
+    std::atomic<int>& cell = known[dev][nc == 8];
+    int n = cell.load(std::memory_order_relaxed);
+    if (n > 0) return n - 1;
+    const auto kern = factgrass_cluster_kernel<128, 128>;
+    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kClusterSmemLimit) != cudaSuccess) return 0;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)nc, 1024, 1);
+    cfg.blockDim = dim3(kFgThreads, 1, 1);
+    cfg.dynamicSmemBytes = 120 * 1024;                 // one thread block per SM
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = (unsigned)nc;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    int count = 0;
+    if (cudaOccupancyMaxActiveClusters(&count, kern, &cfg) != cudaSuccess) count = 0;
+    cell.store(count + 1, std::memory_order_relaxed);
+    return count;
+}
+
 grass_status launch_factgrass_cluster(const LayerDesc* dev_descs, const LayerDesc& single, const ClusterPlan& plan,
                                       int32_t L, int32_t B, int32_t T, const int64_t* tok_begin,
                                       const int32_t* tok_count, int32_t nc, int32_t chunk_len, float* out,
                                       int64_t ld_out, uint32_t* dev_status, cudaStream_t st, int out_bf16)
 {
     auto launch = [&](auto kern) -> grass_status {
-        if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)plan.smem) != cudaSuccess)
+        // the same limit in every call: another thread may be between this and its launch
+        if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kClusterSmemLimit) != cudaSuccess)
             return GRASS_ERR_CUDA;
         int carve = 100;
         {

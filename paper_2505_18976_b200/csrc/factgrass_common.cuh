@@ -52,6 +52,8 @@ struct ClusterPlan {
     size_t smem;          // dynamic shared memory per thread block
 };
 bool cluster_path_fits(const LayerDesc* host_descs, int32_t L, ClusterPlan* plan);
+// clusters of nc thread blocks that the current device can hold with one thread block per SM
+int cluster_capacity(int nc);
 grass_status launch_factgrass_cluster(const LayerDesc* dev_descs, const LayerDesc& single, const ClusterPlan& plan,
                                       int32_t L, int32_t B, int32_t T, const int64_t* tok_begin,
                                       const int32_t* tok_count, int32_t nc, int32_t chunk_len, float* out,

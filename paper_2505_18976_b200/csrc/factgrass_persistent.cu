@@ -519,7 +519,8 @@ grass_status launch_persistent(const LayerDesc* dev_descs, const LayerDesc& sing
     if (launch_status() != GRASS_OK) return GRASS_ERR_CUDA;
     auto launch = [&](auto kern, int pieces) -> grass_status {
         const size_t smem = (size_t)NBUF * 2 * pieces * TILE * tc::ROW_BYTES + (size_t)max_k * 4;
-        if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) return GRASS_ERR_CUDA;
+        // the same limit in every call (96 KB of tiles and the longest bins): another thread may be between this and its launch
+        if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024 + (int)MAX_K * 4) != cudaSuccess) return GRASS_ERR_CUDA;
         // what shared memory does not need is L1, where gathered loads wait
         int carve = 100;
         for (int kb : {64, 100, 132, 164, 196, 228})
