@@ -388,7 +388,8 @@ static CompressPlan plan_compress(int64_t n, int64_t kprime, uint32_t k, int sm_
     // Split of the positions over a cluster of up to 8 thread blocks.  A block's share has to be worth its k bins (zeroed,
     // exchanged and stored): at least k positions, or k / 2 while there are fewer blocks than SMs, and at least 1,024
     // (one row of k' = 8,192, k = 2,048: 8.2 us over 4 blocks, 6.2 us over 8; 512 rows of k' = 65,536: 345 us
-    // over 2 blocks, 332 us over 8).  Streamed rows keep one full round of loads per block.
+    // over 2 blocks, 332 us over 8), and a full round of loads once the blocks fill the machine (318 rows of k' = 10,510,
+    // k = 1,000 in bf16: 47 us over 8 blocks, 36 over 2).  Streamed rows keep one full round of loads per block.
     const int64_t round = (int64_t)pl.threads * U;
     int64_t js = 1;
     if (dense) {
@@ -398,6 +399,7 @@ static CompressPlan plan_compress(int64_t n, int64_t kprime, uint32_t k, int sm_
         while (js < 8) {
             const int64_t share = kprime / (js * 2);
             if (share < 1024 || share < (int64_t)(groups * js < sm_count ? k / 2 : k)) break;
+            if (groups * js >= 4 * sm_count && share < round) break;
             js *= 2;
         }
     }
