@@ -389,7 +389,8 @@ static CompressPlan plan_compress(int64_t n, int64_t kprime, uint32_t k, int sm_
     // exchanged and stored): at least k positions, or k / 2 while there are fewer blocks than SMs, and at least 1,024
     // (one row of k' = 8,192, k = 2,048: 8.2 us over 4 blocks, 6.2 us over 8; 512 rows of k' = 65,536: 345 us
     // over 2 blocks, 332 us over 8), and a full round of loads once the blocks fill the machine (318 rows of k' = 10,510,
-    // k = 1,000 in bf16: 47 us over 8 blocks, 36 over 2).  Streamed rows keep one full round of loads per block.
+    // k = 1,000 in bf16: 47 us over 8 blocks, 36 over 2), half of one where the next split would (100 rows of
+    // k' = 9,000, k = 700: 18.4 over 8, 16.6 over 4).  Streamed rows keep one full round of loads per block.
     const int64_t round = (int64_t)pl.threads * U;
     int64_t js = 1;
     if (dense) {
@@ -399,7 +400,7 @@ static CompressPlan plan_compress(int64_t n, int64_t kprime, uint32_t k, int sm_
         while (js < 8) {
             const int64_t share = kprime / (js * 2);
             if (share < 1024 || share < (int64_t)(groups * js < sm_count ? k / 2 : k)) break;
-            if (groups * js >= 4 * sm_count && share < round) break;
+            if (share < round && (groups * js >= 4 * sm_count || (groups * js * 2 > 4 * sm_count && share < round / 2))) break;
             js *= 2;
         }
     }
