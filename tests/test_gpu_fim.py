@@ -123,6 +123,46 @@ def test_factor_and_apply_shapes(G, k, M, pad):
     assert (x @ A - b).norm() <= u * A.norm() * x.norm()
 
 
+# Pivots at both ends of the fp32 range: below 2^-126 they are subnormal, above 2^126 their reciprocals are
+@pytest.mark.parametrize("scale", [1.0e-38, 1.0, 1.2e38])
+def test_factor_of_scaled_matrices(G, scale):
+    k = 200
+    X = _compressed(4 * k, k, 5)
+    C = torch.corrcoef(X.double().T)
+    A = ((0.3 * C + 0.7 * torch.eye(k, device="cuda", dtype=torch.float64)) * scale).float()
+    st = torch.zeros(1, dtype=torch.int32, device="cuda")
+    L = torch.tril(G.grass_fim_factor(A.clone(), 0.0, dev_status=st)).double() / scale ** 0.5
+    assert int(st.item()) == 0
+    # the bound of test_factor_and_apply_shapes for one pass; a subnormal matrix is updated in steps of 2^-149, one update
+    # for every 8 columns
+    A = A.double() / scale
+    assert (L @ L.T - A).norm() <= 2.0 * k ** 0.5 * 2.0 ** -24 * A.norm() + (k / 8) * k * 2.0 ** -149 / scale
+
+
+# The roots and reciprocals of the pivots themselves, as the factors of 2 x 2 blocks [d x; x y] show them: sqrt(d), x / sqrt(d) and
+# sqrt(y - x^2 / d), here with x = d and y = 2 d, over all of fp32 that leaves room for them.
+def test_roots_and_reciprocals_of_pivots(G):
+    k = 4096
+    gen = torch.Generator(device="cuda").manual_seed(3)
+    d = torch.exp2(torch.rand(k // 2, generator=gen, device="cuda") * 251.0 - 125.0)
+    at = torch.arange(0, k, 2, device="cuda")
+    A = torch.zeros((k, k), device="cuda")
+    A[at, at], A[at + 1, at], A[at, at + 1], A[at + 1, at + 1] = d, d, d, 2 * d
+    L = G.grass_fim_factor(A, 0.0).double()
+    u, root = 2.0 ** -24, d.double().sqrt()
+    # against CUDA's square root, which is correctly rounded: an ulp and a half
+    assert ((L[at, at] - torch.sqrt(d).double()).abs() <= 3.0 * u * root).all()
+    # x times the reciprocal root: its error and one rounding
+    assert ((L[at + 1, at] - root).abs() <= 4.0 * u * root).all()
+    # the second pivot is 2 d - d (d / d): a reciprocal one ulp off (2 u) and two roundings, half of it after the root
+    assert ((L[at + 1, at + 1] - root).abs() <= (3.0 + 2.0) * u * root).all()
+    # subnormal pivots have roots like any other
+    s = torch.rand(4096, generator=gen, device="cuda") * 2.0 ** -126 + 2.0 ** -127
+    A = torch.diag(s)
+    L = torch.diagonal(G.grass_fim_factor(A, 0.0)).double()
+    assert ((L - s.double().sqrt()).abs() <= 3.0 * u * s.double().sqrt()).all()
+
+
 # one sample, fewer samples than a step, a chunk boundary at 8,192; tiles on the diagonal alone, a ragged second tile, many
 # tiles (pairs instead of clusters of eight); columns that start off a 16-byte boundary
 @pytest.mark.parametrize("n,k,off", [(1, 128, 0), (31, 129, 0), (33, 127, 1), (8_192, 64, 0), (8_200, 200, 3), (700, 900, 0)])
