@@ -77,6 +77,17 @@ def test_not_positive_definite_is_flagged(G):
     assert int(st.item()) == G.binding.DEV_NOT_PD
 
 
+def test_pivots_that_are_not_positive_count_as_one(G):
+    F = torch.zeros(140, 140, device="cuda")
+    F[3, 3], F[70, 70], F[80, 80] = -1.0, 4.0, 9.0
+    st = torch.zeros(1, dtype=torch.int32, device="cuda")
+    G.grass_fim_factor(F, 0.0, dev_status=st)
+    want = torch.ones(140, device="cuda")
+    want[70], want[80] = 2.0, 3.0
+    assert int(st.item()) == G.binding.DEV_NOT_PD
+    assert torch.equal(torch.tril(F), torch.diag(want))
+
+
 def test_preconditioned_score(G, oracle_mod):
     """scores[i, m] = <g_i, (F + lam I)^-1 g_test,m> through grass_fim -> factor -> apply -> grass_score."""
     n, k, M, lam = 1500, 192, 40, 5e-2
