@@ -239,15 +239,13 @@ factgrass_kernel(const LayerDesc* __restrict__ descs, const __grid_constant__ La
             // 16 rows x 32 columns per warp, 16 values per thread
             const int c0 = (warp >> 2) * 32;
             uint32_t v[16];
-            tc::tmem_ld_16x256b_x4(tq + (uint32_t)c0, v);
             if constexpr (F32) {
                 uint32_t w[16];
-                tc::tmem_ld_16x256b_x4(tq + (uint32_t)(TN + c0), w);
-                asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+                tc::tmem_ld_16x256b_x4_pair_wait(tq + (uint32_t)c0, v, tq + (uint32_t)(TN + c0), w);
 #pragma unroll
                 for (int e = 0; e < 16; ++e) v[e] = __float_as_uint(__uint_as_float(v[e]) + __uint_as_float(w[e]));
             } else {
-                asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+                tc::tmem_ld_16x256b_x4_wait(tq + (uint32_t)c0, v);
             }
 #pragma unroll
             for (int e = 0; e < 16; ++e) {
@@ -260,15 +258,13 @@ factgrass_kernel(const LayerDesc* __restrict__ descs, const __grid_constant__ La
 #pragma unroll 1
             for (int c0 = (warp >> 2) * 32; c0 < TN; c0 += 64) {
                 uint32_t v[32];
-                tc::tmem_ld32(tq + (uint32_t)c0, v);
                 if constexpr (F32) {
                     uint32_t w[32];
-                    tc::tmem_ld32(tq + (uint32_t)(TN + c0), w);
-                    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+                    tc::tmem_ld32_pair_wait(tq + (uint32_t)c0, v, tq + (uint32_t)(TN + c0), w);
 #pragma unroll
                     for (int e = 0; e < 32; ++e) v[e] = __float_as_uint(__uint_as_float(v[e]) + __uint_as_float(w[e]));
                 } else {
-                    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+                    tc::tmem_ld32_wait(tq + (uint32_t)c0, v);
                 }
 #pragma unroll
                 for (int e = 0; e < 32; ++e) project(a, tn * TN + c0 + e, __uint_as_float(v[e]));

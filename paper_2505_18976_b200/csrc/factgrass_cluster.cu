@@ -297,8 +297,7 @@ factgrass_cluster_kernel(const LayerDesc* __restrict__ descs, const __grid_const
             const int c0 = (warp >> 2) * 32;
             uint32_t v[16];
             if (have) {
-                tc::tmem_ld_16x256b_x4(tq + (uint32_t)c0, v);
-                asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+                tc::tmem_ld_16x256b_x4_wait(tq + (uint32_t)c0, v);
             } else {
 #pragma unroll
                 for (int e = 0; e < 16; ++e) v[e] = 0u;
@@ -316,8 +315,7 @@ factgrass_cluster_kernel(const LayerDesc* __restrict__ descs, const __grid_const
             for (int c0 = (warp >> 2) * 32; c0 < TN; c0 += 64) {
                 uint32_t v[32];
                 if (have) {
-                    tc::tmem_ld32(tq + (uint32_t)c0, v);
-                    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+                    tc::tmem_ld32_wait(tq + (uint32_t)c0, v);
                 } else {
 #pragma unroll
                     for (int e = 0; e < 32; ++e) v[e] = 0u;

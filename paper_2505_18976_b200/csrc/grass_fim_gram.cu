@@ -191,9 +191,7 @@ gram_kernel(const float* __restrict__ X, int32_t n, int32_t k, int64_t ld, int32
         for (int c0 = (warp >> 2) * 32; c0 < TILE; c0 += 64) {
             uint32_t v[32], w[32];
             if (work && ok) {
-                tc::tmem_ld32(tq + (uint32_t)c0, v);
-                tc::tmem_ld32(tq + (uint32_t)(TILE + c0), w);
-                asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+                tc::tmem_ld32_pair_wait(tq + (uint32_t)c0, v, tq + (uint32_t)(TILE + c0), w);
             } else {
 #pragma unroll
                 for (int e = 0; e < 32; ++e) { v[e] = ok ? 0u : 0x7FC00000u; w[e] = 0u; }

@@ -138,8 +138,7 @@ score_bf16_kernel(const __grid_constant__ CUtensorMap map_train, const __grid_co
                 if (ok) {
                     // columns of the second accumulator start at tensor-memory column 256
                     const int sub = c0 >= n_sub ? 1 : 0;
-                    tmem_ld32(tmem_d + ((uint32_t)(warp * 32) << 16) + (uint32_t)(b * 256 + sub * 256 + c0 - sub * n_sub), v);
-                    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+                    tmem_ld32_wait(tmem_d + ((uint32_t)(warp * 32) << 16) + (uint32_t)(b * 256 + sub * 256 + c0 - sub * n_sub), v);
                 } else {
 #pragma unroll
                     for (int e = 0; e < 32; ++e) v[e] = 0x7FC00000u;        // NaN marks an aborted tile

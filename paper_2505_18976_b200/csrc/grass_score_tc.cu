@@ -207,9 +207,8 @@ grass_score_tc_kernel(const __grid_constant__ CUtensorMap map_train, const __gri
                 uint32_t v[32];
                 if (ok) {
                     uint32_t w[32];
-                    tmem_ld32(tmem_d + ((uint32_t)(lane_grp * 32) << 16) + (uint32_t)c0, v);
-                    tmem_ld32(tmem_d + ((uint32_t)(lane_grp * 32) << 16) + (uint32_t)(BN + c0), w);
-                    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+                    const uint32_t acc0 = tmem_d + ((uint32_t)(lane_grp * 32) << 16) + (uint32_t)c0;
+                    tmem_ld32_pair_wait(acc0, v, acc0 + BN, w);
 #pragma unroll
                     for (int e = 0; e < 32; ++e) v[e] = __float_as_uint(__uint_as_float(v[e]) + __uint_as_float(w[e]));
                 } else {
