@@ -56,7 +56,7 @@ factgrass_kernel(const LayerDesc* __restrict__ descs, const __grid_constant__ La
     float* bins = reinterpret_cast<float*>(smem + NBUF * STAGE);
 
     const LayerDesc& L = descs ? descs[blockIdx.z] : single;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int tid = threadIdx.x, lane = tid & 31, warp = __shfl_sync(0xFFFFFFFFu, tid >> 5, 0);
     const int b = blockIdx.y;
     // block tiles of one token chunk are neighbours in launch order: the rows they share are read from
     // HBM once and from L2 by the others
@@ -167,7 +167,7 @@ factgrass_kernel(const LayerDesc* __restrict__ descs, const __grid_constant__ La
         for (int ps = 0; ps < PASS_G; ++ps) put(sg, G_TILE, gL, ps * GG + grpG, rg[ps]);
     };
 
-    const uint32_t smem_base = tc::smem_u32(smem);
+    const uint64_t desc0 = tc::make_smem_desc(tc::smem_u32(smem));      // addresses below are 16-byte units added to it
     const uint32_t idesc = tc::make_idesc(TM, TN);
     bool ok = true;
     prefetch(t_begin);
@@ -180,28 +180,30 @@ factgrass_kernel(const LayerDesc* __restrict__ descs, const __grid_constant__ La
         if (t0 + kTokTile < t_end) prefetch(t0 + kTokTile);
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         __syncthreads();
-        if (tid == 0) {
+        if (warp == 0) {
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            const uint32_t a0 = smem_base + buf * STAGE, g0 = a0 + NP * A_TILE;
+            if (tc::elect_one()) {
+                const uint64_t a0 = desc0 + (uint32_t)(buf * (STAGE >> 4)), g0 = a0 + (NP * A_TILE >> 4);
 #pragma unroll
-            for (int ks = 0; ks < kTokTile / 16; ++ks) {
-                if constexpr (F32) {
-                    // hi*hi goes to the first accumulator, the correction terms to the second (the tensor core
-                    // truncates after every accumulation, so the large sum sees as few of them as possible)
+                for (int ks = 0; ks < kTokTile / 16; ++ks) {
+                    if constexpr (F32) {
+                        // hi*hi goes to the first accumulator, the correction terms to the second (the tensor core
+                        // truncates after every accumulation, so the large sum sees as few of them as possible)
 #pragma unroll
-                    for (int q = 0; q < 6; ++q) {
-                        if (q >= nprod) break;
-                        const uint64_t ad = tc::make_smem_desc(a0 + tc::split_piece_a(q) * A_TILE + ks * 32);
-                        const uint64_t gd = tc::make_smem_desc(g0 + tc::split_piece_b(q) * G_TILE + ks * 32);
-                        tc::umma_bf16(q == 0 ? tmem_d : tmem_d + TN, ad, gd, idesc, (it > 0 || ks > 0 || q > 1) ? 1u : 0u);
+                        for (int q = 0; q < 6; ++q) {
+                            if (q >= nprod) break;
+                            tc::umma_bf16(q == 0 ? tmem_d : tmem_d + TN, a0 + ((tc::split_piece_a(q) * A_TILE + ks * 32) >> 4),
+                                          g0 + ((tc::split_piece_b(q) * G_TILE + ks * 32) >> 4), idesc,
+                                          (it > 0 || ks > 0 || q > 1) ? 1u : 0u);
+                        }
+                    } else {
+                        tc::umma_bf16(tmem_d, a0 + (ks * 32 >> 4), g0 + (ks * 32 >> 4), idesc, (it > 0 || ks > 0) ? 1u : 0u);
                     }
-                } else {
-                    tc::umma_bf16(tmem_d, tc::make_smem_desc(a0 + ks * 32), tc::make_smem_desc(g0 + ks * 32), idesc,
-                                  (it > 0 || ks > 0) ? 1u : 0u);
                 }
+                tc::umma_commit(bar0 + 8 * buf);                       // buffer free once these MMAs have read it
+                if (t0 + kTokTile >= t_end) tc::umma_commit(bar_done); // accumulator complete
             }
-            tc::umma_commit(bar0 + 8 * buf);                       // buffer free once these MMAs have read it
-            if (t0 + kTokTile >= t_end) tc::umma_commit(bar_done); // accumulator complete
+            __syncwarp();
         }
     }
     if (bad && dev_status) atomicOr(dev_status, GRASS_DEV_BAD_INDEX);

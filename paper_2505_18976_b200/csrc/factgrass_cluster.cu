@@ -133,7 +133,7 @@ factgrass_cluster_kernel(const LayerDesc* __restrict__ descs, const __grid_const
 
     cg::cluster_group cluster = cg::this_cluster();
     const uint32_t nc = cluster.num_blocks(), rank = cluster.block_rank();
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int tid = threadIdx.x, lane = tid & 31, warp = __shfl_sync(0xFFFFFFFFu, tid >> 5, 0);
     const bool nc_ok = nc == 1 || nc == 2 || nc == 4 || nc == 8;    // the launcher forms no other clusters
     const int rows = TM / (int)(nc_ok ? nc : 1);
     const uint32_t slice_bytes = (uint32_t)(rows * TN * 4), bar_recv = tc::smem_u32(&recv_bar);
@@ -233,7 +233,7 @@ factgrass_cluster_kernel(const LayerDesc* __restrict__ descs, const __grid_const
         };
 
         // stage 2: C += A'^T G' over this block's tokens, 32 per step
-        const uint32_t smem_base = tc::smem_u32(smem);
+        const uint64_t desc0 = tc::make_smem_desc(tc::smem_u32(smem));  // addresses below are 16-byte units added to it
         const uint32_t idesc = tc::make_idesc(TM, TN);
         auto step = [&](uint32_t (&ra)[PASS_A][8], uint32_t (&rg)[PASS_G][8], int t0, int it) {
             const int buf = it % NBUF;
@@ -243,15 +243,17 @@ factgrass_cluster_kernel(const LayerDesc* __restrict__ descs, const __grid_const
             if (t0 + 2 * kTokTile < t_end) prefetch(ra, rg, t0 + 2 * kTokTile);
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
             __syncthreads();
-            if (tid == 0) {
+            if (warp == 0) {
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                const uint32_t a0 = smem_base + buf * STAGE, g0 = a0 + A_TILE;
+                if (tc::elect_one()) {
+                    const uint64_t a0 = desc0 + (uint32_t)(buf * (STAGE >> 4)), g0 = a0 + (A_TILE >> 4);
 #pragma unroll
-                for (int ks = 0; ks < kTokTile / 16; ++ks)
-                    tc::umma_bf16(tmem_d, tc::make_smem_desc(a0 + ks * 32), tc::make_smem_desc(g0 + ks * 32), idesc,
-                                  (it > 0 || ks > 0) ? 1u : 0u);
-                tc::umma_commit(bar0 + 8 * buf);                       // buffer free once these MMAs have read it
-                if (t0 + kTokTile >= t_end) tc::umma_commit(bar_done); // accumulator complete
+                    for (int ks = 0; ks < kTokTile / 16; ++ks)
+                        tc::umma_bf16(tmem_d, a0 + (ks * 32 >> 4), g0 + (ks * 32 >> 4), idesc, (it > 0 || ks > 0) ? 1u : 0u);
+                    tc::umma_commit(bar0 + 8 * buf);                       // buffer free once these MMAs have read it
+                    if (t0 + kTokTile >= t_end) tc::umma_commit(bar_done); // accumulator complete
+                }
+                __syncwarp();
             }
         };
         prefetch(ra0, rg0, t_begin);

@@ -75,7 +75,7 @@ gram_kernel(const float* __restrict__ X, int32_t n, int32_t k, int64_t ld, int32
 
     cg::cluster_group cluster = cg::this_cluster();
     const int cs = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int tid = threadIdx.x, lane = tid & 31, warp = __shfl_sync(0xFFFFFFFFu, tid >> 5, 0);
     // blockIdx.x = (tile on or above the diagonal, row by row) * nchunks + sample chunk
     const int chunk = (int)(blockIdx.x % (unsigned)nchunks);
     int tm = 0, rest = (int)(blockIdx.x / (unsigned)nchunks);
@@ -135,7 +135,7 @@ gram_kernel(const float* __restrict__ X, int32_t n, int32_t k, int64_t ld, int32
         *reinterpret_cast<uint4*>(strip + 2 * PIECE + off) = lo;
     };
 
-    const uint32_t smem_base = tc::smem_u32(smem);
+    const uint64_t desc0 = make_desc(tc::smem_u32(smem));      // addresses below are 16-byte units added to it
     // as make_idesc, both operands MN-major
     const uint32_t idesc = tc::make_idesc(TILE, TILE) | (1u << 15) | (1u << 16);
     bool ok = true;
@@ -154,20 +154,23 @@ gram_kernel(const float* __restrict__ X, int32_t n, int32_t k, int64_t ld, int32
         if (t0 + STEP < t_end) prefetch(t0 + STEP);
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         __syncthreads();
-        if (tid == 0) {
+        if (warp == 0) {
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            const uint32_t a0 = smem_base + buf * STAGE, g0 = diag ? a0 : a0 + STRIP;
+            if (tc::elect_one()) {
+                const uint64_t a0 = desc0 + (uint32_t)(buf * (STAGE >> 4)), g0 = diag ? a0 : a0 + (STRIP >> 4);
 #pragma unroll
-            for (int ks = 0; ks < STEP / 16; ++ks)
+                for (int ks = 0; ks < STEP / 16; ++ks)
 #pragma unroll
-                for (int q = 0; q < 6; ++q) {
-                    if (q >= nprod) break;
-                    tc::umma_bf16(q == 0 ? tmem_d : tmem_d + TILE, make_desc(a0 + tc::split_piece_a(q) * PIECE + ks * 2 * SBO),
-                                  make_desc(g0 + tc::split_piece_b(q) * PIECE + ks * 2 * SBO), idesc,
-                                  (it > 0 || ks > 0 || q > 1) ? 1u : 0u);
-                }
-            tc::umma_commit(bar0 + 8 * buf);
-            if (t0 + STEP >= t_end) tc::umma_commit(bar_done);
+                    for (int q = 0; q < 6; ++q) {
+                        if (q >= nprod) break;
+                        tc::umma_bf16(q == 0 ? tmem_d : tmem_d + TILE, a0 + ((tc::split_piece_a(q) * PIECE + ks * 2 * (int)SBO) >> 4),
+                                      g0 + ((tc::split_piece_b(q) * PIECE + ks * 2 * (int)SBO) >> 4), idesc,
+                                      (it > 0 || ks > 0 || q > 1) ? 1u : 0u);
+                    }
+                tc::umma_commit(bar0 + 8 * buf);
+                if (t0 + STEP >= t_end) tc::umma_commit(bar_done);
+            }
+            __syncwarp();
         }
     }
     const bool work = it > 0;
