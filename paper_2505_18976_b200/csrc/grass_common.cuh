@@ -104,6 +104,9 @@ size_t sjlt_table_bytes(int64_t n, int64_t p, uint32_t k, uint32_t s, size_t ele
 grass_status launch_sjlt_table(const void* g, grass_dtype dt, int64_t n, int64_t p, int64_t ld, const grass_sjlt_spec& sp, float* out,
                                int64_t ld_out, void* table, uint32_t* dev_status, cudaStream_t st, int out_bf16);
 
+// dynamic shared memory that a thread block may have: 227 KB less 1 KB for what a kernel declares statically
+constexpr size_t kDynSmemLimit = 226 * 1024;
+
 // launch-shape override set through grass_set_tuning, or `dflt` while the key is on automatic
 int64_t tuning(grass_tuning_key key, int64_t dflt);
 

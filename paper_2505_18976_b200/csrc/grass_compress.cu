@@ -490,11 +490,13 @@ static grass_status dispatch_compress(const T* g, int64_t n, int64_t p, int64_t 
                        (uintptr_t)g % (4 * sizeof(T)) == 0 && ld % 4 == 0;
     CompressPlan pl = plan_compress(n, kprime, sp.k, sms, dense);
     pl.out_bf16 = out_bf16;
-    // whole-row thread blocks, one for every SM or more: the index list (up to 48 KB) goes into shared memory
+    // whole-row thread blocks, one for every SM or more: the index list (up to 48 KB) goes into shared memory, where the bins
+    // leave room for it
     pl.idx_smem = 0;
+    const size_t list = ((size_t)kprime * 4 + 15) / 16 * 16, bins = ((size_t)sp.k * sizeof(float) + 15) / 16 * 16;
     if (!dense && idx && pl.jsplit == 1 && pl.S == 1 && pl.use_smem && n >= sms && kprime * 4 <= 48 * 1024 &&
-        (uintptr_t)idx % 16 == 0 && tuning(GRASS_TUNE_COMPRESS_IDX_SMEM, 1) != 0)
-        pl.idx_smem = (uint32_t)((kprime * 4 + 15) / 16 * 16);
+        bins + list <= kDynSmemLimit && (uintptr_t)idx % 16 == 0 && tuning(GRASS_TUNE_COMPRESS_IDX_SMEM, 1) != 0)
+        pl.idx_smem = (uint32_t)list;
     if (out_bf16 && !pl.cluster && (pl.jsplit > 1 || !pl.use_smem)) {
         // a bf16 row is rounded once, at the final store, so it needs a launch shape in which one thread block
         // or one cluster owns the row: no partial sums in global memory

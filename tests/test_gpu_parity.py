@@ -159,6 +159,11 @@ def test_grass_compress_bf16_input(G, W, oracle_mod):
     _grass_case(G, W, oracle_mod, 12, 100_000, 10_000, 1_024, dtype=torch.bfloat16)
 
 
+@pytest.mark.parametrize("n,p,kprime,k", [(200, 20_000, 12_000, 50_000), (160, 9_000, 8_192, 51_200), (149, 13_000, 12_288, 45_000)])
+def test_grass_compress_bins_that_leave_no_room_for_the_index_list(G, W, oracle_mod, n, p, kprime, k):
+    _grass_case(G, W, oracle_mod, n, p, kprime, k)
+
+
 def test_grass_compress_student_t(G, W, oracle_mod):
     _grass_case(G, W, oracle_mod, 8, 1 << 18, 1 << 14, 4_096, zero_prob=0.7, dist="student_t3", scale=1e-2)
 
