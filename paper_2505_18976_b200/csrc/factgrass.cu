@@ -368,8 +368,8 @@ static grass_status run_factgrass(const factgrass_layer* layers, int32_t L, gras
         if (rc != GRASS_OK) return rc;
     }
     int dev = 0, sms = 148;
-    if (cudaGetDevice(&dev) != cudaSuccess) return GRASS_ERR_CUDA;
-    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return GRASS_ERR_CUDA;
+    if (cuda_failed(cudaGetDevice(&dev))) return GRASS_ERR_CUDA;
+    if (cuda_failed(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev))) return GRASS_ERR_CUDA;
     const bool f32 = dt == GRASS_F32;
 
     // Launches of about one wave (few layers x samples, bf16 factors, blocks of one tile) take the cluster kernel:
@@ -478,10 +478,10 @@ static grass_status run_factgrass(const factgrass_layer* layers, int32_t L, gras
     auto launch = [&](auto kern, size_t stage_bytes) -> grass_status {
         const size_t smem = kFgBufs * stage_bytes + bins_bytes;
         // static shared memory counts toward the 48 KB default limit too
-        if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
+        if (cuda_failed(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)))
             return GRASS_ERR_CUDA;
         cudaFuncAttributes fa;
-        if (cudaFuncGetAttributes(&fa, kern) != cudaSuccess) return GRASS_ERR_CUDA;
+        if (cuda_failed(cudaFuncGetAttributes(&fa, kern))) return GRASS_ERR_CUDA;
         const size_t cta_smem = smem + fa.sharedSizeBytes + 1024;   // + the per-CTA reservation
         // resident CTAs per SM from the kernel's own footprint: registers, threads, tensor-memory columns
         // (which the runtime's occupancy query does not count) and shared memory
@@ -508,7 +508,7 @@ static grass_status run_factgrass(const factgrass_layer* layers, int32_t L, gras
                 if ((size_t)kb * 1024 >= (size_t)per_sm * cta_smem) { carve = kb * 100 / 228; break; }
         }
         carve = (int)tuning(GRASS_TUNE_FACTGRASS_CARVEOUT, carve);
-        if (cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, carve) != cudaSuccess)
+        if (cuda_failed(cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, carve)))
             return GRASS_ERR_CUDA;
         // token chunks.  Every chunk pays a fixed projection epilogue (tile*tile hashes and a k-bin flush),
         // so chunks are as long as the machine allows: when there are fewer work items than resident CTA
@@ -547,7 +547,7 @@ static grass_status run_factgrass(const factgrass_layer* layers, int32_t L, gras
         cfg.numAttrs = 1;
         const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, (const LayerDesc*)dev_descs, single, B, T, tok_begin, tok_count,
                                                  (int32_t)max_tiles, (int32_t)chunk_len, out, ld_out, dev_status, nprod, out_bf16 ? 2 : 0);
-        return e == cudaSuccess ? launch_status() : GRASS_ERR_CUDA;
+        return cuda_ok(e);
     };
     const size_t piece = (size_t)tile * tc::ROW_BYTES * 2;   // one bf16 piece of the A tile plus one of the G tile
     if (epi == kEpiBlock) {
@@ -716,12 +716,12 @@ static void* g_static_table_addr[kMaxDevices] = {nullptr};
 static grass_status static_table_address(void** addr)
 {
     int dev = -1;
-    if (cudaGetDevice(&dev) != cudaSuccess) return GRASS_ERR_CUDA;
+    if (cuda_failed(cudaGetDevice(&dev))) return GRASS_ERR_CUDA;
     if (dev < 0 || dev >= kMaxDevices) return GRASS_ERR_UNSUPPORTED;
     std::lock_guard<std::mutex> lock(g_static_mutex);
     if (!g_static_table_addr[dev]) {
         void* p = nullptr;
-        if (cudaGetSymbolAddress(&p, g_static_layer_table) != cudaSuccess || !p) return GRASS_ERR_CUDA;
+        if (cuda_failed(cudaGetSymbolAddress(&p, g_static_layer_table)) || !p) return GRASS_ERR_CUDA;
         g_static_table_addr[dev] = p;
     }
     *addr = g_static_table_addr[dev];

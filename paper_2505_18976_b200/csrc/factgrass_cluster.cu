@@ -423,7 +423,7 @@ bool cluster_path_fits(const LayerDesc* d, int32_t L, ClusterPlan* plan)
     cudaFuncAttributes fa;
     const cudaError_t e = tile == 64 ? cudaFuncGetAttributes(&fa, factgrass_cluster_kernel<64, 64>)
                                      : cudaFuncGetAttributes(&fa, factgrass_cluster_kernel<128, 128>);
-    if (e != cudaSuccess || fa.numRegs <= 0) return false;
+    if (cuda_failed(e) || fa.numRegs <= 0) return false;
     int per_sm = std::min(65536 / (fa.numRegs * kFgThreads), 512 / tile);
     per_sm = std::min<int>(per_sm, (int)((164 * 1024) / (plan->smem + 1024 + 64)));
     plan->per_sm = per_sm;
@@ -437,12 +437,12 @@ int cluster_capacity(int nc)
     constexpr int kDevices = 64;
     static std::atomic<int> known[kDevices][2];
     int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kDevices) return 0;
+    if (cuda_failed(cudaGetDevice(&dev)) || dev < 0 || dev >= kDevices) return 0;
     std::atomic<int>& cell = known[dev][nc == 8];
     int n = cell.load(std::memory_order_relaxed);
     if (n > 0) return n - 1;
     const auto kern = factgrass_cluster_kernel<128, 128>;
-    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kClusterSmemLimit) != cudaSuccess) return 0;
+    if (cuda_failed(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kClusterSmemLimit))) return 0;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)nc, 1024, 1);
     cfg.blockDim = dim3(kFgThreads, 1, 1);
@@ -455,7 +455,7 @@ int cluster_capacity(int nc)
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     int count = 0;
-    if (cudaOccupancyMaxActiveClusters(&count, kern, &cfg) != cudaSuccess) count = 0;
+    if (cuda_failed(cudaOccupancyMaxActiveClusters(&count, kern, &cfg))) count = 0;
     cell.store(count + 1, std::memory_order_relaxed);
     return count;
 }
@@ -467,7 +467,7 @@ grass_status launch_factgrass_cluster(const LayerDesc* dev_descs, const LayerDes
 {
     auto launch = [&](auto kern) -> grass_status {
         // the same limit in every call: another thread may be between this and its launch
-        if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kClusterSmemLimit) != cudaSuccess)
+        if (cuda_failed(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kClusterSmemLimit)))
             return GRASS_ERR_CUDA;
         int carve = 100;
         {
@@ -477,7 +477,7 @@ grass_status launch_factgrass_cluster(const LayerDesc* dev_descs, const LayerDes
                 if ((size_t)kb * 1024 >= need) { carve = (kb * 100 + 227) / 228; break; }
         }
         carve = (int)tuning(GRASS_TUNE_FACTGRASS_CARVEOUT, carve);
-        if (cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, carve) != cudaSuccess)
+        if (cuda_failed(cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, carve)))
             return GRASS_ERR_CUDA;
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3((unsigned)nc, (unsigned)B, (unsigned)L);
@@ -493,7 +493,7 @@ grass_status launch_factgrass_cluster(const LayerDesc* dev_descs, const LayerDes
         cfg.numAttrs = 1;
         cudaError_t e = cudaLaunchKernelEx(&cfg, kern, dev_descs, single, T, tok_begin, tok_count, chunk_len, out,
                                            ld_out, dev_status, out_bf16);
-        return e == cudaSuccess ? launch_status() : GRASS_ERR_CUDA;
+        return cuda_ok(e);
     };
     if (plan.tile_m == 64) return launch(factgrass_cluster_kernel<64, 64>);
     return launch(factgrass_cluster_kernel<128, 128>);

@@ -520,13 +520,13 @@ grass_status launch_persistent(const LayerDesc* dev_descs, const LayerDesc& sing
     auto launch = [&](auto kern, int pieces) -> grass_status {
         const size_t smem = (size_t)NBUF * 2 * pieces * TILE * tc::ROW_BYTES + (size_t)max_k * 4;
         // the same limit in every call (96 KB of tiles and the longest bins): another thread may be between this and its launch
-        if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024 + (int)MAX_K * 4) != cudaSuccess) return GRASS_ERR_CUDA;
+        if (cuda_failed(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024 + (int)MAX_K * 4))) return GRASS_ERR_CUDA;
         // what shared memory does not need is L1, where gathered loads wait
         int carve = 100;
         for (int kb : {64, 100, 132, 164, 196, 228})
             if ((size_t)kb * 1024 >= smem + 7 * 1024) { carve = (kb * 100 + 227) / 228; break; }
         carve = (int)tuning(GRASS_TUNE_FACTGRASS_CARVEOUT, carve);
-        if (cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, carve) != cudaSuccess) return GRASS_ERR_CUDA;
+        if (cuda_failed(cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, carve))) return GRASS_ERR_CUDA;
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3((unsigned)blocks, 1, 1);
         cfg.blockDim = dim3(THREADS, 1, 1);
@@ -538,7 +538,7 @@ grass_status launch_persistent(const LayerDesc* dev_descs, const LayerDesc& sing
         cfg.attrs = attr;
         cfg.numAttrs = 1;
         const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, x, single, max_k);
-        return e == cudaSuccess ? launch_status() : GRASS_ERR_CUDA;
+        return cuda_ok(e);
     };
     return f32 ? launch(factgrass_persistent_kernel<true>, 3) : launch(factgrass_persistent_kernel<false>, 1);
 }

@@ -110,7 +110,15 @@ constexpr size_t kDynSmemLimit = 226 * 1024;
 // launch-shape override set through grass_set_tuning, or `dflt` while the key is on automatic
 int64_t tuning(grass_tuning_key key, int64_t dflt);
 
-inline grass_status cuda_ok(cudaError_t e) { return e == cudaSuccess ? GRASS_OK : GRASS_ERR_CUDA; }
+// The runtime keeps the error of a call that failed until somebody asks for the last one, so whoever reports a failure asks:
+// otherwise the next launch, of another call, would be taken for the one that failed.
+inline bool cuda_failed(cudaError_t e)
+{
+    if (e == cudaSuccess) return false;
+    (void)cudaGetLastError();
+    return true;
+}
+inline grass_status cuda_ok(cudaError_t e) { return cuda_failed(e) ? GRASS_ERR_CUDA : GRASS_OK; }
 
 inline grass_status launch_status()
 {

@@ -441,7 +441,7 @@ static grass_status launch_compress(const T* g, int64_t n, int64_t p, int64_t ld
     auto launch = [&](auto kern) -> grass_status {
         if (smem > 48 * 1024) {
             cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-            if (e != cudaSuccess) return GRASS_ERR_CUDA;
+            if (cuda_failed(e)) return GRASS_ERR_CUDA;
         }
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3((unsigned)groups, (unsigned)pl.jsplit, 1);
@@ -460,7 +460,7 @@ static grass_status launch_compress(const T* g, int64_t n, int64_t p, int64_t ld
         const int use_smem = pl.use_smem;
         cudaError_t e = cudaLaunchKernelEx(&cfg, kern, g, n, p, ld, idx, kprime, sp.k, sp.s, sp.seed, scale, out,
                                            ld_out, j_per_cta, accumulate, use_smem, dev_status, pl.out_bf16, pl.idx_smem);
-        return e == cudaSuccess ? launch_status() : GRASS_ERR_CUDA;
+        return cuda_ok(e);
     };
     if (pl.dense) {
         if (sp.s == 1) return launch(grass_compress_kernel<T, S, U, true, true, kThreads>);
@@ -484,8 +484,8 @@ static grass_status dispatch_compress(const T* g, int64_t n, int64_t p, int64_t 
                                       uint32_t* dev_status, cudaStream_t st, int out_bf16)
 {
     int dev = 0, sms = 148;
-    if (cudaGetDevice(&dev) != cudaSuccess) return GRASS_ERR_CUDA;
-    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return GRASS_ERR_CUDA;
+    if (cuda_failed(cudaGetDevice(&dev))) return GRASS_ERR_CUDA;
+    if (cuda_failed(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev))) return GRASS_ERR_CUDA;
     const bool dense = idx == nullptr && tuning(GRASS_TUNE_COMPRESS_DENSE, 1) != 0 &&
                        (uintptr_t)g % (4 * sizeof(T)) == 0 && ld % 4 == 0;
     CompressPlan pl = plan_compress(n, kprime, sp.k, sms, dense);
@@ -507,7 +507,7 @@ static grass_status dispatch_compress(const T* g, int64_t n, int64_t p, int64_t 
     if (!pl.cluster && (pl.jsplit > 1 || !pl.use_smem)) {
         cudaError_t e = cudaMemset2DAsync(out, (size_t)ld_out * sizeof(float), 0, (size_t)sp.k * sizeof(float),
                                           (size_t)n, st);
-        if (e != cudaSuccess) return GRASS_ERR_CUDA;
+        if (cuda_failed(e)) return GRASS_ERR_CUDA;
     }
     switch (pl.S) {
         case 8: return launch_compress<T, 8, 2>(g, n, p, ld, idx, kprime, sp, out, ld_out, pl, dev_status, st);

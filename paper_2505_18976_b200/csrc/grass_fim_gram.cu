@@ -246,11 +246,11 @@ grass_status launch_fim(const float* X, int64_t n, int64_t k, int64_t ld, float 
 {
     using namespace gram;
     int dev = 0, sms = 148;
-    if (cudaGetDevice(&dev) != cudaSuccess) return GRASS_ERR_CUDA;
-    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return GRASS_ERR_CUDA;
+    if (cuda_failed(cudaGetDevice(&dev))) return GRASS_ERR_CUDA;
+    if (cuda_failed(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev))) return GRASS_ERR_CUDA;
     constexpr size_t smem = (size_t)NBUF * STAGE;
-    if (cudaFuncSetAttribute(gram_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
-        cudaFuncSetAttribute(gram_kernel, cudaFuncAttributePreferredSharedMemoryCarveout, 100) != cudaSuccess)
+    if (cuda_failed(cudaFuncSetAttribute(gram_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) ||
+        cuda_failed(cudaFuncSetAttribute(gram_kernel, cudaFuncAttributePreferredSharedMemoryCarveout, 100)))
         return GRASS_ERR_CUDA;
     const int64_t tiles = (k + TILE - 1) / TILE, ntiles = tiles * (tiles + 1) / 2;
     // Thread blocks per tile: enough to fill the machine (two per SM) with at least four steps each, and no accumulator
@@ -269,7 +269,7 @@ grass_status launch_fim(const float* X, int64_t n, int64_t k, int64_t ld, float 
     chunk = (chunk + STEP - 1) / STEP * STEP;
     if (ntiles * groups * cs > 0x7FFFFFFFLL) return GRASS_ERR_UNSUPPORTED;
     const int add_out = groups > 1;
-    if (add_out && cudaMemset2DAsync(F, (size_t)ld_f * sizeof(float), 0, (size_t)k * sizeof(float), (size_t)k, st) != cudaSuccess)
+    if (add_out && cuda_failed(cudaMemset2DAsync(F, (size_t)ld_f * sizeof(float), 0, (size_t)k * sizeof(float), (size_t)k, st)))
         return GRASS_ERR_CUDA;
     int nprod = (int)tuning(GRASS_TUNE_SPLIT_PRODUCTS, tc::kSplitProductsDefault);
     if (nprod != 3 && nprod != 4) nprod = 6;
@@ -289,7 +289,7 @@ grass_status launch_fim(const float* X, int64_t n, int64_t k, int64_t ld, float 
     const cudaError_t e = cudaLaunchKernelEx(&cfg, gram_kernel, X, (int32_t)n, (int32_t)k, ld, (int32_t)tiles,
                                              (int32_t)(groups * cs), (int32_t)chunk,
                                              scale, F, ld_f, vec_ok, add_out, nprod);
-    return e == cudaSuccess ? launch_status() : GRASS_ERR_CUDA;
+    return cuda_ok(e);
 }
 
 }  // namespace grass

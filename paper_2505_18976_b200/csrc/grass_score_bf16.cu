@@ -255,8 +255,8 @@ grass_status launch_score_bf16(const void* train, int64_t N, int64_t ld_train, c
     using namespace tc::h;
     if (N > 0x7FFFFFFFLL || M > 0x7FFFFFFFLL || D > 0x7FFFFFFFLL) return GRASS_ERR_UNSUPPORTED;
     int dev = 0, sms = 148;
-    if (cudaGetDevice(&dev) != cudaSuccess) return GRASS_ERR_CUDA;
-    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return GRASS_ERR_CUDA;
+    if (cuda_failed(cudaGetDevice(&dev))) return GRASS_ERR_CUDA;
+    if (cuda_failed(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev))) return GRASS_ERR_CUDA;
     Plan p;
     // column tiles: as few as hold 512 test rows each, of equal width
     const int64_t tiles_m = (M + 511) / 512;
@@ -277,11 +277,11 @@ grass_status launch_score_bf16(const void* train, int64_t N, int64_t ld_train, c
     if (!make_map(&map_train, train, N, D, ld_train, true, ROWS) ||
         !make_map(&map_test, test, M, D, ld_test, true, p.width / subs / 2))
         return GRASS_ERR_CUDA;
-    if (adds && cudaMemset2DAsync(scores, (size_t)ld_s * sizeof(float), 0, (size_t)M * sizeof(float), (size_t)N, st) != cudaSuccess)
+    if (adds && cuda_failed(cudaMemset2DAsync(scores, (size_t)ld_s * sizeof(float), 0, (size_t)M * sizeof(float), (size_t)N, st)))
         return GRASS_ERR_CUDA;
     const int out_vec = ((uintptr_t)scores % 16 == 0) && (ld_s % 4 == 0);
     auto launch = [&](auto kern) -> grass_status {
-        if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BUDGET + SCRATCH_BYTES) != cudaSuccess)
+        if (cuda_failed(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BUDGET + SCRATCH_BYTES)))
             return GRASS_ERR_CUDA;
         kern<<<(unsigned)(2 * used), THREADS_H, (size_t)p.stages * stage_bytes + SCRATCH_BYTES, st>>>(map_train, map_test, p, N, M, scores, ld_s,
                                                                                       out_vec);

@@ -321,8 +321,8 @@ grass_status launch_score_tc(const float* train, int64_t N, int64_t ld_train, co
 {
     if (N > 0x7FFFFFFFLL || M > 0x7FFFFFFFLL || D > 0x7FFFFFFFLL) return GRASS_ERR_UNSUPPORTED;
     int dev = 0, sms = 148;
-    if (cudaGetDevice(&dev) != cudaSuccess) return GRASS_ERR_CUDA;
-    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return GRASS_ERR_CUDA;
+    if (cuda_failed(cudaGetDevice(&dev))) return GRASS_ERR_CUDA;
+    if (cuda_failed(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev))) return GRASS_ERR_CUDA;
     tc::ScorePlan p;
     const int64_t tiles_m = (M + tc::BN - 1) / tc::BN;
     p.width = (int)(((M + tiles_m - 1) / tiles_m + 31) / 32 * 32);
@@ -339,9 +339,9 @@ grass_status launch_score_tc(const float* train, int64_t N, int64_t ld_train, co
     const size_t smem = (size_t)p.stages * stage_bytes + (size_t)p.ring * raw_bytes;
     CUtensorMap map_train, map_test;
     if (!make_map(&map_train, train, N, D, ld_train) || !make_map(&map_test, test, M, D, ld_test, false, n_half)) return GRASS_ERR_CUDA;
-    if (cudaFuncSetAttribute(tc::grass_score_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, tc::SMEM_BUDGET) != cudaSuccess)
+    if (cuda_failed(cudaFuncSetAttribute(tc::grass_score_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, tc::SMEM_BUDGET)))
         return GRASS_ERR_CUDA;
-    if (adds && cudaMemset2DAsync(scores, (size_t)ld_s * sizeof(float), 0, (size_t)M * sizeof(float), (size_t)N, st) != cudaSuccess)
+    if (adds && cuda_failed(cudaMemset2DAsync(scores, (size_t)ld_s * sizeof(float), 0, (size_t)M * sizeof(float), (size_t)N, st)))
         return GRASS_ERR_CUDA;
     const int out_vec_ok = ((uintptr_t)scores % 16 == 0) && (ld_s % 4 == 0);
     int nprod = (int)tuning(GRASS_TUNE_SPLIT_PRODUCTS, tc::kSplitProductsDefault);

@@ -316,8 +316,8 @@ static grass_status launch_t(const T* g, int64_t n, int64_t p, int64_t ld, const
     Layout t;
     if (!layout_of(t, p, sp.k, sizeof(T))) return GRASS_ERR_UNSUPPORTED;
     int dev = 0, sms = 148;
-    if (cudaGetDevice(&dev) != cudaSuccess) return GRASS_ERR_CUDA;
-    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return GRASS_ERR_CUDA;
+    if (cuda_failed(cudaGetDevice(&dev))) return GRASS_ERR_CUDA;
+    if (cuda_failed(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev))) return GRASS_ERR_CUDA;
     const int64_t pairs = (n + t.rows - 1) / t.rows, units = pairs * t.nchunks;
     if (t.nchunks > 0x7FFFFFFF) return GRASS_ERR_UNSUPPORTED;
     int64_t per_block = (units + sms - 1) / sms;
@@ -329,7 +329,7 @@ static grass_status launch_t(const T* g, int64_t n, int64_t p, int64_t ld, const
     if (launch_status() != GRASS_OK) return GRASS_ERR_CUDA;
     const size_t psm = (size_t)t.stages * t.stage_bytes + (size_t)t.rows * t.copies * t.k * 4;
     auto launch = [&](auto kern) -> grass_status {
-        if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)psm) != cudaSuccess) return GRASS_ERR_CUDA;
+        if (cuda_failed(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)psm))) return GRASS_ERR_CUDA;
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3((unsigned)blocks, 1, 1);
         cfg.blockDim = dim3(THREADS, 1, 1);
@@ -342,7 +342,7 @@ static grass_status launch_t(const T* g, int64_t n, int64_t p, int64_t ld, const
         cfg.numAttrs = 1;
         const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, g, n, ld, (const uint16_t*)table, t, out, ld_out, units, per_block, out_bf16,
                                                  dev_status);
-        return e == cudaSuccess ? launch_status() : GRASS_ERR_CUDA;
+        return cuda_ok(e);
     };
     return t.rows == 2 ? launch(project_kernel<T, 2>) : launch(project_kernel<T, 1>);
 }

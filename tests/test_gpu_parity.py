@@ -233,6 +233,18 @@ def test_grass_compress_empty_and_errors(G, oracle_mod):
         G.grass_compress(g, G.mask_to_device(idxh), 0, 1, 5)
 
 
+def test_a_failed_call_leaves_no_error_to_the_next(G, W, oracle_mod, tune):
+    """128 x 128 fp32 tiles and 40,000 bins are more shared memory than an SM has: the host refuses the launch."""
+    A = torch.zeros((2, 64, 200), device="cuda")
+    m = G.mask_to_device(G.grass_random_mask_host(200, 128, 1))
+    tune(factgrass_tile=128)
+    with pytest.raises(G.GrassError) as e:
+        G.factgrass_compress(A, A, m, m, 40_000, 1, 0)
+    assert e.value.code == 4
+    tune(factgrass_tile=None)
+    _grass_case(G, W, oracle_mod, 3, 500, 100, 64)
+
+
 def test_grass_compress_run_to_run(G, W, oracle_mod):
     """Float atomics reorder sums: repeated runs agree to a few ulps of the bin's mass."""
     g = W.dense_gradients(32, 100_000, 0.5, "normal", 1.0, 3, device="cuda")
