@@ -90,7 +90,7 @@ extern "C" grass_status grass_validate_mask(const uint32_t* idx, int64_t kprime,
     if (blocks > 148 * 8) blocks = 148 * 8;
     grass::validate_mask_kernel<<<(unsigned)blocks, 256, 0, (cudaStream_t)stream>>>(idx, kprime, p, flag.dev);
     if (grass::launch_status() != GRASS_OK) return GRASS_ERR_CUDA;
-    if (cuda_failed(cudaStreamSynchronize((cudaStream_t)stream))) return GRASS_ERR_CUDA;
+    if (grass::cuda_failed(cudaStreamSynchronize((cudaStream_t)stream))) return GRASS_ERR_CUDA;
     return *flag.host ? GRASS_ERR_BAD_MASK : GRASS_OK;
 }
 
