@@ -478,7 +478,7 @@ static grass_status run_factgrass(const factgrass_layer* layers, int32_t L, gras
     auto launch = [&](auto kern, size_t stage_bytes) -> grass_status {
         const size_t smem = kFgBufs * stage_bytes + bins_bytes;
         // static shared memory counts toward the 48 KB default limit too
-        if (cuda_failed(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)))
+        if (cuda_failed(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDynSmemLimit)))
             return GRASS_ERR_CUDA;
         cudaFuncAttributes fa;
         if (cuda_failed(cudaFuncGetAttributes(&fa, kern))) return GRASS_ERR_CUDA;

@@ -104,7 +104,9 @@ size_t sjlt_table_bytes(int64_t n, int64_t p, uint32_t k, uint32_t s, size_t ele
 grass_status launch_sjlt_table(const void* g, grass_dtype dt, int64_t n, int64_t p, int64_t ld, const grass_sjlt_spec& sp, float* out,
                                int64_t ld_out, void* table, uint32_t* dev_status, cudaStream_t st, int out_bf16);
 
-// dynamic shared memory that a thread block may have: 227 KB less 1 KB for what a kernel declares statically
+// Dynamic shared memory that a thread block may have: 227 KB less 1 KB for what a kernel declares statically.  A kernel whose need
+// varies asks for the right to this much in every call: the limit is the process's, and another thread, with another size,
+// may be between this call's setting and its launch.
 constexpr size_t kDynSmemLimit = 226 * 1024;
 
 // launch-shape override set through grass_set_tuning, or `dflt` while the key is on automatic

@@ -440,7 +440,7 @@ static grass_status launch_compress(const T* g, int64_t n, int64_t p, int64_t ld
     const float scale = 1.0f / sqrtf((float)sp.s);
     auto launch = [&](auto kern) -> grass_status {
         if (smem > 48 * 1024) {
-            cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDynSmemLimit);
             if (cuda_failed(e)) return GRASS_ERR_CUDA;
         }
         cudaLaunchConfig_t cfg = {};

@@ -227,7 +227,7 @@ static grass_status launch_rows_t(const T* g, int64_t n, int64_t p, int64_t ld, 
     const size_t smem = rows_smem_bytes(kprime, sp.k, &idx_bytes);
     const float scale = 1.0f / sqrtf((float)sp.s);
     auto launch = [&](auto kern) -> grass_status {
-        if (cuda_failed(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)))
+        if (cuda_failed(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDynSmemLimit)))
             return GRASS_ERR_CUDA;
         kern<<<dim3((unsigned)n, 1, 1), kRowsThreads, smem, st>>>(g, p, ld, idx, kprime, sp.k, sp.s, sp.seed, scale, out,
                                                                   ld_out, idx_bytes, dev_status, out_bf16);

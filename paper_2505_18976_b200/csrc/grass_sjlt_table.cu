@@ -329,7 +329,7 @@ static grass_status launch_t(const T* g, int64_t n, int64_t p, int64_t ld, const
     if (launch_status() != GRASS_OK) return GRASS_ERR_CUDA;
     const size_t psm = (size_t)t.stages * t.stage_bytes + (size_t)t.rows * t.copies * t.k * 4;
     auto launch = [&](auto kern) -> grass_status {
-        if (cuda_failed(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)psm))) return GRASS_ERR_CUDA;
+        if (cuda_failed(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDynSmemLimit))) return GRASS_ERR_CUDA;
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3((unsigned)blocks, 1, 1);
         cfg.blockDim = dim3(THREADS, 1, 1);
