@@ -15,6 +15,7 @@
 #include <ATen/cuda/EmptyTensor.h>
 #include <c10/cuda/CUDAStream.h>
 #include <torch/csrc/Dtype.h>
+#include <torch/csrc/Exceptions.h>
 #include <torch/csrc/autograd/python_variable.h>
 
 #include "../../include/grass.h"
@@ -132,11 +133,8 @@ const at::Tensor* out_rows(PyObject* out, int64_t rows, int64_t cols, at::Scalar
 
 #define ORDINARY(cond) do { if (!(cond)) Py_RETURN_NONE; } while (0)
 #define GUARD_BEGIN try {
-#define GUARD_END                                            \
-    } catch (const std::exception& e) {                      \
-        PyErr_SetString(PyExc_RuntimeError, e.what());       \
-        return nullptr;                                      \
-    }
+#define GUARD_END }                                          \
+    CATCH_ALL_ERRORS(return nullptr)     // as torch reports them: an allocation that fails is torch.OutOfMemoryError
 
 // grass_compress(g, idx, k, s, seed, out, p, dev_status, out_dtype)
 PyObject* py_grass_compress(PyObject*, PyObject* const* a, Py_ssize_t n)

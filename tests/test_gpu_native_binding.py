@@ -73,3 +73,24 @@ def test_errors_come_from_the_same_place():
     layers = [dict(A=g.view(2, 2, 64), G=g.view(2, 2, 64), mask_in=idx, mask_out=idx, k=8, s=1, seed=0, out_offset=-1)]
     with pytest.raises(ValueError):
         G.GroupedLayers(layers)
+
+
+@pytest.fixture
+def no_more_memory():
+    """Call it, and the allocator gives out nothing that it does not hold already."""
+    def close():
+        torch.cuda.empty_cache()
+        torch.cuda.set_per_process_memory_fraction(0.0)
+    yield close
+    torch.cuda.set_per_process_memory_fraction(1.0)
+
+
+def test_out_of_memory_is_torchs_exception(no_more_memory):
+    g, x = torch.zeros((1 << 16, 8), device="cuda"), torch.zeros((1 << 13, 8), device="cuda")
+    A = torch.zeros((1 << 15, 1, 8), device="cuda")
+    m = G.mask_to_device(G.grass_random_mask_host(8, 4, 1))
+    no_more_memory()
+    for call in (lambda: G.grass_compress(g, None, 4_096, 1, 0), lambda: G.factgrass_compress(A, A, m, m, 8_192, 1, 0),
+                 lambda: G.grass_score(g, x)):
+        with pytest.raises(torch.OutOfMemoryError):
+            call()
