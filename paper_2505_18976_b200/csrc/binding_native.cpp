@@ -133,8 +133,12 @@ const at::Tensor* out_rows(PyObject* out, int64_t rows, int64_t cols, at::Scalar
 
 #define ORDINARY(cond) do { if (!(cond)) Py_RETURN_NONE; } while (0)
 #define GUARD_BEGIN try {
-#define GUARD_END }                                          \
-    CATCH_ALL_ERRORS(return nullptr)     // as torch reports them: an allocation that fails is torch.OutOfMemoryError
+// as torch reports them: an allocation that fails is torch.OutOfMemoryError
+#define GUARD_END                                                           \
+    } catch (const std::exception&) {                                       \
+        torch::translate_exception_to_python(std::current_exception());     \
+        return nullptr;                                                     \
+    }
 
 // grass_compress(g, idx, k, s, seed, out, p, dev_status, out_dtype)
 PyObject* py_grass_compress(PyObject*, PyObject* const* a, Py_ssize_t n)
