@@ -13,7 +13,9 @@
 
 #include <ATen/core/Tensor.h>
 #include <ATen/cuda/EmptyTensor.h>
+#include <c10/cuda/CUDAFunctions.h>
 #include <c10/cuda/CUDAStream.h>
+#include <c10/util/Exception.h>
 #include <torch/csrc/Dtype.h>
 #include <torch/csrc/Exceptions.h>
 #include <torch/csrc/autograd/python_variable.h>
@@ -131,6 +133,21 @@ const at::Tensor* out_rows(PyObject* out, int64_t rows, int64_t cols, at::Scalar
     return t;
 }
 
+// Scratch that the library can do without: none where the pool has no more to give.  It comes from torch's stream-ordered pool
+// of the device whose current stream the call is enqueued on, so it may be handed out again as soon as this tensor is gone, to
+// work that is enqueued behind the kernels that use it.
+void* optional_scratch(size_t* bytes, at::Tensor* keep)
+{
+    if (*bytes == 0) return nullptr;
+    try {
+        *keep = empty2(1, (int64_t)*bytes, at::kByte, at::Device(at::kCUDA, c10::cuda::current_device()));
+        return keep->data_ptr();
+    } catch (const c10::OutOfMemoryError&) {
+        *bytes = 0;
+        return nullptr;
+    }
+}
+
 #define ORDINARY(cond) do { if (!(cond)) Py_RETURN_NONE; } while (0)
 #define GUARD_BEGIN try {
 // as torch reports them: an allocation that fails is torch.OutOfMemoryError
@@ -165,15 +182,9 @@ PyObject* py_grass_compress(PyObject*, PyObject* const* a, Py_ssize_t n)
     void* const st = current_stream();
     const void* gp = g->const_data_ptr();
     void* op = o->data_ptr();
-    // scratch from torch's stream-ordered pool: it may be handed out again as soon as this tensor is gone, to work that
-    // is enqueued behind the kernels that use it
     at::Tensor scratch;
-    void* wp = nullptr;
-    const size_t wbytes = idx ? 0 : api.compress_bytes((grass_dtype)dt, rows, p, idx, &sp);
-    if (wbytes > 0) {
-        scratch = empty2(1, (int64_t)wbytes, at::kByte, g->device());
-        wp = scratch.data_ptr();
-    }
+    size_t wbytes = idx ? 0 : api.compress_bytes((grass_dtype)dt, rows, p, idx, &sp);
+    void* const wp = optional_scratch(&wbytes, &scratch);
     grass_status rc;
     Py_BEGIN_ALLOW_THREADS
     rc = api.compress(gp, (grass_dtype)dt, rows, p, ld, idx, kprime, &sp, op, (grass_dtype)odt, ld_out, wp, wbytes, dev_status, st);
@@ -209,13 +220,8 @@ PyObject* py_factgrass_compress(PyObject*, PyObject* const* a, Py_ssize_t n)
     // Long fp32 calls above 64 x 64 can use a table of the projection; the rest would leave the scratch alone
     // (bf16 rows of one layer go to the cluster kernel).
     at::Tensor scratch;
-    void* wp = nullptr;
-    size_t wbytes = 0;
-    if (dt == GRASS_F32 && std::max(kin, kout) > 64 && B * T >= 8192) {
-        wbytes = api.grouped_bytes(1);
-        scratch = empty2(1, (int64_t)wbytes, at::kByte, A->device());
-        wp = scratch.data_ptr();
-    }
+    size_t wbytes = dt == GRASS_F32 && std::max(kin, kout) > 64 && B * T >= 8192 ? api.grouped_bytes(1) : 0;
+    void* const wp = optional_scratch(&wbytes, &scratch);
     const factgrass_layer layer = {ap, gp, mi, mo, (int32_t)d_in, (int32_t)d_out, (int32_t)kin, (int32_t)kout, sp, 0};
     grass_status rc;
     Py_BEGIN_ALLOW_THREADS

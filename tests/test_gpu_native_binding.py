@@ -94,3 +94,14 @@ def test_out_of_memory_is_torchs_exception(no_more_memory):
                  lambda: G.grass_score(g, x)):
         with pytest.raises(torch.OutOfMemoryError):
             call()
+
+
+def test_calls_do_without_the_scratch_that_they_cannot_have(no_more_memory):
+    """Plain SJLT of a batch wants a table of 2 bytes per position; with `out` given it needs no memory at all."""
+    n, p, k = 32, 1 << 24, 256
+    g = torch.zeros((n, p), device="cuda")
+    g[:, ::4_097] = 1.0
+    want, out = G.grass_compress(g, None, k, 1, 0), torch.empty((n, k), device="cuda")
+    no_more_memory()
+    assert G.grass_compress(g, None, k, 1, 0, out=out) is out
+    assert torch.equal(out, want)      # sums of ones, exact in any order
