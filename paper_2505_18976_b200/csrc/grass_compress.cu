@@ -350,7 +350,7 @@ struct CompressPlan {
     int U;          // gathered loads in flight per thread and sample
 };
 
-static CompressPlan plan_compress(int64_t n, int64_t kprime, uint32_t k, int sm_count, bool dense)
+static CompressPlan plan_compress(int64_t n, int64_t p, int64_t kprime, uint32_t k, int sm_count, bool dense)
 {
     CompressPlan pl;
     pl.dense = dense;
@@ -379,36 +379,45 @@ static CompressPlan plan_compress(int64_t n, int64_t kprime, uint32_t k, int sm_
     bool whole = false;
     if (!dense) {
         whole = S == 1 && groups >= sm_count && kprime <= (int64_t)4 * kThreads * U;
-        int t = whole ? kThreads : 2 * kThreads;
+        int t = whole || (!pl.use_smem && groups >= (int64_t)sm_count * 4) ? kThreads : 2 * kThreads;
         if (whole)
             while ((int64_t)t * U < kprime) t *= 2;
         t = (int)tuning(GRASS_TUNE_COMPRESS_THREADS, t);
         pl.threads = (t == 2 * kThreads || t == 4 * kThreads) ? t : kThreads;
     }
     // Split of the positions over a cluster of up to 8 thread blocks.  A block's share has to be worth its k bins (zeroed,
-    // exchanged and stored): at least k positions, or k / 2 while there are fewer blocks than SMs, and at least 1,024
-    // (one row of k' = 8,192, k = 2,048: 8.2 us over 4 blocks, 6.2 us over 8; 512 rows of k' = 65,536: 345 us
-    // over 2 blocks, 332 us over 8), and a full round of loads once the blocks fill the machine (318 rows of k' = 10,510,
-    // k = 1,000 in bf16: 47 us over 8 blocks, 36 over 2), half of one where the next split would (100 rows of
-    // k' = 9,000, k = 700: 18.4 over 8, 16.6 over 4).  Streamed rows keep one full round of loads per block.
+    // exchanged and stored): at least k positions, k / 2 while there are fewer blocks than SMs and k / 4 while the next split
+    // has room beside the rest (one block per SM, two with bins of up to 48 KB), and at least 1,024 (one row of k' = 8,192, k =
+    // 2,048: 8.2 us over 4 blocks, 6.2 us over 8; 17 rows of k' = 8,192, k = 20,000: 14.4 us over one, 10.3 over 4; 512 rows of
+    // k' = 65,536: 345 us over 2 blocks, 332 us over 8), and a full round of loads once the blocks fill the machine (318 rows
+    // of k' = 10,510, k = 1,000 in bf16: 47 us over 8 blocks, 36 over 2), half of one where the next split would (100 rows of
+    // k' = 9,000, k = 700: 18.4 over 8, 16.6 over 4).  Many rows under a mask of every second element or more are not split:
+    // their loads are short (3,000 rows of 33,000 elements, all kept, k = 2,048: 413 us over 8 blocks, 261 over one; 600 rows of
+    // 200,000 elements, every second kept: 287 over one, 261 over 8).
+    // Streamed rows, and rows without bins in shared memory, keep one full round of 256 threads' loads per block and go up to
+    // four blocks per SM; the latter run 256 threads once their rows make that many (671 rows of k' = 100,000, k = 200,000: 524 us,
+    // 613 with 512 threads).
     const int64_t round = (int64_t)pl.threads * U;
+    const int64_t max_js = std::max<int64_t>(1, kprime / ((int64_t)kThreads * U));
+    const int64_t fit = pl.use_smem ? std::max<int64_t>(1, std::min<int64_t>(2, kDynSmemLimit / (bin_bytes + 1024))) : 2;
     int64_t js = 1;
-    if (dense) {
-        const int64_t max_js = std::max<int64_t>(1, kprime / round);
+    if (dense || (!pl.use_smem && !whole)) {
         while (js < 8 && groups * js < (int64_t)sm_count * 4 && js * 2 <= max_js) js *= 2;
-    } else if (!whole) {
+    } else if (!whole && !(p <= 2 * kprime && groups >= (int64_t)(kprime <= 65536 ? 6 : 16) * sm_count)) {
         while (js < 8) {
             const int64_t share = kprime / (js * 2);
-            if (share < 1024 || share < (int64_t)(groups * js < sm_count ? k / 2 : k)) break;
+            const bool room = groups * js * 2 <= sm_count * (bin_bytes <= 48 * 1024 ? fit : 1);
+            if (share < 1024 || share < (int64_t)(room ? k / 4 : (groups * js < sm_count ? k / 2 : k))) break;
             if (share < round && (groups * js >= 4 * sm_count || (groups * js * 2 > 4 * sm_count && share < round / 2))) break;
             js *= 2;
         }
     }
     pl.cluster = 1;
-    const int64_t max_js = std::max<int64_t>(1, kprime / ((int64_t)kThreads * U));
-    if (groups * js < sm_count && js * 2 <= max_js && js == 8) {
-        // very few samples: split wider than a cluster allows and reduce with global atomics
-        js = ((int64_t)sm_count * 2 + groups - 1) / groups;
+    if (groups * js < sm_count && js * 2 <= max_js && (js == 8 || groups * 16 <= sm_count)) {
+        // Very few samples: split wider than a cluster allows and reduce with global atomics, as many blocks as are resident
+        // with their bins (2 rows of k' = 100,000, k = 30,000: 31 us over 2 blocks each, 10.4 over 48; 5 rows at k = 50,000, where
+        // an SM holds one block: 31 us over 2, 15.4 over 24, 19.5 over 48).
+        js = std::min((sm_count * 2 + groups - 1) / groups, std::max<int64_t>(1, sm_count * fit / groups));
         if (js > max_js) js = max_js;
         pl.cluster = 0;
     }
@@ -488,7 +497,7 @@ static grass_status dispatch_compress(const T* g, int64_t n, int64_t p, int64_t 
     if (cuda_failed(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev))) return GRASS_ERR_CUDA;
     const bool dense = idx == nullptr && tuning(GRASS_TUNE_COMPRESS_DENSE, 1) != 0 &&
                        (uintptr_t)g % (4 * sizeof(T)) == 0 && ld % 4 == 0;
-    CompressPlan pl = plan_compress(n, kprime, sp.k, sms, dense);
+    CompressPlan pl = plan_compress(n, p, kprime, sp.k, sms, dense);
     pl.out_bf16 = out_bf16;
     // whole-row thread blocks, one for every SM or more: the index list (up to 48 KB) goes into shared memory, where the bins
     // leave room for it

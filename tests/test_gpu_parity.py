@@ -164,6 +164,14 @@ def test_grass_compress_bins_that_leave_no_room_for_the_index_list(G, W, oracle_
     _grass_case(G, W, oracle_mod, n, p, kprime, k)
 
 
+# Splits of the positions: without bins in shared memory, wider than a cluster with bins that fill an SM, shares of a quarter
+# of the bins, many rows that are not split
+@pytest.mark.parametrize("n,p,kprime,k", [(1, 150_000, 100_000, 100_000), (3, 40_000, 33_000, 51_300), (2, 200_000, 100_000, 30_000),
+                                          (5, 120_000, 100_000, 50_000), (17, 20_000, 8_192, 20_000), (900, 9_001, 9_001, 300)])
+def test_grass_compress_position_splits(G, W, oracle_mod, n, p, kprime, k):
+    _grass_case(G, W, oracle_mod, n, p, kprime, k)
+
+
 def test_grass_compress_student_t(G, W, oracle_mod):
     _grass_case(G, W, oracle_mod, 8, 1 << 18, 1 << 14, 4_096, zero_prob=0.7, dist="student_t3", scale=1e-2)
 
