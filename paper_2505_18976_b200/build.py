@@ -12,7 +12,7 @@ CSRC = os.path.join(HERE, "csrc")
 SO = os.path.join(HERE, "libgrass_b200.so")
 NATIVE = os.path.join(HERE, "_native.so")
 NATIVE_SRC = "binding_native.cpp"
-SOURCES = ["grass_compress.cu", "grass_compress_rows.cu", "grass_sjlt_table.cu", "factgrass.cu", "factgrass_cluster.cu", "factgrass_persistent.cu", "grass_score.cu", "grass_score_tc.cu", "grass_score_bf16.cu", "grass_fim.cu", "grass_fim_gram.cu", "grass_util.cu"]
+SOURCES = ["grass_compress.cu", "grass_compress_rows.cu", "grass_sjlt_table.cu", "factgrass.cu", "factgrass_cluster.cu", "factgrass_persistent.cu", "grass_score.cu", "grass_score_tc.cu", "grass_score_bf16.cu", "grass_fim.cu", "grass_fim_gram.cu", "grass_fim_blocks.cu", "grass_util.cu"]
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
               "-Xcompiler", "-fPIC", "-cudart", "static"]
 

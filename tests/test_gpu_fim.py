@@ -134,6 +134,27 @@ def test_factor_and_apply_shapes(G, k, M, pad):
     assert (x @ A - b).norm() <= u * A.norm() * x.norm()
 
 
+# Many right-hand sides are solved block column by block column: ragged last block, ragged last tile of rows, row strides
+@pytest.mark.parametrize("k,M,pad", [(63, 16_400, 1), (64, 16_400, 0), (130, 16_411, 3), (513, 16_411, 2), (1_030, 5_003, 0)])
+def test_apply_many_right_hand_sides(G, k, M, pad):
+    X = _compressed(2 * k + 3, k, 70 + k)
+    F = torch.full((k, k + pad), float("nan"), device="cuda")[:, :k]
+    G.grass_fim(X, out=F)
+    A = F.double() + 0.05 * torch.eye(k, device="cuda", dtype=torch.float64)
+    G.grass_fim_factor(F, 0.05)
+    wide = torch.full((M, k + pad), float("nan"), device="cuda")
+    Bm = wide[:, :k]
+    Bm.copy_(_compressed(M, k, 71 + k))
+    b, few = Bm.double(), Bm[:100].clone()
+    G.grass_fim_apply(F, Bm)
+    assert pad == 0 or torch.isnan(wide[:, k:]).all()
+    x, y = Bm.double(), G.grass_fim_apply(F, few).double()
+    # the bound of test_factor_and_apply_shapes, and the same for the difference from a solve of the first rows alone
+    u = 6.0 * k ** 0.5 * 2.0 ** -24
+    assert (x @ A - b).norm() <= u * A.norm() * x.norm()
+    assert ((x[:100] - y) @ A).norm() <= 2.0 * u * A.norm() * y.norm()
+
+
 # Pivots at both ends of the fp32 range: below 2^-126 they are subnormal, above 2^126 their reciprocals are
 @pytest.mark.parametrize("scale", [1.0e-38, 1.0, 1.2e38])
 def test_factor_of_scaled_matrices(G, scale):
