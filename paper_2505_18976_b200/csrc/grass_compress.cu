@@ -577,11 +577,20 @@ extern "C" grass_status grass_compress_ws(const void* g, grass_dtype dt, int64_t
         return grass::cuda_ok(cudaMemset2DAsync(out, (size_t)ld_out * osz, 0, (size_t)spec->k * osz, (size_t)n, st));
     }
     if (!idx && workspace) {
-        // Short fp32 rows that the streamed path can read with vector loads stay there: emptying the bins after every two
-        // rows costs the table's kernel what it saves (2,048 x 20,000, k = 4,096: 76 against 85 us dense, 41 against 45 at
-        // 99 % zeros; at 50,000 positions 158 against 137 and 74 against 63).
-        const bool streamed = dt == GRASS_F32 && (uintptr_t)g % 16 == 0 && ld % 4 == 0 && p < 32768 && spec->k <= 8192 &&
-                              grass::tuning(GRASS_TUNE_COMPRESS_DENSE, -1) != 2;
+        // Short rows that the streamed path can read with vector loads stay there: emptying the bins after every two rows costs
+        // the table's kernel what it saves (fp32, 2,048 x 20,000, k = 4,096: 76 against 85 us dense, 41 against 45 at 99 %
+        // zeros; at 50,000 positions 158 against 137 and 74 against 63.  bf16, whose streamed path costs more per value,
+        // 4,096 rows: 4,000 positions, k = 2,048 39 against 57 us dense; 8,000, k = 1,024 74 against 82; 16,000 156 against 130).
+        // A bf16 result is rounded once, so a row is one block's there; the streamed path makes a row a cluster's, and the
+        // gathers do for unaligned rows (fp32, 64 x 300,000, k = 2,048: 55 us against 150; 140 rows 81 against 150; 300 rows
+        // of bf16 534 against 290; unaligned, 64 rows 94 against 105, 100 rows 136 against 105).
+        const bool f32 = dt == GRASS_F32, vec = (uintptr_t)g % (f32 ? 16 : 8) == 0 && ld % 4 == 0;
+        const bool brief = f32 ? p < 32768 && spec->k <= 8192 : p < (spec->k <= 1024 ? 10000 : 6000) && spec->k <= 4096;
+        int dev = 0, sms = 148;
+        if (grass::cuda_failed(cudaGetDevice(&dev)) || grass::cuda_failed(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)))
+            return GRASS_ERR_CUDA;
+        const bool few = out_bf16 && n < (vec ? sms : sms / 2);
+        const bool streamed = ((vec && brief) || few) && grass::tuning(GRASS_TUNE_COMPRESS_DENSE, -1) != 2;
         const size_t need = streamed ? 0 : grass_compress_workspace_bytes(dt, n, p, idx, spec);
         if (need > 0 && workspace_bytes >= need && (uintptr_t)workspace % 128 == 0)
             return grass::launch_sjlt_table(g, dt, n, p, ld, *spec, out, ld_out, workspace, dev_status, st, out_bf16);
