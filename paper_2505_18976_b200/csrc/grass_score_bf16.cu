@@ -16,7 +16,7 @@
 // delivers (128 + M / 2) rows per block and 64 k-values, hence the 256-row pairs and a tile as wide as the test set.  One
 // turn of the issuing threads (wait, expect, load; wait, multiply, commit) takes 600 cycles whatever it moves, 16 KB of
 // train rows a turn are then 3.7-4.8 TB/s over the chip and 32 KB 6.7: stages of 128 k-values wherever three of them fit.
-// Measured (before: 256-column pairs for M > 256, one block per 128 rows for M <= 256): 4,656 x 300 x 49,152 285 -> 140 us,
+// Measured (before: 256-column pairs for M > 256, one block per 128 rows for M <= 256): 4,656 x 300 x 49,152 285 -> 138 us,
 // 16,384 x 256 x 16,384 148 -> 128 us, 16,384 x 256 x 4,096 46 -> 42 us, 3,854 x 4 x 55,512 127 -> 83 us (5.2 TB/s).
 //   warp 0-3  drain the accumulator, warp 4 allocates tensor memory and issues the MMAs (leader), warp 5 issues the loads
 // Every mbarrier wait is bounded; a block whose wait expires marks its part with NaN and still reaches the cluster barrier.
@@ -258,18 +258,41 @@ grass_status launch_score_bf16(const void* train, int64_t N, int64_t ld_train, c
     if (cuda_failed(cudaGetDevice(&dev))) return GRASS_ERR_CUDA;
     if (cuda_failed(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev))) return GRASS_ERR_CUDA;
     Plan p;
-    // column tiles: as few as hold 512 test rows each, of equal width
-    const int64_t tiles_m = (M + 511) / 512;
-    const int64_t want_w = (M + tiles_m - 1) / tiles_m;
-    p.width = (int)(want_w <= 256 ? (want_w + 31) / 32 * 32 : (want_w + 63) / 64 * 64);
-    const int subs = p.width > 256 ? 2 : 1;
-    const int box_bytes = A_BYTES + p.width / 2 * ROW;
-    const int kw = 3 * 2 * box_bytes <= SMEM_BUDGET && D > BKH ? 2 : 1;
-    const int stage_bytes = kw * box_bytes;
-    p.stages = std::min(MAX_STAGES, SMEM_BUDGET / stage_bytes);
+    int subs = 1, kw = 1, stage_bytes = 0;
+    int64_t tiles_m = 1, ktiles = 1, run = 1;
+    // column tiles: as few as hold `cap` test rows each, of equal width
+    auto shape = [&](int64_t cap) {
+        tiles_m = (M + cap - 1) / cap;
+        const int64_t want_w = (M + tiles_m - 1) / tiles_m;
+        p.width = (int)(want_w <= 256 ? (want_w + 31) / 32 * 32 : (want_w + 63) / 64 * 64);
+        subs = p.width > 256 ? 2 : 1;
+        const int box_bytes = A_BYTES + p.width / 2 * ROW;
+        kw = 3 * 2 * box_bytes <= SMEM_BUDGET && D > BKH ? 2 : 1;
+        stage_bytes = kw * box_bytes;
+        ktiles = (D + kw * BKH - 1) / (kw * BKH);
+        run = D > 16384 ? MAX_RUN / (kw * BKH) : ktiles;
+    };
     p.tiles_n = (N + 2 * ROWS - 1) / (2 * ROWS);
-    const int64_t ktiles = (D + kw * BKH - 1) / (kw * BKH);
-    const int64_t run = D > 16384 ? MAX_RUN / (kw * BKH) : ktiles;
+    // Tiles of up to 512 test rows read the train rows once for two accumulators, but take twice as long to drain as tiles of
+    // up to 256, which decides for all but large problems (4,656 x 300 x 49,152: 138 us in one tile of 320, 197 in two; 4,656 x
+    // 512 x 1,024: 39 and 22; 1,000 x 512 x 512: 23 and 14).  Estimated in microseconds: 64 k-values are a turn of the issuing
+    // threads or the operands' way from L2, whichever is longer; then the drain and, for pieces of tiles, the zeroing.  Of 310
+    // combinations of N = 1 .. 8,000, M = 257 .. 1,024 and D = 64 .. 49,152 two were more than 4 % slower than with 512.
+    auto estimate = [&]() {
+        const double t = kw * std::max(0.3 / kw, std::max(0.2 / 256 * p.width, 0.3 / 256 * (128 + p.width / 2)));
+        tc::WorkPlan trial;
+        bool unused;
+        int64_t least;
+        tc::plan_work(trial, p.tiles_n * tiles_m, ktiles, run, sms / 2, (int64_t)((1.0 + 0.025 * p.width) / t), (int64_t)(4.0 / t), 0, &unused, &least);
+        return (double)least * t;
+    };
+    shape(512);
+    if (subs == 2) {
+        const double wide = estimate();
+        shape(256);
+        if (wide <= estimate()) shape(512);
+    }
+    p.stages = std::min(MAX_STAGES, SMEM_BUDGET / stage_bytes);
     // 64 k-values take about 0.3 us
     bool adds;
     const int64_t used = plan_work(p.work, p.tiles_n * tiles_m, ktiles, run, sms / 2, 10 / kw, 12 / kw, tuning(GRASS_TUNE_SCORE_SPLITS, -1), &adds);

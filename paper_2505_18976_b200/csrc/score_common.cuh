@@ -173,9 +173,10 @@ __device__ __forceinline__ bool next_segment(const WorkPlan& p, int64_t& u, int6
 }
 // Chooses the cheapest of: whole tiles, pieces of tiles (one per pair), an even cut of all units.  Costs in k tiles:
 // drain = emptying the pipeline and the accumulators after a segment, zero = zeroing the output that pieces are added
-// into.  forced > 0: that many pieces per tile.  Returns the number of pairs; *adds: pieces are added.
+// into.  forced > 0: that many pieces per tile.  Returns the number of pairs; *adds: pieces are added; *least (nullable):
+// the cost of the plan that was found, forced or not.
 inline int64_t plan_work(WorkPlan& p, int64_t tiles, int64_t ktiles, int64_t max_run, int64_t pairs, int64_t drain, int64_t zero,
-                         int64_t forced, bool* adds)
+                         int64_t forced, bool* adds, int64_t* least = nullptr)
 {
     p.ktiles = ktiles;
     p.units = tiles * ktiles;
@@ -194,7 +195,8 @@ inline int64_t plan_work(WorkPlan& p, int64_t tiles, int64_t ktiles, int64_t max
     }
     const int64_t even = (p.units + pairs - 1) / pairs;
     const int64_t segments = even / p.run + 2;             // at most
-    if (even + segments * drain + zero < best) { p.split = 0; p.per_pair = even; }
+    if (even + segments * drain + zero < best) { best = even + segments * drain + zero; p.split = 0; p.per_pair = even; }
+    if (least) *least = best;
     if (forced > 0) {
         p.per_pair = (ktiles + std::min(forced, ktiles) - 1) / std::min(forced, ktiles);
         p.split = (ktiles + p.per_pair - 1) / p.per_pair;

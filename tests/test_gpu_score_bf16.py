@@ -87,10 +87,11 @@ def test_score_of_a_bf16_cache_tracks_the_fp32_scores(G):
     assert float(((full - half).abs() / scale).max()) < 2.0 ** -9
 
 
-# Stages of one and of two boxes (D up to 64 and beyond; widths that leave no room for three long stages), one and two
-# accumulators, several column tiles; ranges of k that begin and end inside a tile, runs of 8,192; ragged last rows
+# Stages of one and of two boxes (D up to 64 and beyond; widths that leave no room for three long stages), one and (where the
+# problem is large) two accumulators, several column tiles; ranges of k that begin and end inside a tile, runs of 8,192; ragged last rows
 @pytest.mark.parametrize("N,M,D", [(256, 32, 64), (255, 33, 72), (600, 300, 1_000), (1_000, 384, 136), (300, 385, 2_056),
-                                   (700, 512, 512), (150, 1_100, 8_200), (2_900, 260, 17_000), (40_000, 20, 128)])
+                                   (700, 512, 512), (150, 1_100, 8_200), (2_900, 260, 17_000), (40_000, 20, 128),
+                                   (4_700, 310, 20_008), (4_700, 500, 20_008), (16_500, 512, 4_104)])
 def test_score_bf16_shapes(G, N, M, D):
     g = torch.Generator(device="cuda")
     g.manual_seed(N + M)
