@@ -262,7 +262,8 @@ grass_status launch_fim(const float* X, int64_t n, int64_t k, int64_t ld, float 
     // With many tiles, pairs: wide clusters leave SMs of a partition idle (36 tiles: 58 us with pairs and 75 with eights
     // at n = 4,656, k = 1,024); with few tiles, eights save global reductions (3 tiles: 18 against 30 us at n = 512).
     int64_t cs = 1;
-    while (cs * 2 <= want && cs < (ntiles >= 16 ? 2 : 8)) cs *= 2;
+    // (eight also where there are too few samples for them: each stores an eighth of the tile)
+    while (cs < (ntiles >= 16 ? 2 : 8) && (cs * 2 <= want || ntiles < 16)) cs *= 2;
     int64_t groups = std::max<int64_t>(1, want / cs);
     groups = std::max<int64_t>(groups, (n + 8192 * cs - 1) / (8192 * cs));
     int64_t chunk = (n + groups * cs - 1) / (groups * cs);
