@@ -379,7 +379,7 @@ static CompressPlan plan_compress(int64_t n, int64_t p, int64_t kprime, uint32_t
     bool whole = false;
     if (!dense) {
         whole = S == 1 && groups >= sm_count && kprime <= (int64_t)4 * kThreads * U;
-        int t = whole || (!pl.use_smem && groups >= (int64_t)sm_count * 4) ? kThreads : 2 * kThreads;
+        int t = whole || (!pl.use_smem && p > 2 * kprime && groups >= (int64_t)sm_count * 4) ? kThreads : 2 * kThreads;
         if (whole)
             while ((int64_t)t * U < kprime) t *= 2;
         t = (int)tuning(GRASS_TUNE_COMPRESS_THREADS, t);
@@ -395,8 +395,8 @@ static CompressPlan plan_compress(int64_t n, int64_t p, int64_t kprime, uint32_t
     // their loads are short (3,000 rows of 33,000 elements, all kept, k = 2,048: 413 us over 8 blocks, 261 over one; 600 rows of
     // 200,000 elements, every second kept: 287 over one, 261 over 8).
     // Streamed rows, and rows without bins in shared memory, keep one full round of 256 threads' loads per block and go up to
-    // four blocks per SM; the latter run 256 threads once their rows make that many (671 rows of k' = 100,000, k = 200,000: 524 us,
-    // 613 with 512 threads).
+    // four blocks per SM; under sparse masks the latter run 256 threads once their rows make that many (671 rows of k' =
+    // 100,000 of 800,000, k = 200,000: 524 us, 613 with 512 threads; 1,024 whole rows of 65,536, k = 60,000: 641 and 504).
     const int64_t round = (int64_t)pl.threads * U;
     const int64_t max_js = std::max<int64_t>(1, kprime / ((int64_t)kThreads * U));
     const int64_t fit = pl.use_smem ? std::max<int64_t>(1, std::min<int64_t>(2, kDynSmemLimit / (bin_bytes + 1024))) : 2;
