@@ -417,11 +417,14 @@ static grass_status run_factgrass(const factgrass_layer* layers, int32_t L, gras
     // 3,072 at 128 x 128: 27.7 -> 28.8 us at 1.7 steps, 38.7 -> 40.5 at 3.5, 62.3 -> 61.7 at 6.9; at 72 x 72: 39.8 -> 33.7 at
     // 3.5.  With an item for every SM the streaming kernel projects as often, at four tiles per block, and the persistent
     // one is faster down to one step per item (16 layers of 16 x 32 tokens, 128 x 128 bf16: 75.5 -> 34.8 us).
-    // bf16 (half the bytes, one accumulator) leaves the projection more of the time: layers with a side of at most 64, which the
-    // streaming kernel covers with two tiles instead of four, stay there (24 layers x 8 x 256, 128 x 32: 25 us there, 38 here;
-    // 128 x 64 with 1,024 tokens is even: 129 and 120), and so do up to 64 tokens per item with fewer than three items for two SMs
-    // (156 items of 16 tokens, 128 x 128: 26.7 us there, 30.8 here; 240 items: 32.9 and 30.8).  fp32 is 1.3 to 3 times as fast
-    // here in all of these.
+    // bf16 (half the bytes, one accumulator) leaves the projection more of the time, and the streaming kernel is the faster one
+    //  - for layers with a side of at most 64, two of its tiles instead of four, while there are fewer than two items per SM and
+    //    two thread blocks with their bins fit the 64 KB that it gives to shared memory (248 items of 250 tokens, 96 x 48, k
+    //    = 1,536: 33 us there, 46 here; 336 items: 104 and 59; 160 items, k = 4,096: 87 and 37), with up to 64 tokens for half
+    //    an item more and with small k throughout (336 items of 33 tokens, 128 x 16, k = 1,024: 22.6 and 30.7; 720: 35 and 41);
+    //  - for up to 64 tokens per item, small k and few more items than SMs (160 items of 16 tokens, k = 1,024, 128 x 128: 26.7 us
+    //    there, 30.8 here; k = 1,536: 30.9 and 29.6; 216 items: 30.2 and 30.8).
+    // fp32 is 1.1 to 3 times as fast here in all of these.
     auto persistent = [&](const LayerDesc* hd) {
         const int64_t forced = tuning(GRASS_TUNE_FACTGRASS_PATH, -1);
         if (epi != kEpiSjlt || out_bf16 || T <= 0 || !table || cluster_nc > 1 || !persistent_fits(hd, L, B, tok_count)) return false;
@@ -429,8 +432,14 @@ static grass_status run_factgrass(const factgrass_layer* layers, int32_t L, gras
         const int64_t items = (int64_t)L * B, steps = (T + kTokTile - 1) / kTokTile * items;
         if (!f32) {
             int32_t wide = 0;
-            for (int l = 0; l < L; ++l) wide += std::min(hd[l].kin, hd[l].kout) > (T >= 1024 ? 32 : 64);
-            if (2 * wide < L || (T <= 2 * kTokTile && 2 * items < 3 * (int64_t)sms)) return false;
+            for (int l = 0; l < L; ++l) wide += std::min(hd[l].kin, hd[l].kout) > 64;
+            const bool brief = T <= 2 * kTokTile, small_k = max_k <= 1024;
+            if (2 * wide < L) {
+                if (max_k <= 3500 && 2 * items < (brief ? 5 : 4) * (int64_t)sms) return false;
+                if (brief && small_k) return false;
+            } else if (brief && small_k && 4 * items < 5 * (int64_t)sms) {
+                return false;
+            }
         }
         return max_kk > 64 && (items >= sms || steps >= (max_kk > 96 ? 4 : 3) * (int64_t)sms);
     };
