@@ -154,6 +154,15 @@ grass_status factgrass_compress_grouped_out(const factgrass_layer* layers /*host
                                             void* stream);
 
 /*
+ * Scratch of a single layer: factgrass_compress_grouped_out with L = 1 and a workspace of this many bytes (256-byte
+ * aligned) projects through a table where that is the faster way; 0 means that the call would not use it.  Without
+ * it, and in factgrass_compress, factgrass_compress_varlen and factgrass_compress_grouped_static, which take none, fp32
+ * layers run on the streaming kernel: the same results up to the order of additions.
+ */
+size_t factgrass_compress_workspace_bytes(grass_dtype dt, int32_t B, int32_t T, int32_t kin, int32_t kout,
+                                          const grass_sjlt_spec* spec /*host*/);
+
+/*
  * grass_compress_out with device scratch.  The identity mask (plain SJLT) of a large batch is projected through a table
  * of the projection that the call builds once for all samples; the table lives in the caller's scratch.
  *   grass_compress_workspace_bytes  what the call with these arguments would use; 0 means it uses none.

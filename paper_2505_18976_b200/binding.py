@@ -34,7 +34,8 @@ EXPORTS = ("grass_compress", "factgrass_compress", "factgrass_compress_grouped",
            "factmask_compress_grouped",
            "factgrass_grouped_workspace_bytes", "factgrass_compress_grouped_static", "grass_score", "grass_sjlt_table", "grass_validate_mask",
            "grass_random_mask_host", "grass_status_string", "grass_to_bf16", "grass_score_bf16", "grass_set_tuning",
-           "grass_compress_out", "factgrass_compress_grouped_out", "grass_compress_workspace_bytes", "grass_compress_ws")
+           "grass_compress_out", "factgrass_compress_grouped_out", "grass_compress_workspace_bytes", "grass_compress_ws",
+           "factgrass_compress_workspace_bytes")
 
 # grass_tuning_key in include/grass.h
 TUNE = {"compress_samples": 0, "compress_jsplit": 1, "compress_cluster": 2, "compress_dense": 3,
@@ -101,6 +102,8 @@ def lib() -> ctypes.CDLL:
                                                         vp, vp, vp, i64, vp, ctypes.c_size_t, vp, vp]
         L.factgrass_grouped_workspace_bytes.restype = ctypes.c_size_t
         L.factgrass_grouped_workspace_bytes.argtypes = [i32]
+        L.factgrass_compress_workspace_bytes.restype = ctypes.c_size_t
+        L.factgrass_compress_workspace_bytes.argtypes = [ctypes.c_int, i32, i32, i32, i32, sp]
         L.factgrass_compress_grouped_static.restype = st
         L.factgrass_compress_grouped_static.argtypes = [ctypes.POINTER(FactgrassLayer), i32, ctypes.c_int, i32, i32, vp,
                                                         i64, vp, vp]
@@ -135,7 +138,7 @@ def lib() -> ctypes.CDLL:
         L.grass_status_string.argtypes = [st]
         from . import _native as native     # built beside the library; missing = not built, no fallback
         native.bind(GrassError, *(ctypes.cast(getattr(L, f), vp).value for f in (
-            "grass_compress_ws", "factgrass_grouped_workspace_bytes", "factgrass_compress_varlen", "factgrass_compress_grouped_out",
+            "grass_compress_ws", "factgrass_compress_workspace_bytes", "factgrass_compress_varlen", "factgrass_compress_grouped_out",
             "factgrass_compress_grouped_varlen", "grass_score", "grass_score_bf16", "grass_compress_workspace_bytes")))
         _native = native
         _lib = L

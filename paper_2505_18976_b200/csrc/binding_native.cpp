@@ -28,7 +28,7 @@ namespace {
 struct Api {
     decltype(&::grass_compress_ws) compress = nullptr;
     decltype(&::grass_compress_workspace_bytes) compress_bytes = nullptr;
-    decltype(&::factgrass_grouped_workspace_bytes) grouped_bytes = nullptr;
+    decltype(&::factgrass_compress_workspace_bytes) layer_bytes = nullptr;
     decltype(&::factgrass_compress_varlen) factgrass_varlen = nullptr;
     decltype(&::factgrass_compress_grouped_out) grouped_out = nullptr;
     decltype(&::factgrass_compress_grouped_varlen) grouped_varlen = nullptr;
@@ -217,10 +217,8 @@ PyObject* py_factgrass_compress(PyObject*, PyObject* const* a, Py_ssize_t n)
     void* const st = current_stream();
     const void *ap = A->const_data_ptr(), *gp = G->const_data_ptr();
     float* op = static_cast<float*>(o->data_ptr());
-    // Long fp32 calls above 64 x 64 can use a table of the projection; the rest would leave the scratch alone
-    // (bf16 rows of one layer go to the cluster kernel).
     at::Tensor scratch;
-    size_t wbytes = dt == GRASS_F32 && std::max(kin, kout) > 64 && B * T >= 8192 ? api.grouped_bytes(1) : 0;
+    size_t wbytes = api.layer_bytes((grass_dtype)dt, (int32_t)B, (int32_t)T, (int32_t)kin, (int32_t)kout, &sp);
     void* const wp = optional_scratch(&wbytes, &scratch);
     const factgrass_layer layer = {ap, gp, mi, mo, (int32_t)d_in, (int32_t)d_out, (int32_t)kin, (int32_t)kout, sp, 0};
     grass_status rc;
@@ -442,7 +440,7 @@ PyObject* py_bind(PyObject*, PyObject* const* a, Py_ssize_t n)
     }
     api.compress = (decltype(api.compress))p[0];
     api.compress_bytes = (decltype(api.compress_bytes))p[7];
-    api.grouped_bytes = (decltype(api.grouped_bytes))p[1];
+    api.layer_bytes = (decltype(api.layer_bytes))p[1];
     api.factgrass_varlen = (decltype(api.factgrass_varlen))p[2];
     api.grouped_out = (decltype(api.grouped_out))p[3];
     api.grouped_varlen = (decltype(api.grouped_varlen))p[4];

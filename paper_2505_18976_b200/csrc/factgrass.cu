@@ -332,6 +332,35 @@ static grass_status fill_desc(LayerDesc& d, const factgrass_layer& l, int tile, 
     return GRASS_OK;
 }
 
+// A share ends with a projection, so it wants a few 32-token steps: with fewer (layer, sample) items than SMs four
+// per SM (three up to 96 x 96, where the projection is half as long); measured in fp32, streaming -> persistent, 768 x
+// 3,072 at 128 x 128: 27.7 -> 28.8 us at 1.7 steps, 38.7 -> 40.5 at 3.5, 62.3 -> 61.7 at 6.9; at 72 x 72: 39.8 -> 33.7 at
+// 3.5.  With an item for every SM the streaming kernel projects as often, at four tiles per block, and the persistent
+// one is faster down to one step per item (16 layers of 16 x 32 tokens, 128 x 128 bf16: 75.5 -> 34.8 us).
+// bf16 (half the bytes, one accumulator) leaves the projection more of the time, and the streaming kernel is the faster one
+//  - for layers with a side of at most 64, two of its tiles instead of four, while there are fewer than two items per SM and
+//    two thread blocks with their bins fit the 64 KB that it gives to shared memory (248 items of 250 tokens, 96 x 48, k
+//    = 1,536: 33 us there, 46 here; 336 items: 104 and 59; 160 items, k = 4,096: 87 and 37), with up to 64 tokens for half
+//    an item more and with small k throughout (336 items of 33 tokens, 128 x 16, k = 1,024: 22.6 and 30.7; 720: 35 and 41);
+//  - for up to 64 tokens per item, small k and few more items than SMs (160 items of 16 tokens, k = 1,024, 128 x 128: 26.7 us
+//    there, 30.8 here; k = 1,536: 30.9 and 29.6; 216 items: 30.2 and 30.8).
+// fp32 is 1.1 to 3 times as fast here in all of these.
+// (wide: layers with both sides above 64)
+static bool persistent_pays(bool f32, int32_t L, int32_t B, int32_t T, int32_t max_kk, uint32_t max_k, int32_t wide, int sms)
+{
+    const int64_t items = (int64_t)L * B, steps = (T + kTokTile - 1) / kTokTile * items;
+    if (!f32) {
+        const bool brief = T <= 2 * kTokTile, small_k = max_k <= 1024;
+        if (2 * wide < L) {
+            if (max_k <= 3500 && 2 * items < (brief ? 5 : 4) * (int64_t)sms) return false;
+            if (brief && small_k) return false;
+        } else if (brief && small_k && 4 * items < 5 * (int64_t)sms) {
+            return false;
+        }
+    }
+    return max_kk > 64 && (items >= sms || steps >= (max_kk > 96 ? 4 : 3) * (int64_t)sms);
+}
+
 static grass_status run_factgrass(const factgrass_layer* layers, int32_t L, grass_dtype dt, int32_t B, int32_t T,
                                   const int64_t* tok_begin, const int32_t* tok_count, float* out, int64_t ld_out,
                                   void* workspace, size_t workspace_bytes, uint32_t* dev_status, cudaStream_t st,
@@ -412,36 +441,13 @@ static grass_status run_factgrass(const factgrass_layer* layers, int32_t L, gras
     // The table of the projections sits behind the descriptors where the workspace has room for it.
     const size_t table_off = ((size_t)L * sizeof(LayerDesc) + 255) / 256 * 256;
     void* const table = workspace && workspace_bytes >= table_off + persistent_table_bytes(L) ? (char*)workspace + table_off : nullptr;
-    // A share ends with a projection, so it wants a few 32-token steps: with fewer (layer, sample) items than SMs four
-    // per SM (three up to 96 x 96, where the projection is half as long); measured in fp32, streaming -> persistent, 768 x
-    // 3,072 at 128 x 128: 27.7 -> 28.8 us at 1.7 steps, 38.7 -> 40.5 at 3.5, 62.3 -> 61.7 at 6.9; at 72 x 72: 39.8 -> 33.7 at
-    // 3.5.  With an item for every SM the streaming kernel projects as often, at four tiles per block, and the persistent
-    // one is faster down to one step per item (16 layers of 16 x 32 tokens, 128 x 128 bf16: 75.5 -> 34.8 us).
-    // bf16 (half the bytes, one accumulator) leaves the projection more of the time, and the streaming kernel is the faster one
-    //  - for layers with a side of at most 64, two of its tiles instead of four, while there are fewer than two items per SM and
-    //    two thread blocks with their bins fit the 64 KB that it gives to shared memory (248 items of 250 tokens, 96 x 48, k
-    //    = 1,536: 33 us there, 46 here; 336 items: 104 and 59; 160 items, k = 4,096: 87 and 37), with up to 64 tokens for half
-    //    an item more and with small k throughout (336 items of 33 tokens, 128 x 16, k = 1,024: 22.6 and 30.7; 720: 35 and 41);
-    //  - for up to 64 tokens per item, small k and few more items than SMs (160 items of 16 tokens, k = 1,024, 128 x 128: 26.7 us
-    //    there, 30.8 here; k = 1,536: 30.9 and 29.6; 216 items: 30.2 and 30.8).
-    // fp32 is 1.1 to 3 times as fast here in all of these.
     auto persistent = [&](const LayerDesc* hd) {
         const int64_t forced = tuning(GRASS_TUNE_FACTGRASS_PATH, -1);
         if (epi != kEpiSjlt || out_bf16 || T <= 0 || !table || cluster_nc > 1 || !persistent_fits(hd, L, B, tok_count)) return false;
         if (forced != -1) return forced == 2;
-        const int64_t items = (int64_t)L * B, steps = (T + kTokTile - 1) / kTokTile * items;
-        if (!f32) {
-            int32_t wide = 0;
-            for (int l = 0; l < L; ++l) wide += std::min(hd[l].kin, hd[l].kout) > 64;
-            const bool brief = T <= 2 * kTokTile, small_k = max_k <= 1024;
-            if (2 * wide < L) {
-                if (max_k <= 3500 && 2 * items < (brief ? 5 : 4) * (int64_t)sms) return false;
-                if (brief && small_k) return false;
-            } else if (brief && small_k && 4 * items < 5 * (int64_t)sms) {
-                return false;
-            }
-        }
-        return max_kk > 64 && (items >= sms || steps >= (max_kk > 96 ? 4 : 3) * (int64_t)sms);
+        int32_t wide = 0;
+        for (int l = 0; l < L; ++l) wide += std::min(hd[l].kin, hd[l].kout) > 64;
+        return persistent_pays(f32, L, B, T, max_kk, max_k, wide, sms);
     };
 
     // a single layer travels as a kernel parameter: no descriptor copy, whoever provided a workspace
@@ -677,6 +683,25 @@ extern "C" grass_status factmask_compress_grouped(const factgrass_layer* layers,
     if (!workspace) return GRASS_ERR_INVALID_ARG;
     return grass::run_factmask(layers, L, dt, B, T, out, ld_out, workspace, workspace_bytes, dev_status,
                                (cudaStream_t)stream);
+}
+
+extern "C" size_t factgrass_compress_workspace_bytes(grass_dtype dt, int32_t B, int32_t T, int32_t kin, int32_t kout,
+                                                     const grass_sjlt_spec* spec)
+{
+    using namespace grass;
+    // bf16 rows of one layer go to the cluster kernel while they are few, and are not worth a table beyond that
+    if (dt != GRASS_F32 || B <= 0 || T <= 0 || !spec) return 0;
+    LayerDesc d;
+    std::memset(&d, 0, sizeof d);
+    d.kin = kin;
+    d.kout = kout;
+    d.k = spec->k;
+    d.s = spec->s;
+    int dev = 0, sms = 148;
+    if (cuda_failed(cudaGetDevice(&dev)) || cuda_failed(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev))) return 0;
+    const bool pays = persistent_fits(&d, 1, B, nullptr) &&
+                      persistent_pays(true, 1, B, T, std::max(kin, kout), d.k, std::min(kin, kout) > 64, sms);
+    return pays ? factgrass_grouped_workspace_bytes(1) : 0;
 }
 
 extern "C" size_t factgrass_grouped_workspace_bytes(int32_t L)

@@ -1,5 +1,7 @@
 """The compiled marshalling of the binding against the ctypes code it stands in for: same results, same exceptions,
 and no verdict of its own on operands that are out of the ordinary."""
+import ctypes
+
 import pytest
 import torch
 
@@ -105,3 +107,19 @@ def test_calls_do_without_the_scratch_that_they_cannot_have(no_more_memory):
     no_more_memory()
     assert G.grass_compress(g, None, k, 1, 0, out=out) is out
     assert torch.equal(out, want)      # sums of ones, exact in any order
+
+
+@pytest.mark.parametrize("n,T", [(150, 40), (40, 500)])
+def test_single_fp32_layers_get_the_table_where_the_library_would_use_it(n, T, monkeypatch):
+    """An item for every SM, and steps for every SM; against the ctypes code, which hands over no scratch."""
+    gen = torch.Generator("cuda").manual_seed(2)
+    A, Gr = (torch.randn((n, T, d), generator=gen, device="cuda") for d in (200, 150))
+    mi, mo = (G.mask_to_device(G.grass_random_mask_host(d, 100, s)) for d, s in ((200, 2), (150, 3)))
+    spec = B.SjltSpec(4_096, 1, 9)
+    scratch = lambda rows: G.lib().factgrass_compress_workspace_bytes(B.F32, rows, T, 100, 100, ctypes.byref(spec))  # noqa: E731
+    assert scratch(n) > 0 and scratch(4) == 0
+    fast = G.factgrass_compress(A, Gr, mi, mo, 4_096, 1, 9)
+    monkeypatch.setattr(B, "_fast", lambda: _Declines())
+    slow = G.factgrass_compress(A, Gr, mi, mo, 4_096, 1, 9)
+    # sums of T products of two unit normals, 10,000 / 4,096 of them per bin, in two orders of fp32 additions
+    assert (fast - slow).abs().max() <= 64 * 2.0 ** -24 * T ** 0.5 * float(slow.abs().max())
