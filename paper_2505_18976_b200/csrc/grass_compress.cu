@@ -45,7 +45,7 @@ __device__ __forceinline__ void load4(const __nv_bfloat16* p, float (&v)[4])
 
 // DENSE: identity mask on vector-aligned rows (plain SJLT, the k' = p case of Section 3.3.1).  Rows are then
 // streamed with vector loads, four consecutive positions per thread, and S > 1 samples share each hash.
-// NT: threads per CTA (the gather path runs with 256 or 512; the streamed path always with kThreads).
+// NT: threads per CTA (the gather path runs with 256, 512 or 1,024; the streamed path always with kThreads).
 template <typename T, int S, int U, bool S1, bool DENSE, int NT>
 __global__ void __launch_bounds__(NT, DENSE ? 4 : (U >= 16 ? 1024 : 2048) / NT)
 grass_compress_kernel(const T* __restrict__ g, int64_t n, int64_t p, int64_t ld,
@@ -346,7 +346,7 @@ struct CompressPlan {
     int cluster;    // the jsplit CTAs are one thread-block cluster (DSMEM reduction)
     int out_bf16;   // rows are stored as bf16 (final store only)
     uint32_t idx_smem;  // bytes of shared memory for a copy of the index list (0: indices are read from global memory)
-    int threads;    // threads per CTA of the gather path (256 or 512)
+    int threads;    // threads per CTA of the gather path (256, 512 or 1,024)
     int U;          // gathered loads in flight per thread and sample
 };
 

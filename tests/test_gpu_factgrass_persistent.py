@@ -33,7 +33,7 @@ def _compare(layers, dtype, B, T, lens, path):
         keep.append((A, Gr, mi, mo, kin, kout, k, off))
         off += k
     out = torch.full((B, off), float("nan"), device="cuda")
-    ws = torch.empty(G.factgrass_grouped_workspace_bytes(len(layers)), dtype=torch.uint8, device="cuda")
+    ws = torch.full((G.factgrass_grouped_workspace_bytes(len(layers)),), 0xA5, dtype=torch.uint8, device="cuda")
     st = torch.zeros(1, dtype=torch.int32, device="cuda")
     with G.tuning(factgrass_path=path):
         if lens is None:
@@ -43,6 +43,9 @@ def _compare(layers, dtype, B, T, lens, path):
                                                 tok_count=torch.tensor(lengths).cuda(), dev_status=st)
         torch.cuda.synchronize()
     assert int(st.item()) == 0
+    # this kernel, and no other, writes the tables of the projections: 128 x 128 entries of 16 bits per layer, behind the descriptors
+    tables = ws[ws.numel() - len(layers) * 2 * 128 * 128:].view(len(layers), -1)
+    assert (tables != 0xA5).any(dim=1).all(), "another kernel took the call"
     host = out.cpu().numpy()
     for n, (A, Gr, mi, mo, kin, kout, k, o) in enumerate(keep):
         ref, absum = oracle.factgrass_varlen(W.bits_of(A), W.bits_of(Gr), mi, mo, k, 1, n + 5, begin, lengths, dtype=name)
