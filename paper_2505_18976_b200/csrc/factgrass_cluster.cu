@@ -455,7 +455,7 @@ int cluster_capacity(int nc)
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     int count = 0;
-    if (cuda_failed(cudaOccupancyMaxActiveClusters(&count, kern, &cfg))) count = 0;
+    if (cuda_failed(cudaOccupancyMaxActiveClusters(&count, kern, &cfg))) return 0;      // not kept: the next call asks again
     cell.store(count + 1, std::memory_order_relaxed);
     return count;
 }
