@@ -16,7 +16,8 @@
 // delivers (128 + M / 2) rows per block and 64 k-values, hence the 256-row pairs and a tile as wide as the test set.  One
 // turn of the issuing threads (wait, expect, load; wait, multiply, commit) takes 600 cycles whatever it moves, 16 KB of
 // train rows a turn are then 3.7-4.8 TB/s over the chip and 32 KB 6.7: stages of 128 k-values wherever three of them fit.
-// Measured (before: 256-column pairs for M > 256, one block per 128 rows for M <= 256): 4,656 x 300 x 49,152 285 -> 138 us,
+// Measured (before: 256-column pairs for M > 256, one block per 128 rows for M <= 256): 4,656 x 300 x 49,152 285 -> 138 us on
+// a cool chip (164 in a loop that the power cap holds),
 // 16,384 x 256 x 16,384 148 -> 128 us, 16,384 x 256 x 4,096 46 -> 42 us, 3,854 x 4 x 55,512 127 -> 83 us (5.2 TB/s).
 //   warp 0-3  drain the accumulator, warp 4 allocates tensor memory and issues the MMAs (leader), warp 5 issues the loads
 // Every mbarrier wait is bounded; a block whose wait expires marks its part with NaN and still reaches the cluster barrier.

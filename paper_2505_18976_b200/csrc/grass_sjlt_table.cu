@@ -7,9 +7,10 @@
 //   share a chunk of the table.  31 warps walk the chunk 128 positions at a time and add the non-zero values into k bins
 //   per row in shared memory; the cost of that follows the non-zeros (Section 3.1).  The (rows, chunk) units are cut
 //   evenly over the blocks, so there is no last wave; a row that two blocks share is added into zeroes.
-// What bounds it: the shared-memory fp32 atomics (13.5 cycles per warp with every lane active, 6.2 at 30 %, 3.5 at 10 %,
-// against 5.9 in which HBM delivers 32 fp32 values) for dense inputs, HBM for sparse ones.
-// 1,024 x 131,072, k = 4,096, against the streamed path: fp32 230 -> 150 us at 70 % zeros, 109 -> 97 at 99 % (5.5 TB/s);
+// What bounds it: for dense inputs the shared-memory fp32 additions, each a compare-and-swap; HBM for sparse ones (99 % zeros: 5.5
+// TB/s).  Between the two neither accounts for all of the time: at 70 % zeros HBM needs 86 of 154 us and the additions, at the
+// rate that a kernel of nothing else showed, 89, and the rows and the table pass through the same shared memory.
+// 1,024 x 131,072, k = 4,096, against the streamed path: fp32 230 -> 154 us at 70 % zeros, 109 -> 97 at 99 %;
 // bf16 303 -> 139; k = 32,768 615 -> 202.
 // (Turning the projection around instead, lists of positions per bucket summed without atomics, was built and measured:
 // its 16-bit lists cost 30 instructions per 32 buckets and chunk and it ran at 260 us whatever the sparsity.)
