@@ -68,6 +68,27 @@ __device__ __forceinline__ uint16_t gather_u16(const uint16_t* p)
 __device__ __forceinline__ float elem_value(float x) { return x; }
 __device__ __forceinline__ float elem_value(__nv_bfloat16 x) { return __bfloat162float(x); }
 
+// A kernel that is launched as a programmatic dependent (early_launch) starts while the kernel before it in the stream still
+// runs.  Before early_wait() it touches nothing but its own shared memory; early_go() lets the next one in.  (A kernel that reads before it waits, behind a set-up kernel of its own call, relies on that
+// one to be launched the ordinary way.)
+__device__ __forceinline__ void early_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// an address that is not known before early_wait(): read-only loads through it stay behind the wait, which the compiler would
+// otherwise be free to pass with them
+template <typename T>
+__device__ __forceinline__ T* waited(T* p)
+{
+    asm volatile("" : "+l"(p)::"memory");
+    return p;
+}
+__device__ __forceinline__ void early_go() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+inline cudaLaunchAttribute early_launch()
+{
+    cudaLaunchAttribute a;
+    a.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    a.val.programmaticStreamSerializationAllowed = 1;
+    return a;
+}
+
 // final store of a compressed value: fp32, or bf16 rounded to nearest even (a cache of compressed vectors kept
 // at half the size; everything before the store is fp32)
 __device__ __forceinline__ void store_out(float* out, int64_t off, float v, int out_bf16)

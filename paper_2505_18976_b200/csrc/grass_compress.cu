@@ -48,8 +48,8 @@ __device__ __forceinline__ void load4(const __nv_bfloat16* p, float (&v)[4])
 // NT: threads per CTA (the gather path runs with 256, 512 or 1,024; the streamed path always with kThreads).
 template <typename T, int S, int U, bool S1, bool DENSE, int NT>
 __global__ void __launch_bounds__(NT, DENSE ? 4 : (U >= 16 ? 1024 : 2048) / NT)
-grass_compress_kernel(const T* __restrict__ g, int64_t n, int64_t p, int64_t ld,
-                      const uint32_t* __restrict__ idx, int64_t kprime, uint32_t k, uint32_t s,
+grass_compress_kernel(const T* g, int64_t n, int64_t p, int64_t ld,
+                      const uint32_t* idx, int64_t kprime, uint32_t k, uint32_t s,
                       uint64_t seed, float scale, float* __restrict__ out, int64_t ld_out,
                       int64_t j_per_cta, int accumulate, int use_smem, uint32_t* dev_status, int out_bf16,
                       uint32_t idx_smem_bytes)
@@ -70,16 +70,22 @@ grass_compress_kernel(const T* __restrict__ g, int64_t n, int64_t p, int64_t ld,
     uint32_t* sidx = reinterpret_cast<uint32_t*>(bins + (use_smem ? ((size_t)S * k + 3) / 4 * 4 : 0));
     const uint32_t idx_bulk = idx_smem_bytes ? (uint32_t)((kprime * 4) & ~(int64_t)15) : 0u;
     if (idx_smem_bytes && tid == 0) {
-        const uint32_t bar = tc::smem_u32(&idx_bar);
-        tc::mbar_init(bar, 1);
+        tc::mbar_init(tc::smem_u32(&idx_bar), 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        if (idx_bulk > 0) {
-            tc::expect_tx(bar, idx_bulk);
-            tc::bulk_copy(tc::smem_u32(sidx), idx, idx_bulk, bar);
-        }
     }
+    // The launch and the zeroing lie under the end of the kernel before (calls one after the other: one row of k' = 8,192 6.15 ->
+    // 4.72 us, 256 rows 16.1 -> 15.0).
     if (use_smem)
         for (uint32_t i = tid; i < (uint32_t)S * k; i += nthr) bins[i] = 0.0f;
+    early_wait();
+    early_go();
+    g = waited(g);
+    idx = waited(idx);
+    if (idx_bulk > 0 && tid == 0) {
+        const uint32_t bar = tc::smem_u32(&idx_bar);
+        tc::expect_tx(bar, idx_bulk);
+        tc::bulk_copy(tc::smem_u32(sidx), idx, idx_bulk, bar);
+    }
     if (idx_smem_bytes)
         for (int64_t j = idx_bulk / 4 + tid; j < kprime; j += nthr) sidx[j] = __ldg(idx + j);   // at most 3 entries
     if (use_smem || idx_smem_bytes) __syncthreads();
@@ -457,15 +463,17 @@ static grass_status launch_compress(const T* g, int64_t n, int64_t p, int64_t ld
         cfg.blockDim = dim3((unsigned)(pl.dense ? kThreads : pl.threads), 1, 1);
         cfg.dynamicSmemBytes = smem;
         cfg.stream = st;
-        cudaLaunchAttribute attr[1];
+        cudaLaunchAttribute attr[2];
+        cfg.attrs = attr;
+        cfg.numAttrs = 0;
         if (pl.cluster) {
-            attr[0].id = cudaLaunchAttributeClusterDimension;
-            attr[0].val.clusterDim.x = 1;
-            attr[0].val.clusterDim.y = (unsigned)pl.jsplit;
-            attr[0].val.clusterDim.z = 1;
-            cfg.attrs = attr;
-            cfg.numAttrs = 1;
+            cudaLaunchAttribute& a = attr[cfg.numAttrs++];
+            a.id = cudaLaunchAttributeClusterDimension;
+            a.val.clusterDim.x = 1;
+            a.val.clusterDim.y = (unsigned)pl.jsplit;
+            a.val.clusterDim.z = 1;
         }
+        if (accumulate != 1) attr[cfg.numAttrs++] = early_launch();        // (else a memset comes before)
         const int use_smem = pl.use_smem;
         cudaError_t e = cudaLaunchKernelEx(&cfg, kern, g, n, p, ld, idx, kprime, sp.k, sp.s, sp.seed, scale, out,
                                            ld_out, j_per_cta, accumulate, use_smem, dev_status, pl.out_bf16, pl.idx_smem);

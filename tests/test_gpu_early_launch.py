@@ -1,0 +1,87 @@
+"""Kernels that start while the kernel before them still runs: what that one writes is read complete, and what it reads is not
+overwritten; on a stream, and recorded into a graph behind every kind of node."""
+import pytest
+import torch
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def G():
+    import paper_2505_18976_b200 as g
+    g.lib()
+    return g
+
+
+def _calls(G):
+    """Each writes its input, runs a call on it and returns the result; the second argument counts up."""
+    g = torch.randn((64, 65_536), device="cuda")
+    idx = G.mask_to_device(G.grass_random_mask_host(65_536, 8_192, 3))
+    few = G.mask_to_device(G.grass_random_mask_host(65_536, 1_024, 4))
+    A = torch.randn((4, 96, 200), device="cuda").to(torch.bfloat16)
+    Gr = torch.randn((4, 96, 300), device="cuda").to(torch.bfloat16)
+    mi, mo = (G.mask_to_device(G.grass_random_mask_host(d, 64, d)) for d in (200, 300))
+
+    def clusters():
+        g.neg_()
+        return G.grass_compress(g[:3], idx, 2_048, 1, 5)
+
+    def rows():
+        g.neg_()
+        return G.grass_compress(g, few, 512, 1, 5)
+
+    def dense():
+        g.neg_()
+        return G.grass_compress(g[:4], None, 2_048, 1, 5)
+
+    def layer():
+        A.neg_()
+        return G.factgrass_compress(A, Gr, mi, mo, 1_024, 1, 5)
+
+    return dict(clusters=clusters, rows=rows, dense=dense, layer=layer)
+
+
+# sums in another order: at most some tens of fp32 additions per value
+def _same(a, b):
+    return (a - b).abs().max() <= 2.0 ** -18 * b.abs().max()
+
+
+@pytest.mark.parametrize("name", ["clusters", "rows", "dense", "layer"])
+def test_chained_calls_read_finished_inputs(G, name):
+    call = _calls(G)[name]
+    outs = [call() for _ in range(60)]
+    torch.cuda.synchronize()
+    for i, o in enumerate(outs):
+        assert _same(o if i % 2 == 0 else -o, outs[0]), i
+
+
+@pytest.mark.parametrize("before", ["nothing", "kernel", "copy", "download", "fill", "join", "call"])
+def test_recorded_behind_any_node(G, before):
+    g = torch.randn((64, 65_536), device="cuda")
+    idx = G.mask_to_device(G.grass_random_mask_host(65_536, 8_192, 3))
+    ref = G.grass_compress(g, idx, 2_048, 1, 5)
+    x, y, host = torch.zeros(1_000, device="cuda"), torch.empty(1_000, device="cuda"), torch.empty(1_000).pin_memory()
+    main, side = torch.cuda.Stream(), torch.cuda.Stream()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=main):
+        if before == "kernel":
+            x.add_(1)
+        elif before == "copy":
+            y.copy_(x)
+        elif before == "download":
+            host.copy_(x, non_blocking=True)
+        elif before == "fill":
+            x.zero_()
+        elif before == "join":
+            side.wait_stream(main)
+            with torch.cuda.stream(side):
+                x.add_(1)
+            y.add_(1)
+            main.wait_stream(side)
+        elif before == "call":
+            G.grass_compress(g, idx, 2_048, 1, 5)
+        out = G.grass_compress(g, idx, 2_048, 1, 5)
+    for _ in range(3):
+        graph.replay()
+    torch.cuda.synchronize()
+    assert _same(out, ref)
