@@ -495,7 +495,12 @@ grass_status launch_factgrass_cluster(const LayerDesc* dev_descs, const LayerDes
         attr[0].val.clusterDim.z = 1;
         attr[1] = early_launch();
         cfg.attrs = attr;
-        cfg.numAttrs = dev_descs ? 1 : 2;                  // (a descriptor table is copied to the device just before)
+        // not behind the copy of a descriptor table, and not with more than one thread block per SM: the next call's would take the
+        // places that are left and be spread unevenly
+        int dev = 0, sms = 0;
+        if (cuda_failed(cudaGetDevice(&dev)) || cuda_failed(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)))
+            return GRASS_ERR_CUDA;
+        cfg.numAttrs = !dev_descs && (int64_t)nc * B * L <= sms ? 2 : 1;
         cudaError_t e = cudaLaunchKernelEx(&cfg, kern, dev_descs, single, T, tok_begin, tok_count, chunk_len, out,
                                            ld_out, dev_status, out_bf16);
         return cuda_ok(e);

@@ -72,14 +72,15 @@ __device__ __forceinline__ float elem_value(__nv_bfloat16 x) { return __bfloat16
 // runs.  Before early_wait() it touches nothing but its own shared memory; early_go() lets the next one in.  (A kernel that reads before it waits, behind a set-up kernel of its own call, relies on that
 // one to be launched the ordinary way.)
 __device__ __forceinline__ void early_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-// an address that is not known before early_wait(): read-only loads through it stay behind the wait, which the compiler would
-// otherwise be free to pass with them
+// A value that is not known before early_wait(): read-only loads from addresses that depend on it stay behind the wait, which the
+// compiler would otherwise be free to pass with them.
 template <typename T>
 __device__ __forceinline__ T* waited(T* p)
 {
     asm volatile("" : "+l"(p)::"memory");
     return p;
 }
+__device__ __forceinline__ void waited(int& x) { asm volatile("" : "+r"(x)::"memory"); }
 __device__ __forceinline__ void early_go() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 inline cudaLaunchAttribute early_launch()
 {

@@ -48,14 +48,14 @@ __device__ __forceinline__ void load4(const __nv_bfloat16* p, float (&v)[4])
 // NT: threads per CTA (the gather path runs with 256, 512 or 1,024; the streamed path always with kThreads).
 template <typename T, int S, int U, bool S1, bool DENSE, int NT>
 __global__ void __launch_bounds__(NT, DENSE ? 4 : (U >= 16 ? 1024 : 2048) / NT)
-grass_compress_kernel(const T* g, int64_t n, int64_t p, int64_t ld,
-                      const uint32_t* idx, int64_t kprime, uint32_t k, uint32_t s,
+grass_compress_kernel(const T* __restrict__ g, int64_t n, int64_t p, int64_t ld,
+                      const uint32_t* __restrict__ idx, int64_t kprime, uint32_t k, uint32_t s,
                       uint64_t seed, float scale, float* __restrict__ out, int64_t ld_out,
                       int64_t j_per_cta, int accumulate, int use_smem, uint32_t* dev_status, int out_bf16,
                       uint32_t idx_smem_bytes)
 {
     extern __shared__ float bins[];  // S * k when use_smem
-    const int tid = threadIdx.x;
+    int tid = threadIdx.x;
     constexpr int nthr = NT;
     static_assert(!DENSE || NT == kThreads, "the streamed path is written for kThreads threads");
     const int64_t i0 = (int64_t)blockIdx.x * S;
@@ -69,23 +69,25 @@ grass_compress_kernel(const T* g, int64_t n, int64_t p, int64_t ld,
     __shared__ __align__(8) unsigned long long idx_bar;
     uint32_t* sidx = reinterpret_cast<uint32_t*>(bins + (use_smem ? ((size_t)S * k + 3) / 4 * 4 : 0));
     const uint32_t idx_bulk = idx_smem_bytes ? (uint32_t)((kprime * 4) & ~(int64_t)15) : 0u;
-    if (idx_smem_bytes && tid == 0) {
-        tc::mbar_init(tc::smem_u32(&idx_bar), 1);
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    // The launch lies under the end of the kernel before (calls one after the other: one row of k' = 8,192 6.15 -> 4.96 us, 256 rows
+    // 16.1 -> 15.1).  Zeroing the bins ahead of the wait as well gained another 0.1 us there, but cost registers that the bf16
+    // gathers do not have (61 rows of k' = 32,768: 32.0 us, 33.9 so).  Behind a memset there is nothing to wait for.
+    if (accumulate != 1) {
+        early_wait();
+        early_go();
     }
-    // The launch and the zeroing lie under the end of the kernel before (calls one after the other: one row of k' = 8,192 6.15 ->
-    // 4.72 us, 256 rows 16.1 -> 15.0).
+    waited(tid);               // every address below depends on it
+    if (idx_smem_bytes && tid == 0) {
+        const uint32_t bar = tc::smem_u32(&idx_bar);
+        tc::mbar_init(bar, 1);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        if (idx_bulk > 0) {
+            tc::expect_tx(bar, idx_bulk);
+            tc::bulk_copy(tc::smem_u32(sidx), idx, idx_bulk, bar);
+        }
+    }
     if (use_smem)
         for (uint32_t i = tid; i < (uint32_t)S * k; i += nthr) bins[i] = 0.0f;
-    early_wait();
-    early_go();
-    g = waited(g);
-    idx = waited(idx);
-    if (idx_bulk > 0 && tid == 0) {
-        const uint32_t bar = tc::smem_u32(&idx_bar);
-        tc::expect_tx(bar, idx_bulk);
-        tc::bulk_copy(tc::smem_u32(sidx), idx, idx_bulk, bar);
-    }
     if (idx_smem_bytes)
         for (int64_t j = idx_bulk / 4 + tid; j < kprime; j += nthr) sidx[j] = __ldg(idx + j);   // at most 3 entries
     if (use_smem || idx_smem_bytes) __syncthreads();
@@ -354,12 +356,14 @@ struct CompressPlan {
     uint32_t idx_smem;  // bytes of shared memory for a copy of the index list (0: indices are read from global memory)
     int threads;    // threads per CTA of the gather path (256, 512 or 1,024)
     int U;          // gathered loads in flight per thread and sample
+    int sms;
 };
 
 static CompressPlan plan_compress(int64_t n, int64_t p, int64_t kprime, uint32_t k, int sm_count, bool dense)
 {
     CompressPlan pl;
     pl.dense = dense;
+    pl.sms = sm_count;
     const size_t bin_bytes = (size_t)k * sizeof(float);
     const size_t smem_cap = 200 * 1024;
     pl.use_smem = bin_bytes <= smem_cap;
@@ -473,7 +477,9 @@ static grass_status launch_compress(const T* g, int64_t n, int64_t p, int64_t ld
             a.val.clusterDim.y = (unsigned)pl.jsplit;
             a.val.clusterDim.z = 1;
         }
-        if (accumulate != 1) attr[cfg.numAttrs++] = early_launch();        // (else a memset comes before)
+        // Not behind a memset, and not where the blocks of split rows fill more than one place per SM: the next call's then take
+        // the places that are left, and are spread unevenly (42 rows of k' = 49,677, 336 blocks: 30.9 us a call, 32.7 so)
+        if (accumulate != 1 && (pl.jsplit == 1 || groups * pl.jsplit <= pl.sms)) attr[cfg.numAttrs++] = early_launch();
         const int use_smem = pl.use_smem;
         cudaError_t e = cudaLaunchKernelEx(&cfg, kern, g, n, p, ld, idx, kprime, sp.k, sp.s, sp.seed, scale, out,
                                            ld_out, j_per_cta, accumulate, use_smem, dev_status, pl.out_bf16, pl.idx_smem);
