@@ -71,11 +71,9 @@ grass_compress_kernel(const T* __restrict__ g, int64_t n, int64_t p, int64_t ld,
     const uint32_t idx_bulk = idx_smem_bytes ? (uint32_t)((kprime * 4) & ~(int64_t)15) : 0u;
     // The launch lies under the end of the kernel before (calls one after the other: one row of k' = 8,192 6.15 -> 4.96 us, 256 rows
     // 16.1 -> 15.1).  Zeroing the bins ahead of the wait as well gained another 0.1 us there, but cost registers that the bf16
-    // gathers do not have (61 rows of k' = 32,768: 32.0 us, 33.9 so).  Behind a memset there is nothing to wait for.
-    if (accumulate != 1) {
-        early_wait();
-        early_go();
-    }
+    // gathers do not have (61 rows of k' = 32,768: 32.0 us, 33.9 so).
+    early_wait();
+    early_go();
     waited(tid);               // every address below depends on it
     if (idx_smem_bytes && tid == 0) {
         const uint32_t bar = tc::smem_u32(&idx_bar);
@@ -477,9 +475,10 @@ static grass_status launch_compress(const T* g, int64_t n, int64_t p, int64_t ld
             a.val.clusterDim.y = (unsigned)pl.jsplit;
             a.val.clusterDim.z = 1;
         }
-        // Not behind a memset, and not where the blocks of split rows fill more than one place per SM: the next call's then take
-        // the places that are left, and are spread unevenly (42 rows of k' = 49,677, 336 blocks: 30.9 us a call, 32.7 so)
-        if (accumulate != 1 && (pl.jsplit == 1 || groups * pl.jsplit <= pl.sms)) attr[cfg.numAttrs++] = early_launch();
+        // Not where clusters fill more than one place per SM: the next call's then take the places that are left, and are spread
+        // unevenly (42 rows of k' = 49,677, 336 blocks: 30.9 us a call, 32.7 so).  The wide splits have a memset between them
+        // (4 rows of k' = 44,531: 11.1 -> 8.2 us).
+        if (accumulate == 1 || (pl.jsplit == 1 || groups * pl.jsplit <= pl.sms)) attr[cfg.numAttrs++] = early_launch();
         const int use_smem = pl.use_smem;
         cudaError_t e = cudaLaunchKernelEx(&cfg, kern, g, n, p, ld, idx, kprime, sp.k, sp.s, sp.seed, scale, out,
                                            ld_out, j_per_cta, accumulate, use_smem, dev_status, pl.out_bf16, pl.idx_smem);

@@ -20,6 +20,8 @@ def _calls(G):
     few = G.mask_to_device(G.grass_random_mask_host(65_536, 1_024, 4))
     A = torch.randn((4, 96, 200), device="cuda").to(torch.bfloat16)
     Gr = torch.randn((4, 96, 300), device="cuda").to(torch.bfloat16)
+    wide_g = torch.randn((2, 600_001), device="cuda")
+    wide_idx = G.mask_to_device(G.grass_random_mask_host(600_001, 110_000, 6))
     mi, mo = (G.mask_to_device(G.grass_random_mask_host(d, 64, d)) for d in (200, 300))
 
     def clusters():
@@ -30,6 +32,10 @@ def _calls(G):
         g.neg_()
         return G.grass_compress(g, few, 512, 1, 5)
 
+    def wide():                # zeroed by a memset, then added into by more blocks than a cluster has
+        wide_g.neg_()
+        return G.grass_compress(wide_g, wide_idx, 1_024, 1, 5)
+
     def dense():
         g.neg_()
         return G.grass_compress(g[:4], None, 2_048, 1, 5)
@@ -38,7 +44,17 @@ def _calls(G):
         A.neg_()
         return G.factgrass_compress(A, Gr, mi, mo, 1_024, 1, 5)
 
-    return dict(clusters=clusters, rows=rows, dense=dense, layer=layer)
+    train, test = torch.randn((300, 520), device="cuda"), torch.randn((40, 520), device="cuda")
+
+    def score():
+        train.neg_()
+        return G.grass_score(train, test)
+
+    def score_bf16():
+        train.neg_()
+        return G.grass_score_bf16(train.to(torch.bfloat16), test.to(torch.bfloat16))
+
+    return dict(clusters=clusters, rows=rows, wide=wide, dense=dense, layer=layer, score=score, score_bf16=score_bf16)
 
 
 # sums in another order: at most some tens of fp32 additions per value
@@ -46,7 +62,7 @@ def _same(a, b):
     return (a - b).abs().max() <= 2.0 ** -18 * b.abs().max()
 
 
-@pytest.mark.parametrize("name", ["clusters", "rows", "dense", "layer"])
+@pytest.mark.parametrize("name", ["clusters", "rows", "wide", "dense", "layer", "score", "score_bf16"])
 def test_chained_calls_read_finished_inputs(G, name):
     call = _calls(G)[name]
     outs = [call() for _ in range(60)]
@@ -85,3 +101,16 @@ def test_recorded_behind_any_node(G, before):
         graph.replay()
     torch.cuda.synchronize()
     assert _same(out, ref)
+
+
+@pytest.mark.parametrize("name", ["clusters", "wide", "dense", "layer", "score", "score_bf16"])
+def test_recorded_calls(G, name):
+    call = _calls(G)[name]
+    ref = call()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        outs = [call(), call()]
+    for _ in range(3):
+        graph.replay()
+    torch.cuda.synchronize()
+    assert _same(outs[1], ref) and _same(-outs[0], ref)
