@@ -113,6 +113,8 @@ score_bf16_kernel(const __grid_constant__ CUtensorMap map_train, const __grid_co
     __syncthreads();
     cluster_sync_all();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    early_wait();                  // (launch and set-up lie under the end of the kernel before)
+    early_go();
     const uint32_t tmem_d = tmem_base_slot;
     const uint32_t smem_base = smem_u32(smem);
 
@@ -307,9 +309,15 @@ grass_status launch_score_bf16(const void* train, int64_t N, int64_t ld_train, c
     auto launch = [&](auto kern) -> grass_status {
         if (cuda_failed(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BUDGET + SCRATCH_BYTES)))
             return GRASS_ERR_CUDA;
-        kern<<<(unsigned)(2 * used), THREADS_H, (size_t)p.stages * stage_bytes + SCRATCH_BYTES, st>>>(map_train, map_test, p, N, M, scores, ld_s,
-                                                                                      out_vec);
-        return launch_status();
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3((unsigned)(2 * used), 1, 1);
+        cfg.blockDim = dim3(THREADS_H, 1, 1);
+        cfg.dynamicSmemBytes = (size_t)p.stages * stage_bytes + SCRATCH_BYTES;
+        cfg.stream = st;
+        cudaLaunchAttribute attr[1] = {early_launch()};
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        return cuda_ok(cudaLaunchKernelEx(&cfg, kern, map_train, map_test, p, N, M, scores, ld_s, out_vec));
     };
     if (kw == 2) return subs == 2 ? launch(score_bf16_kernel<2, 2>) : launch(score_bf16_kernel<2, 1>);
     return subs == 2 ? launch(score_bf16_kernel<1, 2>) : launch(score_bf16_kernel<1, 1>);

@@ -113,6 +113,8 @@ grass_score_tc_kernel(const __grid_constant__ CUtensorMap map_train, const __gri
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     cluster_sync_all();            // both blocks' barriers are initialised before anybody arrives remotely
+    early_wait();                  // (launch and set-up lie under the end of the kernel before)
+    early_go();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem_d = tmem_base_slot;
     const uint32_t smem_base = smem_u32(smem);
@@ -346,9 +348,15 @@ grass_status launch_score_tc(const float* train, int64_t N, int64_t ld_train, co
     const int out_vec_ok = ((uintptr_t)scores % 16 == 0) && (ld_s % 4 == 0);
     int nprod = (int)tuning(GRASS_TUNE_SPLIT_PRODUCTS, tc::kSplitProductsDefault);
     if (nprod != 3 && nprod != 4) nprod = 6;
-    tc::grass_score_tc_kernel<<<(unsigned)(2 * used), tc::THREADS, smem, st>>>(map_train, map_test, p, N, M, scores, ld_s, out_vec_ok,
-                                                                              nprod);
-    return launch_status();
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(2 * used), 1, 1);
+    cfg.blockDim = dim3(tc::THREADS, 1, 1);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1] = {early_launch()};
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cuda_ok(cudaLaunchKernelEx(&cfg, tc::grass_score_tc_kernel, map_train, map_test, p, N, M, scores, ld_s, out_vec_ok, nprod));
 }
 
 }  // namespace grass
