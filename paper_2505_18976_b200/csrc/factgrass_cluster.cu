@@ -148,7 +148,6 @@ factgrass_cluster_kernel(const LayerDesc* __restrict__ descs, const __grid_const
     // The launch lies under the end of the kernel before (32 x 512 tokens, 768 x 3,072, 128 x 128, calls one after the other: 28.2 ->
     // 26.7 us).
     early_wait();
-    early_go();
     const LayerDesc& L = descs ? descs[blockIdx.z] : single;
     const int b = blockIdx.y;
     const int kin = L.kin, kout = L.kout;
@@ -196,6 +195,7 @@ factgrass_cluster_kernel(const LayerDesc* __restrict__ descs, const __grid_const
     for (uint32_t i = tid; i < k; i += kFgThreads) bins[i] = 0.0f;
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
+    early_go();                                           // (this block has its tensor memory)
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem_d = tmem_slot;
 

@@ -69,8 +69,12 @@ __device__ __forceinline__ float elem_value(float x) { return x; }
 __device__ __forceinline__ float elem_value(__nv_bfloat16 x) { return __bfloat162float(x); }
 
 // A kernel that is launched as a programmatic dependent (early_launch) starts while the kernel before it in the stream still
-// runs.  Before early_wait() it touches nothing but its own shared memory; early_go() lets the next one in.  (A kernel that reads before it waits, behind a set-up kernel of its own call, relies on that
-// one to be launched the ordinary way.)
+// runs.  Before early_wait() it touches nothing but its own shared memory and takes no tensor memory; early_go() lets the next
+// one in, and comes after the barrier behind the thread block's own tcgen05.alloc.  The order matters on both sides: an
+// allocation waits, without a limit, for columns that another thread block of the SM holds, and that one may be a successor that
+// waits for this grid to end.  The successor may also be another program's, with rules of its own.
+// (A kernel that reads before it waits, behind a set-up kernel of its own call, relies on that one to be launched the ordinary
+// way, and to need no tensor memory.)
 __device__ __forceinline__ void early_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 // A value that is not known before early_wait(): read-only loads from addresses that depend on it stay behind the wait, which the
 // compiler would otherwise be free to pass with them.

@@ -104,17 +104,19 @@ grass_score_tc_kernel(const __grid_constant__ CUtensorMap map_train, const __gri
         abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
+    __syncwarp();
+    cluster_sync_all();            // both blocks' barriers are initialised before anybody arrives remotely
+    early_wait();                  // (launch and set-up lie under the end of the kernel before)
     if (warp == PWARPS) {
         asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base_slot)),
                      "r"(TMEM_COLS)
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
     }
+    // (what the other block has allocated the MMAs touch only after its operands, which come after this barrier there)
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
-    cluster_sync_all();            // both blocks' barriers are initialised before anybody arrives remotely
-    early_wait();                  // (launch and set-up lie under the end of the kernel before)
-    early_go();
+    early_go();                    // (this block has its tensor memory)
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem_d = tmem_base_slot;
     const uint32_t smem_base = smem_u32(smem);
