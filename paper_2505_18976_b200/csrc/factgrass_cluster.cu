@@ -408,6 +408,8 @@ static size_t cluster_smem_bytes(int tile, uint32_t max_k)
     const size_t recv_bins = ((size_t)max_k + 8) * sizeof(float);       // NC * ceil(k / NC) <= k + NC - 1
     return kFgBufs * stage + recv + bins + recv_bins;
 }
+// an SM has 228 KB, 1 KB of it reserved per thread block
+static_assert(kSoleSmem + 1024 + kFgBufs * 2 * 64 * tc::ROW_BYTES + 64 * 64 * 4 + 1024 > 228 * 1024, "no block of this kernel beside one of a pair");
 
 bool cluster_path_fits(const LayerDesc* d, int32_t L, ClusterPlan* plan)
 {

@@ -134,6 +134,11 @@ grass_status launch_sjlt_table(const void* g, grass_dtype dt, int64_t n, int64_t
 // varies asks for the right to this much in every call: the limit is the process's, and another thread, with another size,
 // may be between this call's setting and its launch.
 constexpr size_t kDynSmemLimit = 226 * 1024;
+// Least dynamic shared memory of the kernels that run in pairs of thread blocks with all of tensor memory.  It leaves no room for a
+// block of the FactGraSS cluster kernel on the same SM (calls on two streams may run at once): of such a block and a pair, each
+// could otherwise hold the columns that the other's partner waits for.  (The remaining pairs of kernels that wait for other thread
+// blocks have columns for all that shared memory and registers let in.)
+constexpr size_t kSoleSmem = 196 * 1024;
 
 // launch-shape override set through grass_set_tuning, or `dflt` while the key is on automatic
 int64_t tuning(grass_tuning_key key, int64_t dflt);

@@ -41,6 +41,7 @@ constexpr uint32_t COLS = 512;                 // all of tensor memory: two accu
 constexpr int64_t MAX_RUN = 8192;              // k-values per accumulator run when D > 16,384
 
 constexpr int SCRATCH_BYTES = EPI_WARPS * 32 * 16 * 4;         // the epilogue warps' transposition buffers, behind the stages
+static_assert(kSoleSmem <= SMEM_BUDGET + SCRATCH_BYTES, "what the kernel asks the right to");
 
 struct Plan {
     WorkPlan work;         // k tiles of KW * 64 k-values, one stage each
@@ -314,7 +315,7 @@ grass_status launch_score_bf16(const void* train, int64_t N, int64_t ld_train, c
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3((unsigned)(2 * used), 1, 1);
         cfg.blockDim = dim3(THREADS_H, 1, 1);
-        cfg.dynamicSmemBytes = (size_t)p.stages * stage_bytes + SCRATCH_BYTES;
+        cfg.dynamicSmemBytes = std::max(kSoleSmem, (size_t)p.stages * stage_bytes + SCRATCH_BYTES);
         cfg.stream = st;
         cudaLaunchAttribute attr[1] = {early_launch()};
         cfg.attrs = attr;

@@ -114,3 +114,25 @@ def test_recorded_calls(G, name):
         graph.replay()
     torch.cuda.synchronize()
     assert _same(outs[1], ref) and _same(-outs[0], ref)
+
+
+# calls that take tensor memory, on two streams at once: clusters of the layer's blocks beside pairs of the score's
+@pytest.mark.parametrize("M", [96, 192, 400])
+def test_layers_beside_scores(G, M):
+    A = torch.randn((3, 200, 200), device="cuda").to(torch.bfloat16)
+    Gr = torch.randn((3, 200, 300), device="cuda").to(torch.bfloat16)
+    mi, mo = (G.mask_to_device(G.grass_random_mask_host(d, 64, d)) for d in (200, 300))
+    train = torch.randn((900, 1_024), device="cuda").to(torch.bfloat16)
+    test = torch.randn((M, 1_024), device="cuda").to(torch.bfloat16)
+    layer = lambda: G.factgrass_compress(A, Gr, mi, mo, 512, 1, 5)
+    score = lambda: G.grass_score_bf16(train, test)
+    ref_l, ref_s = layer(), score()
+    torch.cuda.synchronize()
+    streams = [torch.cuda.Stream(), torch.cuda.Stream()]
+    outs = [], []
+    for _ in range(40):
+        for call, stream, out in zip((layer, score), streams, outs):
+            with torch.cuda.stream(stream):
+                out.append(call())
+    torch.cuda.synchronize()
+    assert all(_same(o, ref_l) for o in outs[0]) and all(_same(o, ref_s) for o in outs[1])
