@@ -305,6 +305,8 @@ grass_status grass_fim(const float* X, int64_t n, int64_t k, int64_t ld, float* 
  * Preconditioned scores <g_test, F^-1 g_i> = <F^-1 g_test, g_i>: apply to the (few) test rows, then call
  * grass_score(train, solved_test).  fp32 throughout: the relative error grows with the condition
  * number of F + lambda*I.
+ * grass_fim_apply has no dev_status argument: should one of its bounded waits ever expire, the rows that were solved
+ * together with it (up to 32) are filled with NaN.
  */
 grass_status grass_fim_factor(float* F, int64_t k, int64_t ld_f, float lambda, uint32_t* dev_status, void* stream);
 grass_status grass_fim_apply(const float* L, int64_t k, int64_t ld_f, float* Bm, int64_t M, int64_t ld_b,
@@ -356,7 +358,8 @@ typedef enum {
     GRASS_TUNE_COMPRESS_THREADS = 13,  /* grass_compress gather path: threads per block (256, 512, 1024) */
     GRASS_TUNE_COMPRESS_IDX_SMEM = 14, /* grass_compress gather path: 0 = never copy the index list into shared memory */
     GRASS_TUNE_SCORE_BF16_SOLO = 15,   /* grass_score_bf16: accepted, without effect (thread-block pairs take every shape) */
-    GRASS_TUNE_COUNT = 16
+    GRASS_TUNE_FIM_EXPIRE = 16,        /* grass_fim_apply: the thread block of every cluster (0 .. 7) that takes its waits as expired */
+    GRASS_TUNE_COUNT = 17
 } grass_tuning_key;
 #define GRASS_TUNE_AUTO (-1)
 grass_status grass_set_tuning(grass_tuning_key key, int64_t value);

@@ -206,3 +206,18 @@ def test_fim_shapes(G, n, k, off):
     # six bf16 products keep each product to 2^-23; accumulators are truncated once per 16 samples
     assert ((F - ref).abs() <= 2.0 ** -22 * absum + 2.0 * (n / 16 + 64) ** 0.5 * 2.0 ** -23 * absum).all()
     assert (F - F.T).abs().max() <= 2.0 ** -21 * absum.max()
+
+
+# A wait that expires in one thread block of a cluster spoils what the others go on with: all rows of all clusters are NaN, whichever
+# block it was, and the next call is sound.  (The block takes its waits as expired without having waited, and then waits.)
+@pytest.mark.parametrize("k,M,block", [(1_030, 40, 0), (1_030, 40, 5), (300, 33, 2), (130, 700, 1)])
+def test_expired_wait_leaves_no_finite_row(G, tune, k, M, block):
+    F = G.grass_fim(_compressed(k + 64, k, 80 + k))
+    G.grass_fim_factor(F, 0.1)
+    B = _compressed(M, k, 81 + k)
+    ref = G.grass_fim_apply(F, B.clone())
+    tune(fim_expire=block)
+    got = G.grass_fim_apply(F, B.clone())
+    tune(fim_expire=None)
+    assert torch.isnan(got).all()
+    assert torch.equal(G.grass_fim_apply(F, B.clone()), ref)
