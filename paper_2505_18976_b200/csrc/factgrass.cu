@@ -486,7 +486,7 @@ static grass_status run_factgrass(const factgrass_layer* layers, int32_t L, gras
     }
     if (cluster_nc > 0)
         return launch_factgrass_cluster(dev_descs, single, cplan, L, B, T, tok_begin, tok_count, cluster_nc,
-                                        cluster_chunk, out, ld_out, dev_status, st, out_bf16);
+                                        cluster_chunk, out, ld_out, dev_status, sms, st, out_bf16);
     // A bf16 row is rounded once, at the final store, so the streaming kernel takes it only where one thread block
     // owns a whole (layer, sample): one block tile, the whole token sum (at most 8,192 tokens), bins in shared memory
     if (out_bf16 && (max_tiles > 1 || max_k != max_k_smem || T > 8192 || epi != kEpiSjlt)) return GRASS_ERR_UNSUPPORTED;

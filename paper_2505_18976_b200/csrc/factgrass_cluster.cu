@@ -469,7 +469,7 @@ int cluster_capacity(int nc)
 grass_status launch_factgrass_cluster(const LayerDesc* dev_descs, const LayerDesc& single, const ClusterPlan& plan,
                                       int32_t L, int32_t B, int32_t T, const int64_t* tok_begin,
                                       const int32_t* tok_count, int32_t nc, int32_t chunk_len, float* out,
-                                      int64_t ld_out, uint32_t* dev_status, cudaStream_t st, int out_bf16)
+                                      int64_t ld_out, uint32_t* dev_status, int sms, cudaStream_t st, int out_bf16)
 {
     auto launch = [&](auto kern) -> grass_status {
         // the same limit in every call: another thread may be between this and its launch
@@ -499,9 +499,6 @@ grass_status launch_factgrass_cluster(const LayerDesc* dev_descs, const LayerDes
         cfg.attrs = attr;
         // not behind the copy of a descriptor table, and not with more than one thread block per SM: the next call's would take the
         // places that are left and be spread unevenly
-        int dev = 0, sms = 0;
-        if (cuda_failed(cudaGetDevice(&dev)) || cuda_failed(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)))
-            return GRASS_ERR_CUDA;
         cfg.numAttrs = !dev_descs && (int64_t)nc * B * L <= sms ? 2 : 1;
         cudaError_t e = cudaLaunchKernelEx(&cfg, kern, dev_descs, single, T, tok_begin, tok_count, chunk_len, out,
                                            ld_out, dev_status, out_bf16);

@@ -57,7 +57,7 @@ int cluster_capacity(int nc);
 grass_status launch_factgrass_cluster(const LayerDesc* dev_descs, const LayerDesc& single, const ClusterPlan& plan,
                                       int32_t L, int32_t B, int32_t T, const int64_t* tok_begin,
                                       const int32_t* tok_count, int32_t nc, int32_t chunk_len, float* out,
-                                      int64_t ld_out, uint32_t* dev_status, cudaStream_t st, int out_bf16);
+                                      int64_t ld_out, uint32_t* dev_status, int sms, cudaStream_t st, int out_bf16);
 
 // The persistent kernel (factgrass_persistent.cu).  persistent_fits: every layer of the call is one block of at most
 // 128 x 128 whose projection can be a table.  table: device scratch of persistent_table_bytes(L).
