@@ -104,8 +104,7 @@ def test_preconditioned_score(G, oracle_mod):
 
 
 # Sizes at which the one-launch kernels change shape: one block, one block and a row, a last block of one row; the first
-# trailing update just within / beyond one thread block per tile (k = 1,088 / 1,152); clusters of 1, 2, 4, 8 and
-# 2 .. 32 right-hand sides each; row strides that rule out 16-byte loads.
+# trailing update just within / beyond one thread block per tile (k = 1,088 / 1,152); row strides that rule out 16-byte loads.
 @pytest.mark.parametrize("k,M,pad", [(1, 1, 0), (63, 2, 1), (64, 40, 0), (65, 5, 3), (128, 600, 4), (129, 33, 1), (320, 1, 0),
                                      (576, 130, 2), (1088, 260, 0), (1152, 300, 1), (1345, 37, 4), (256, 5000, 0)])
 def test_factor_and_apply_shapes(G, k, M, pad):
@@ -221,3 +220,57 @@ def test_expired_wait_leaves_no_finite_row(G, tune, k, M, block):
     tune(fim_expire=None)
     assert torch.isnan(got).all()
     assert torch.equal(G.grass_fim_apply(F, B.clone()), ref)
+
+
+# Every number of right-hand sides per cluster with every number of thread blocks, whichever the sizes would choose: as many blocks
+# of 64 columns as thread blocks and one more (the buffers of the solved blocks come round), the last one ragged or whole, and
+# several rounds; rows that leave one over, a last cluster of one row; strides that rule out 16-byte copies.
+@pytest.mark.parametrize("rows", [2, 4, 8, 16, 32])
+@pytest.mark.parametrize("blocks", [1, 2, 4, 8])
+def test_apply_every_cluster_shape(G, tune, blocks, rows):
+    for k, M, pad in ((64 * blocks, 2 * rows + 1, 0), (64 * blocks + 1, rows, 1), (64 * (2 * blocks + 1) + 37, 3 * rows - 1, 3),
+                      (64 * (3 * blocks + 2), rows + 1, 4)):
+        X = _compressed(2 * k + 3, k, 90 + k)
+        F = torch.full((k, k + pad), float("nan"), device="cuda")[:, :k]
+        G.grass_fim(X, out=F)
+        A = F.double() + 0.05 * torch.eye(k, device="cuda", dtype=torch.float64)
+        G.grass_fim_factor(F, 0.05)
+        wide = torch.full((M + 1, k + pad), float("nan"), device="cuda")
+        Bm = wide[:M, :k]
+        Bm.copy_(_compressed(M, k, 91 + k))
+        b = Bm.double()
+        tune(fim_rows=rows, fim_cluster=blocks)
+        G.grass_fim_apply(F, Bm)
+        assert torch.isnan(wide[M]).all() and (pad == 0 or torch.isnan(wide[:, k:]).all())
+        x = Bm.double()
+        # the bound of test_factor_and_apply_shapes
+        u = 6.0 * k ** 0.5 * 2.0 ** -24
+        assert (x @ A - b).norm() <= u * A.norm() * x.norm(), (k, M)
+        # row by row, so that no row hides behind the others
+        assert ((x @ A - b).norm(dim=1) <= 4.0 * u * A.norm() * x.norm(dim=1)).all(), (k, M)
+
+
+# The block columns' path takes few right-hand sides as well: one row, a last tile of one row, a ragged last block
+@pytest.mark.parametrize("k,M,pad", [(1, 1, 0), (64, 65, 0), (130, 1, 3), (193, 129, 1)])
+def test_apply_block_columns_of_few_rows(G, tune, k, M, pad):
+    F = torch.full((k, k + pad), float("nan"), device="cuda")[:, :k]
+    G.grass_fim(_compressed(2 * k + 3, k, 97 + k), out=F)
+    A = F.double() + 0.05 * torch.eye(k, device="cuda", dtype=torch.float64)
+    G.grass_fim_factor(F, 0.05)
+    B = _compressed(M, k, 98 + k)
+    tune(fim_cluster=0)
+    x = G.grass_fim_apply(F, B.clone()).double()
+    u = 6.0 * k ** 0.5 * 2.0 ** -24
+    assert (x @ A - B.double()).norm() <= u * A.norm() * x.norm()
+
+
+# ... and the sizes' own choice where it is one of the larger shapes (32 rows in one block and in two, 16 in eight)
+@pytest.mark.parametrize("k,M", [(64, 2_500), (1_216, 1_200), (1_792, 1_750), (1_280, 140), (512, 8), (500, 2_900)])
+def test_apply_sizes_of_the_larger_shapes(G, k, M):
+    F = G.grass_fim(_compressed(2 * k + 3, k, 95 + k))
+    A = F.double() + 0.05 * torch.eye(k, device="cuda", dtype=torch.float64)
+    G.grass_fim_factor(F, 0.05)
+    B = _compressed(M, k, 96 + k)
+    x = G.grass_fim_apply(F, B.clone()).double()
+    u = 6.0 * k ** 0.5 * 2.0 ** -24
+    assert (x @ A - B.double()).norm() <= u * A.norm() * x.norm()
