@@ -360,7 +360,7 @@ typedef enum {
     GRASS_TUNE_SCORE_BF16_SOLO = 15,   /* grass_score_bf16: accepted, without effect (thread-block pairs take every shape) */
     GRASS_TUNE_FIM_EXPIRE = 16,        /* grass_fim_apply: the thread block of every cluster (0 .. 7) that takes its waits as expired */
     GRASS_TUNE_FIM_ROWS = 17,          /* grass_fim_apply: right-hand sides per cluster (2, 4, 8, 16, 32) */
-    GRASS_TUNE_FIM_CLUSTER = 18,       /* grass_fim_apply: thread blocks per cluster (1, 2, 4, 8; no more than blocks of 64 in k); 0 = no clusters, block column by block column */
+    GRASS_TUNE_FIM_CLUSTER = 18,       /* grass_fim_apply: thread blocks per cluster (1, 2, 4, 8; at most k / 64); 0 = block column by block column */
     GRASS_TUNE_COUNT = 19
 } grass_tuning_key;
 #define GRASS_TUNE_AUTO (-1)

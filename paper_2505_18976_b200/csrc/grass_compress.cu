@@ -69,8 +69,8 @@ grass_compress_kernel(const T* __restrict__ g, int64_t n, int64_t p, int64_t ld,
     __shared__ __align__(8) unsigned long long idx_bar;
     uint32_t* sidx = reinterpret_cast<uint32_t*>(bins + (use_smem ? ((size_t)S * k + 3) / 4 * 4 : 0));
     const uint32_t idx_bulk = idx_smem_bytes ? (uint32_t)((kprime * 4) & ~(int64_t)15) : 0u;
-    // The launch lies under the end of the kernel before (calls one after the other: one row of k' = 8,192 6.15 -> 4.96 us, 256 rows
-    // 16.1 -> 15.1).  Zeroing the bins ahead of the wait as well gained another 0.1 us there, but cost registers that the bf16
+    // The launch lies under the end of the kernel before (calls one after the other: one row of k' = 8,192 6.15 -> 5.0 us, 256 rows
+    // 16.1 -> 15.2).  Zeroing the bins ahead of the wait as well gained another 0.1 us there, but cost registers that the bf16
     // gathers do not have (61 rows of k' = 32,768: 32.0 us, 33.9 so).
     early_wait();
     early_go();

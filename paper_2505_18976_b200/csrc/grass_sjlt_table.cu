@@ -8,8 +8,9 @@
 //   per row in shared memory; the cost of that follows the non-zeros (Section 3.1).  The (rows, chunk) units are cut
 //   evenly over the blocks, so there is no last wave; a row that two blocks share is added into zeroes.
 // What bounds it: for dense inputs the shared-memory fp32 additions, each a compare-and-swap; HBM for sparse ones (99 % zeros: 5.5
-// TB/s).  Between the two neither accounts for all of the time: at 70 % zeros HBM needs 86 of 154 us and the additions, at the
-// rate that a kernel of nothing else showed, 89, and the rows and the table pass through the same shared memory.
+// TB/s).  In between the additions, the rows and the table share the pipe to shared memory: at 70 % zeros it is busy for 73 % of the
+// cycles (DRAM 44 %), 70 % of that with additions (a warp's takes 5.4 cycles for ten active lanes: one to read, four to swap, and
+// repeats) and 29 % with rows and table; the warps wait for its answers.
 // 1,024 x 131,072, k = 4,096, against the streamed path: fp32 230 -> 154 us at 70 % zeros, 109 -> 97 at 99 %;
 // bf16 303 -> 139; k = 32,768 615 -> 202.
 // (Turning the projection around instead, lists of positions per bucket summed without atomics, was built and measured:
