@@ -102,6 +102,23 @@ __device__ __forceinline__ void store_out(float* out, int64_t off, float v, int 
     else out[off] = v;
 }
 
+// four consecutive outputs, at a multiple of four elements; vec: out and its row stride allow one store
+__device__ __forceinline__ void store_out4(float* out, int64_t off, const float4& v, int out_bf16, bool vec)
+{
+    if (!vec) {
+        store_out(out, off, v.x, out_bf16);
+        store_out(out, off + 1, v.y, out_bf16);
+        store_out(out, off + 2, v.z, out_bf16);
+        store_out(out, off + 3, v.w, out_bf16);
+    } else if (out_bf16) {
+        const __nv_bfloat162 a = __floats2bfloat162_rn(v.x, v.y), b = __floats2bfloat162_rn(v.z, v.w);
+        *reinterpret_cast<uint2*>(reinterpret_cast<__nv_bfloat16*>(out) + off) =
+            make_uint2(*reinterpret_cast<const uint32_t*>(&a), *reinterpret_cast<const uint32_t*>(&b));
+    } else {
+        *reinterpret_cast<float4*>(out + off) = v;
+    }
+}
+
 template <typename T> struct elem;
 template <> struct elem<float> {
     static __device__ __forceinline__ float load(const float* p)
