@@ -192,7 +192,7 @@ factgrass_cluster_kernel(const LayerDesc* __restrict__ descs, const __grid_const
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
-    for (uint32_t i = tid; i < k; i += kFgThreads) bins[i] = 0.0f;
+    for (uint32_t i = 4 * tid; i < k; i += 4 * kFgThreads) *reinterpret_cast<float4*>(bins + i) = make_float4(0.0f, 0.0f, 0.0f, 0.0f);   // (rounded up to four)
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     early_go();                                           // (this block has its tensor memory)
@@ -380,16 +380,32 @@ factgrass_cluster_kernel(const LayerDesc* __restrict__ descs, const __grid_const
     asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 
     // reduce: slice o of the accumulator goes to thread block o's second receive area ...
-    if (nc_ok) {
+    const bool quads = nc_ok && k % (4 * nc) == 0;            // slices of whole groups of four bins (32 x 512 tokens, 768 x 3,072: 26.64 us one by one, 26.40 so)
+    if (quads) {
+        for (uint32_t i = 4 * tid; i < k; i += 4 * kFgThreads) {
+            const uint32_t o = i / per;
+            *reinterpret_cast<float4*>(cluster.map_shared_rank(recv_bins, o) + rank * per + (i - o * per)) = *reinterpret_cast<const float4*>(bins + i);
+        }
+    } else if (nc_ok) {
         for (uint32_t i = tid; i < k; i += kFgThreads) {
             const uint32_t o = i / per;
             cluster.map_shared_rank(recv_bins, o)[rank * per + (i - o * per)] = bins[i];
         }
     }
     cluster.sync();      // ... and after this barrier nobody touches another thread block's memory
-    if (nc_ok) {
-        const int64_t orow = (int64_t)b * ld_out + L.out_offset;
-        const uint32_t lo = rank * per, hi = min(lo + per, k);
+    const int64_t orow = (int64_t)b * ld_out + L.out_offset;
+    const uint32_t lo = rank * per, hi = min(lo + per, k);
+    if (quads) {
+        const bool vec = orow % 4 == 0 && (uintptr_t)out % (out_bf16 ? 8 : 16) == 0;
+        for (uint32_t i = 4 * tid; i < per; i += 4 * kFgThreads) {
+            float4 acc = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+            for (uint32_t q = 0; q < nc; ++q) {
+                const float4 x = *reinterpret_cast<const float4*>(recv_bins + q * per + i);
+                acc.x += x.x; acc.y += x.y; acc.z += x.z; acc.w += x.w;
+            }
+            store_out4(out, orow + lo + i, acc, out_bf16, vec);
+        }
+    } else if (nc_ok) {
         for (uint32_t i = lo + tid; i < hi; i += kFgThreads) {
             float acc = 0.0f;
             for (uint32_t q = 0; q < nc; ++q) acc += recv_bins[q * per + (i - lo)];
