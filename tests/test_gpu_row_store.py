@@ -30,3 +30,18 @@ def test_rows_of_any_length_and_alignment(n, k, off, pad, out_dtype):
     if out_dtype == torch.bfloat16:
         tol = tol + 2.0 ** -8 * ref.abs()
     assert ((out - ref).abs() <= tol).all()
+
+
+# grass_fim stores four entries at a time in whole tiles off the diagonal: tiles at the edge, few tiles and many (added up by several
+# clusters), rows that begin off a 16-byte boundary
+@pytest.mark.parametrize("n,k,pad", [(300, 256, 0), (300, 256, 1), (300, 257, 3), (5_000, 1_024, 0), (5_000, 1_024, 2), (5_000, 900, 4)])
+def test_fim_rows_of_any_alignment(n, k, pad):
+    gen = torch.Generator("cuda").manual_seed(n + k)
+    X = torch.randn((n, k), generator=gen, device="cuda")
+    wide = torch.full((k, k + pad), 7.0, device="cuda")
+    F = G.grass_fim(X, out=wide[:, :k]).double()
+    assert (wide[:, k:] == 7.0).all()
+    Xd = X.double()
+    ref, absum = Xd.T @ Xd / n, Xd.abs().T @ Xd.abs() / n
+    # six bf16 products keep each product to 2^-23; accumulators are truncated once per 16 samples
+    assert ((F - ref).abs() <= 2.0 ** -22 * absum + 2.0 * (n / 16 + 64) ** 0.5 * 2.0 ** -23 * absum).all()
