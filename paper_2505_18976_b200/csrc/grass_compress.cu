@@ -466,7 +466,8 @@ static grass_status launch_compress(const T* g, int64_t n, int64_t p, int64_t ld
     if (pl.idx_smem) smem = (smem + 15) / 16 * 16 + pl.idx_smem;       // a copy of the index list
     const float scale = 1.0f / sqrtf((float)sp.s);
     auto launch = [&](auto kern) -> grass_status {
-        if (smem > 48 * 1024) {
+        // without this a block may have 48 KB, and idx_bar is part of them (k' = 8,192, k = 4,096: bins and list are 48 KB by themselves)
+        if (smem > 47 * 1024) {
             cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDynSmemLimit);
             if (cuda_failed(e)) return GRASS_ERR_CUDA;
         }
