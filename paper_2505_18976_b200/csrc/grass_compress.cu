@@ -17,6 +17,7 @@
 #include <cooperative_groups.h>
 
 #include <algorithm>
+#include <type_traits>
 
 namespace cg = cooperative_groups;
 
@@ -46,7 +47,17 @@ __device__ __forceinline__ void load4(const __nv_bfloat16* p, float (&v)[4])
 // DENSE: identity mask on vector-aligned rows (plain SJLT, the k' = p case of Section 3.3.1).  Rows are then
 // streamed with vector loads, four consecutive positions per thread, and S > 1 samples share each hash.
 // NT: threads per CTA (the gather path runs with 256, 512 or 1,024; the streamed path always with kThreads).
-template <typename T, int S, int U, bool S1, bool DENSE, int NT>
+// FORM: which of its launches an instance of the gather is for.  2,048 threads per SM leave a thread 32 registers, and what one
+// launch needs (global reductions, positions of 64 bits, the ways to store a row) costs the loads of another.  In us, one instance for
+// all and these: 256 rows of k' = 8,192, p = 65,536, stored one by one (odd row stride) and four at a time, k = 2,048 19.6 and 19.4,
+// 19.1 and 18.8; k = 16,384 29.5 and 24.2, 21.0 and 20.4; k = 32,768 41.7 and 29.3, 28.7 and 27.1; clusters: one row of k' = 8,192,
+// k = 2,048 4.85, 4.23; 61 rows of bf16, k' = 32,768, k = 8,192 32.9, 30.8; 512 rows of k' = 65,536, k = 4,096 199, 173.  Slower: 888
+// rows of k' = 8,192, k = 2,048 48.9, 50.2; 17 of k = 20,000 13.4, 13.5.
+constexpr int kAny = 0;         // every launch
+constexpr int kRows = 1;        // one block owns a row (bins in shared memory, plain stores)
+constexpr int kRows4 = 2;       // the same, rows stored four at a time: k, their stride and their address allow it
+constexpr int kCluster = 3;     // a cluster owns a row
+template <typename T, int S, int U, bool S1, bool DENSE, int NT, int FORM = kAny>
 __global__ void __launch_bounds__(NT, DENSE ? 4 : (U >= 16 ? 1024 : 2048) / NT)
 grass_compress_kernel(const T* __restrict__ g, int64_t n, int64_t p, int64_t ld,
                       const uint32_t* __restrict__ idx, int64_t kprime, uint32_t k, uint32_t s,
@@ -54,14 +65,21 @@ grass_compress_kernel(const T* __restrict__ g, int64_t n, int64_t p, int64_t ld,
                       int64_t j_per_cta, int accumulate, int use_smem, uint32_t* dev_status, int out_bf16,
                       uint32_t idx_smem_bytes)
 {
-    extern __shared__ __align__(16) float bins[];  // S * k when use_smem
+    extern __shared__ __align__(16) float bins[];  // S * k when use_smem, rounded up to four
+    constexpr bool whole = FORM == kRows || FORM == kRows4;
+    if (FORM != kAny) {
+        use_smem = 1;
+        accumulate = whole ? 0 : 2;
+        if (!whole) idx_smem_bytes = 0;
+    }
+    using pos_t = std::conditional_t<FORM == kAny, int64_t, uint32_t>;      // positions of the gather
     int tid = threadIdx.x;
     constexpr int nthr = NT;
     static_assert(!DENSE || NT == kThreads, "the streamed path is written for kThreads threads");
     const int64_t i0 = (int64_t)blockIdx.x * S;
     const int ns = (int)((n - i0) < (int64_t)S ? (n - i0) : (int64_t)S);
-    const int64_t j0 = (int64_t)blockIdx.y * j_per_cta;
-    const int64_t j1 = (j0 + j_per_cta) < kprime ? (j0 + j_per_cta) : kprime;
+    const int64_t j0 = whole ? 0 : (int64_t)blockIdx.y * j_per_cta;
+    const int64_t j1 = whole || (j0 + j_per_cta) >= kprime ? kprime : (j0 + j_per_cta);
 
     // Whole-row thread blocks keep the index list in shared memory (idx_smem_bytes > 0: one bulk copy, started
     // before anything else): every thread block of the launch reads the whole list, and hundreds of them asking L2
@@ -85,11 +103,8 @@ grass_compress_kernel(const T* __restrict__ g, int64_t n, int64_t p, int64_t ld,
         }
     }
     if (use_smem)
-        for (uint32_t i = 4 * tid; i < (uint32_t)S * k; i += 4 * nthr) {
-            if (i + 4 <= (uint32_t)S * k) *reinterpret_cast<float4*>(bins + i) = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-            else
-                for (uint32_t e = i; e < (uint32_t)S * k; ++e) bins[e] = 0.0f;
-        }
+#pragma unroll 1
+        for (uint32_t i = 4 * tid; i < (uint32_t)S * k; i += 4 * nthr) *reinterpret_cast<float4*>(bins + i) = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
     if (idx_smem_bytes)
         for (int64_t j = idx_bulk / 4 + tid; j < kprime; j += nthr) sidx[j] = __ldg(idx + j);   // at most 3 entries
     if (use_smem || idx_smem_bytes) __syncthreads();
@@ -221,14 +236,14 @@ grass_compress_kernel(const T* __restrict__ g, int64_t n, int64_t p, int64_t ld,
         }
     } else
     // the trip count is the same for every lane of a warp (the warp votes below)
-    for (int64_t jw = j0 + (tid & ~31); jw < j1; jw += (int64_t)nthr * U) {
-        const int64_t jb = jw + (tid & 31);
+    for (pos_t jw = (pos_t)j0 + (tid & ~31); jw < (pos_t)j1; jw += (pos_t)nthr * U) {
+        const pos_t jb = jw + (tid & 31);
         uint32_t col[U];
         bool ok[U];
 #pragma unroll
         for (int u = 0; u < U; ++u) {
-            const int64_t j = jb + (int64_t)u * nthr;
-            ok[u] = j < j1;
+            const pos_t j = jb + (pos_t)u * nthr;
+            ok[u] = j < (pos_t)j1;
             uint32_t c = 0;
             if (ok[u]) c = idx_in_smem ? sidx[j] : (idx ? __ldg(idx + j) : (uint32_t)j);
             if ((int64_t)c >= p) { bad = bad || ok[u]; ok[u] = false; c = 0; }
@@ -255,7 +270,7 @@ grass_compress_kernel(const T* __restrict__ g, int64_t n, int64_t p, int64_t ld,
                     float x = v[0][0];
 #pragma unroll
                     for (int t = 1; t < U; ++t) x = (u == t) ? v[t][0] : x;
-                    const uint64_t j = (uint64_t)(jb + (int64_t)u * nthr);
+                    const uint64_t j = (uint64_t)(jb + (pos_t)u * nthr);
                     const uint32_t draws = S1 ? 1u : s;
                     for (uint32_t r = 0; r < draws; ++r) {
                         const uint64_t h = sjlt_hash_counter(seed, S1 ? (j + 1) : (j * s + r + 1));
@@ -276,7 +291,7 @@ grass_compress_kernel(const T* __restrict__ g, int64_t n, int64_t p, int64_t ld,
 #pragma unroll
                 for (int si = 0; si < S; ++si) any = any || (v[u][si] != 0.0f);
                 if (!any) continue;
-                const uint64_t j = (uint64_t)(jb + (int64_t)u * nthr);
+                const uint64_t j = (uint64_t)(jb + (pos_t)u * nthr);
                 const uint32_t draws = S1 ? 1u : s;
                 for (uint32_t r = 0; r < draws; ++r) {
                     const uint64_t h = sjlt_hash_counter(seed, S1 ? (j + 1) : (j * s + r + 1));
@@ -315,8 +330,6 @@ grass_compress_kernel(const T* __restrict__ g, int64_t n, int64_t p, int64_t ld,
         cluster.sync();  // nobody leaves while its bins may still be read
     } else if (use_smem) {
         __syncthreads();
-        // Four bins at a time, as they are emptied (256 x 65,536, k' = 8,192, k = 2,048: 15.2 us one at a time, 14.6 so; one row 4.99, 4.83)
-        const bool vec_out = ld_out % 4 == 0 && (uintptr_t)out % (out_bf16 ? 8 : 16) == 0;
         for (int si = 0; si < ns; ++si) {
             float* dst = out + (i0 + si) * ld_out;
             const float* src = bins + (uint32_t)si * k;
@@ -325,9 +338,10 @@ grass_compress_kernel(const T* __restrict__ g, int64_t n, int64_t p, int64_t ld,
                     const float x = src[i];
                     if (x != 0.0f) atomicAdd(dst + i, x);
                 }
-            } else if (k % 4 == 0) {
+            } else if (FORM == kRows4) {
+#pragma unroll 1
                 for (uint32_t i = 4 * tid; i < k; i += 4 * nthr)
-                    store_out4(out, (i0 + si) * ld_out + i, *reinterpret_cast<const float4*>(src + i), out_bf16, vec_out);
+                    store_out4(out, (i0 + si) * ld_out + i, *reinterpret_cast<const float4*>(src + i), out_bf16, true);
             } else {
                 for (uint32_t i = tid; i < k; i += nthr) store_out(out, (i0 + si) * ld_out + i, src[i], out_bf16);
             }
@@ -461,7 +475,7 @@ static grass_status launch_compress(const T* g, int64_t n, int64_t p, int64_t ld
     if (pl.dense) j_per_cta = (j_per_cta + 3) / 4 * 4;      // vector loads start on multiples of four positions
     // 0: one CTA owns the row, plain stores; 1: global reductions into a zeroed row; 2: cluster reduction
     const int accumulate = pl.cluster ? 2 : ((pl.jsplit > 1 || !pl.use_smem) ? 1 : 0);
-    size_t smem = pl.use_smem ? (size_t)S * sp.k * sizeof(float) : 0;
+    size_t smem = pl.use_smem ? ((size_t)S * sp.k + 3) / 4 * 16 : 0;
     if (pl.dense) smem = ((smem + 7) & ~(size_t)7) + kQueueBytes;      // the warps' non-zero queues
     if (pl.idx_smem) smem = (smem + 15) / 16 * 16 + pl.idx_smem;       // a copy of the index list
     const float scale = 1.0f / sqrtf((float)sp.s);
@@ -499,16 +513,29 @@ static grass_status launch_compress(const T* g, int64_t n, int64_t p, int64_t ld
         if (sp.s == 1) return launch(grass_compress_kernel<T, S, U, true, true, kThreads>);
         return launch(grass_compress_kernel<T, S, U, false, true, kThreads>);
     }
-    if (pl.threads == 2 * kThreads) {
-        if (sp.s == 1) return launch(grass_compress_kernel<T, S, U, true, false, 2 * kThreads>);
-        return launch(grass_compress_kernel<T, S, U, false, false, 2 * kThreads>);
+    auto gather = [&](auto form) -> grass_status {
+        constexpr int F = decltype(form)::value;
+        if (pl.threads == 2 * kThreads) {
+            if (sp.s == 1) return launch(grass_compress_kernel<T, S, U, true, false, 2 * kThreads, F>);
+            return launch(grass_compress_kernel<T, S, U, false, false, 2 * kThreads, F>);
+        }
+        if (pl.threads == 4 * kThreads) {
+            if (sp.s == 1) return launch(grass_compress_kernel<T, S, U, true, false, 4 * kThreads, F>);
+            return launch(grass_compress_kernel<T, S, U, false, false, 4 * kThreads, F>);
+        }
+        if (sp.s == 1) return launch(grass_compress_kernel<T, S, U, true, false, kThreads, F>);
+        return launch(grass_compress_kernel<T, S, U, false, false, kThreads, F>);
+    };
+    if constexpr (S == 1 && U == 8) {
+        if (pl.use_smem && kprime < 0x7FFF0000) {          // (a block's last round of positions ends within 32 bits)
+            if (accumulate == 2) return gather(std::integral_constant<int, kCluster>{});
+            if (accumulate == 0) {
+                const bool four = sp.k % 4 == 0 && ld_out % 4 == 0 && (uintptr_t)out % (pl.out_bf16 ? 8 : 16) == 0;
+                return four ? gather(std::integral_constant<int, kRows4>{}) : gather(std::integral_constant<int, kRows>{});
+            }
+        }
     }
-    if (pl.threads == 4 * kThreads) {
-        if (sp.s == 1) return launch(grass_compress_kernel<T, S, U, true, false, 4 * kThreads>);
-        return launch(grass_compress_kernel<T, S, U, false, false, 4 * kThreads>);
-    }
-    if (sp.s == 1) return launch(grass_compress_kernel<T, S, U, true, false, kThreads>);
-    return launch(grass_compress_kernel<T, S, U, false, false, kThreads>);
+    return gather(std::integral_constant<int, kAny>{});
 }
 
 template <typename T>
