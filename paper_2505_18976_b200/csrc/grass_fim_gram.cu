@@ -16,7 +16,7 @@
 // What bounds it: the six products (12 MMAs of 64 cycles per step and SM) once two thread blocks per SM hide the
 // loads and the split of each other.  It still runs at about half that rate: shared memory serves the MMAs' operand
 // reads (128 bytes a cycle at M = N = 128) and the split's stores.  Measured against the gathering kernel used before
-// (4-byte loads, column by column): n = 4,656, k = 1,024 117 -> 54 us, 48 with its results stored four at a time, n = 16,384, k = 4,096 2,090 -> 1,675 us.
+// (4-byte loads, column by column): n = 4,656, k = 1,024 117 -> 54 us, 46 with its results stored four at a time, n = 16,384, k = 4,096 2,090 -> 1,675 us.
 #include "factgrass_common.cuh"
 
 #include <cooperative_groups.h>
@@ -38,6 +38,7 @@ constexpr int STAGE = 2 * STRIP;              // 48 KB
 constexpr uint32_t LBO = (STEP / 8) * 1024;   // bytes between blocks of 64 columns
 constexpr uint32_t SBO = 1024;                // bytes between groups of 8 samples
 constexpr uint32_t ACC_COLS = 2 * TILE;
+static_assert(THREADS % TILE == 0, "the rows of a thread stay the same");
 constexpr int CHUNKS = TILE / 8;              // 16-byte chunks (8 columns) per sample
 constexpr int PER_THREAD = STEP * CHUNKS / THREADS;    // chunks per thread, strip and step (2)
 static_assert(PER_THREAD * THREADS == STEP * CHUNKS, "even split");
@@ -57,11 +58,13 @@ __device__ __forceinline__ uint64_t make_desc(uint32_t addr)
     return (uint64_t)((addr >> 4) & 0x3FFF) | ((uint64_t)(LBO >> 4) << 16) | ((uint64_t)(SBO >> 4) << 32) | (1ull << 46) |
            (2ull << 61);
 }
-// where element (row, c) of a slice sits: 16-byte chunks xor-ed with the row, so that the writers (lanes on
-// consecutive rows) and the readers (lanes on consecutive chunks) are both free of bank conflicts
+// where element (row, c) of a slice sits: 16-byte chunks xor-ed with the row, so that the writers (lanes on consecutive rows) and the
+// readers of rows (lanes on consecutive chunks) are free of bank conflicts.  The readers of four rows of a column (lanes four rows
+// apart) are too at 16 and 32 rows to a slice, meet in pairs at 64 and four at a time at 128; without bits 3 and 4 of the row two,
+// four, eight and sixteen at a time.
 __device__ __forceinline__ int slice_offset(int row, int c)
 {
-    return row * TILE + ((((c >> 2) ^ (row & 7)) << 2) | (c & 3));
+    return row * TILE + ((((c >> 2) ^ (row & 7) ^ ((row >> 2) & 2) ^ ((row >> 4) & 1)) << 2) | (c & 3));
 }
 
 __global__ void __launch_bounds__(THREADS, 2)
@@ -251,16 +254,16 @@ gram_kernel(const float* __restrict__ X, int32_t n, int32_t k, int64_t ld, int32
     }
     __syncthreads();
     if (whole) {
-        for (int e = tid; e < R * TILE / 4; e += THREADS) {
-            const int row = e % (R / 4) * 4, c = e / (R / 4);      // consecutive threads: consecutive columns of the mirror image
+        // consecutive threads: consecutive columns of the mirror image (R / 4 divides THREADS: the rows of a thread stay the same)
+        const int row = tid % (R / 4) * 4;
+        for (int c = tid / (R / 4); c < TILE; c += THREADS / (R / 4))
             emit4(c_base + c, a_base + row, make_float4(recv[slice_offset(row, c)], recv[slice_offset(row + 1, c)],
                                                         recv[slice_offset(row + 2, c)], recv[slice_offset(row + 3, c)]));
-        }
         return;
     }
-    for (int e = tid; e < R * TILE; e += THREADS) {
-        const int row = e % R, c = e / R;
-        const int a = a_base + row, cc = c_base + c;
+    const int row = tid % R, a = a_base + row;
+    for (int c = tid / R; c < TILE; c += THREADS / R) {
+        const int cc = c_base + c;
         if (a < k && cc < k && (!diag || a < cc)) emit(cc, a, recv[slice_offset(row, c)]);
     }
 }
