@@ -32,8 +32,10 @@ def test_factgrass_cluster_result_anywhere(k, off, pad, out_dtype):
     D = torch.randn((B, T, d_out), generator=gen, device="cuda").to(torch.bfloat16)
     mi, mo = (G.mask_to_device(G.grass_random_mask_host(d, m, d)) for d, m in ((d_in, 64), (d_out, 48)))
     wide = torch.full((B, off + k + pad), 7.0, device="cuda", dtype=out_dtype)
+    layers = G.GroupedLayers([dict(A=A, G=D, mask_in=mi, mask_out=mo, k=k, s=1, seed=99, out_offset=0)])
+    ws = torch.empty(G.factgrass_grouped_workspace_bytes(1), dtype=torch.uint8, device="cuda")
     with G.tuning(factgrass_path=1):
-        out = G.factgrass_compress(A, D, mi, mo, k, 1, 99, out=wide[:, off:off + k]).double()
+        out = G.factgrass_compress_grouped(layers, wide[:, off:off + k], ws).double()
     assert (wide[:, :off] == 7.0).all() and (wide[:, off + k:] == 7.0).all()
     a, d = A[:, :, mi.long()].double(), D[:, :, mo.long()].double()
     bucket, sign = G.grass_sjlt_table(k, 1, 99, a.shape[2] * d.shape[2])
