@@ -177,6 +177,14 @@ def _need_cuda(*ts) -> None:
             raise ValueError("device tensors required (the library has no CPU path)")
 
 
+def _need_f32_rows(out: torch.Tensor) -> None:
+    """Results that a call writes as fp32, row by row."""
+    if out.dtype != torch.float32:
+        raise TypeError(f"the result is written as float32, not {out.dtype}")
+    if out.dim() > 1 and out.shape[-1] > 1 and out.stride(-1) != 1:
+        raise ValueError("the rows of the result must be contiguous")
+
+
 def _need_device_readable(*ts) -> None:
     """Inputs the kernels only gather from: device tensors, or page-locked host tensors (which the device
     addresses directly; the kernels then pull the masked elements across the bus)."""
@@ -263,6 +271,7 @@ def factgrass_compress(A: torch.Tensor, G: torch.Tensor, mask_in: torch.Tensor, 
     assert G.shape[:2] == (B, T) and A.dtype == G.dtype
     if out is None:
         out = torch.empty((B, k), dtype=torch.float32, device=_compute_device(A))
+    _need_f32_rows(out)
     spec = SjltSpec(k, s, seed & 0xFFFFFFFFFFFFFFFF)
     _check(lib().factgrass_compress(_ptr(A), _ptr(G), _dt(A), B, T, d_in, d_out, _ptr(mask_in), mask_in.numel(),
                                     _ptr(mask_out), mask_out.numel(), ctypes.byref(spec), _ptr(out),
@@ -301,6 +310,7 @@ def factgrass_compress_varlen(A: torch.Tensor, G: torch.Tensor, mask_in: torch.T
         assert A.numel() >= B * T_max * d_in and G.numel() >= B * T_max * d_out
     if out is None:
         out = torch.empty((B, k), dtype=torch.float32, device=_compute_device(A))
+    _need_f32_rows(out)
     spec = SjltSpec(k, s, seed & 0xFFFFFFFFFFFFFFFF)
     _check(lib().factgrass_compress_varlen(_ptr(A), _ptr(G), _dt(A), B, T_max, _ptr(tok_begin), _ptr(tok_count),
                                            d_in, d_out, _ptr(mask_in), mask_in.numel(), _ptr(mask_out),
@@ -421,6 +431,7 @@ def grass_score(train: torch.Tensor, test: torch.Tensor, out: Optional[torch.Ten
     assert test.shape[1] == D
     if out is None:
         out = torch.empty((N, M), dtype=torch.float32, device=train.device)
+    _need_f32_rows(out)
     _check(lib().grass_score(_ptr(train), N, train.stride(0) if N > 1 else D, _ptr(test), M,
                              test.stride(0) if M > 1 else D, D, _ptr(out), out.stride(0) if N > 1 else M,
                              _stream()), "grass_score")
@@ -455,6 +466,7 @@ def grass_score_bf16(train: torch.Tensor, test: torch.Tensor, out: Optional[torc
     assert test.shape[1] == D
     if out is None:
         out = torch.empty((N, M), dtype=torch.float32, device=train.device)
+    _need_f32_rows(out)
     _check(lib().grass_score_bf16(_ptr(train), N, train.stride(0) if N > 1 else D, _ptr(test), M,
                                   test.stride(0) if M > 1 else D, D, _ptr(out), out.stride(0) if N > 1 else M,
                                   _stream()), "grass_score_bf16")
@@ -473,6 +485,7 @@ def grass_mask(g: torch.Tensor, idx: torch.Tensor, out: Optional[torch.Tensor] =
     kp = idx.numel()
     if out is None:
         out = torch.empty((n, kp), dtype=torch.float32, device=_compute_device(g))
+    _need_f32_rows(out)
     _check(lib().grass_mask(_ptr(g), _dt(g), n, p, ld, _ptr(idx), kp, _ptr(out),
                             out.stride(0) if n > 1 else max(out.shape[1], kp), _ptr(dev_status), _stream()), "grass_mask")
     return out
@@ -493,6 +506,7 @@ def factmask_compress(A: torch.Tensor, G: torch.Tensor, mask_in: torch.Tensor, m
     kp = kin * kout
     if out is None:
         out = torch.empty((B, kp), dtype=torch.float32, device=_compute_device(A))
+    _need_f32_rows(out)
     _check(lib().factmask_compress(_ptr(A), _ptr(G), _dt(A), B, T, d_in, d_out, _ptr(mask_in), kin,
                                    _ptr(mask_out), kout, _ptr(out),
                                    out.stride(0) if B > 1 else max(out.shape[1], kp), _ptr(dev_status), _stream()),
