@@ -22,7 +22,7 @@
 //
 // What bounds it: DRAM for the gathers (32 x 512 tokens, 768 x 3,072, 128 x 128: 14.4 us for 100 MB of 64-byte pieces), and
 // around them 3 us until the first loads are out and 9 us of exchange, projection and reduction, which nothing
-// overlaps in a launch of one wave: 28.3 us in all (28.9 with the exchange by plain stores).
+// overlaps in a launch of one wave: 26.2 us in all (the exchange by plain stores: 0.6 us more).
 #include "factgrass_common.cuh"
 
 #include <cooperative_groups.h>
@@ -380,7 +380,7 @@ factgrass_cluster_kernel(const LayerDesc* __restrict__ descs, const __grid_const
     asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 
     // reduce: slice o of the accumulator goes to thread block o's second receive area ...
-    const bool quads = nc_ok && k % (4 * nc) == 0;            // slices of whole groups of four bins (32 x 512 tokens, 768 x 3,072: 26.64 us one by one, 26.40 so)
+    const bool quads = nc_ok && k % (4 * nc) == 0;            // slices of whole groups of four bins (32 x 512 tokens, 768 x 3,072, one by one and so: k = 4,096 26.5 us, 26.2; 8,192 28.5, 27.6; the same with an odd row stride)
     if (quads) {
         for (uint32_t i = 4 * tid; i < k; i += 4 * kFgThreads) {
             const uint32_t o = i / per;

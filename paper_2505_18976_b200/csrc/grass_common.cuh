@@ -102,7 +102,8 @@ __device__ __forceinline__ void store_out(float* out, int64_t off, float v, int 
     else out[off] = v;
 }
 
-// four consecutive outputs, at a multiple of four elements; vec: out and its row stride allow one store
+// four consecutive outputs, at a multiple of four elements; vec: out and its row stride allow one store.  Without it lanes four elements
+// apart cost the short slices of a cluster nothing, but whole rows a third (grass_compress.cu stores those by consecutive lanes)
 __device__ __forceinline__ void store_out4(float* out, int64_t off, const float4& v, int out_bf16, bool vec)
 {
     if (!vec) {

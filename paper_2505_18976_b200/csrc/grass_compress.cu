@@ -404,9 +404,9 @@ static CompressPlan plan_compress(int64_t n, int64_t p, int64_t kprime, uint32_t
     const int64_t groups = (n + S - 1) / S;
     // With a row for every SM, a thread block of up to 1,024 threads takes a whole row in one round of loads: no
     // position split, so no cluster, no exchange of bins and no thread blocks left waiting for a slot
-    // (256 x 65,536, k' = 8,192: 25.2 -> 22.9 us).  Everything else runs 512 threads: the loads in flight per SM come
-    // from resident threads, and a few long rows then keep the machine busy (61 rows of k' = 32,768: 55 us with
-    // 256 threads, 33 us with 512).
+    // (256 x 65,536, k' = 8,192: 16.9 us over two blocks of 512 threads or four of 256, 14.5 over one).  Everything else runs
+    // 512 threads: the loads in flight per SM come from resident threads, and a few long rows then keep the machine busy (61
+    // rows of k' = 32,768: 54 us with 256 threads, 31 us with 512).
     pl.threads = kThreads;
     bool whole = false;
     if (!dense) {
@@ -419,13 +419,13 @@ static CompressPlan plan_compress(int64_t n, int64_t p, int64_t kprime, uint32_t
     }
     // Split of the positions over a cluster of up to 8 thread blocks.  A block's share has to be worth its k bins (zeroed,
     // exchanged and stored): at least k positions, k / 2 while there are fewer blocks than SMs and k / 4 while the next split
-    // has room beside the rest (one block per SM, two with bins of up to 48 KB), and at least 1,024 (one row of k' = 8,192, k =
-    // 2,048: 8.2 us over 4 blocks, 6.2 us over 8; 17 rows of k' = 8,192, k = 20,000: 14.4 us over one, 10.3 over 4; 512 rows of
-    // k' = 65,536: 345 us over 2 blocks, 332 us over 8), and a full round of loads once the blocks fill the machine (318 rows
-    // of k' = 10,510, k = 1,000 in bf16: 47 us over 8 blocks, 36 over 2), half of one where the next split would (100 rows of
-    // k' = 9,000, k = 700: 18.4 over 8, 16.6 over 4).  Many rows under a mask of every second element or more are not split:
-    // their loads are short (3,000 rows of 33,000 elements, all kept, k = 2,048: 413 us over 8 blocks, 261 over one; 600 rows of
-    // 200,000 elements, every second kept: 287 over one, 261 over 8).
+    // has room beside the rest (one block per SM, two with bins of up to 48 KB), and at least 1,024 (17 rows of k' = 8,192, k =
+    // 20,000, which the line leaves at one block: 11.1 us, 7.9 over 4; 512 rows of k' = 65,536: 338 us over 2 blocks, 323 us
+    // over 8; one row of k' = 8,192, k = 2,048: 4.7 us over 4 blocks, 4.8 over 8), and a full round of loads once the blocks
+    // fill the machine (318 rows of k' = 10,510, k = 1,000 in bf16: 43 us over 8 blocks, 41 over 2), half of one where the next
+    // split would (100 rows of k' = 9,000, k = 700: 16.7 over 8, 14.5 over 4).  Many rows under a mask of every second element
+    // or more are not split: their loads are short (3,000 rows of 33,000 elements, all kept, k = 2,048: 345 us over 8 blocks,
+    // 258 over one; 600 rows of 200,000 elements, every second kept: 236 over one, 170 over 8).
     // Streamed rows, and rows without bins in shared memory, keep one full round of 256 threads' loads per block and go up to
     // four blocks per SM; under sparse masks the latter run 256 threads once their rows make that many (671 rows of k' =
     // 100,000 of 800,000, k = 200,000: 524 us, 613 with 512 threads; 1,024 whole rows of 65,536, k = 60,000: 641 and 504).
@@ -447,8 +447,8 @@ static CompressPlan plan_compress(int64_t n, int64_t p, int64_t kprime, uint32_t
     pl.cluster = 1;
     if (groups * js < sm_count && js * 2 <= max_js && (js == 8 || groups * 16 <= sm_count)) {
         // Very few samples: split wider than a cluster allows and reduce with global atomics, as many blocks as are resident
-        // with their bins (2 rows of k' = 100,000, k = 30,000: 31 us over 2 blocks each, 10.4 over 48; 5 rows at k = 50,000, where
-        // an SM holds one block: 31 us over 2, 15.4 over 24, 19.5 over 48).
+        // with their bins (2 rows of k' = 100,000, k = 30,000: 42 us over 2 blocks each, 10.4 over 48; 5 rows at k = 50,000, where
+        // an SM holds one block: 59 us over 2, 14.4 over 29, 19.2 over 48).
         js = std::min((sm_count * 2 + groups - 1) / groups, std::max<int64_t>(1, sm_count * fit / groups));
         if (js > max_js) js = max_js;
         pl.cluster = 0;

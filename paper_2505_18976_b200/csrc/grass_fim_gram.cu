@@ -225,12 +225,14 @@ gram_kernel(const float* __restrict__ X, int32_t n, int32_t k, int64_t ld, int32
         if (add_out) atomicAdd(p, x); else *p = x;
     };
     // four entries of a row of F at once where it allows that (vec_f), which a tile on the diagonal or at the edge does not (n = 4,656,
-    // k = 1,024, four clusters to a tile: 54.0 us entry by entry, 47.7 so)
+    // k = 1,024, four clusters to a tile: 54.0 us entry by entry, 47.7 so, 45.7 without the bank conflicts of the mirror image)
     auto emit4 = [&](int64_t r, int64_t c, const float4& x) {
         float* p = F + r * ld_f + c;
         if (!add_out) *reinterpret_cast<float4*>(p) = x;
         else asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(p), "f"(x.x), "f"(x.y), "f"(x.z), "f"(x.w) : "memory");
     };
+    // The others leave entry by entry, by the thread that added up the four: one after the other by consecutive lanes, from slice 0 and
+    // behind a barrier, was slower (k = 1,023 54.1 us, 55.3 so; k = 2,050 244, 247).
     const bool whole = vec_f && !diag && a_base + R <= k && c_base + TILE <= k;
     for (int e = tid; e < R * CHUNKS * 2; e += THREADS) {
         const int row = e / (CHUNKS * 2), c = e % (CHUNKS * 2) * 4, off = slice_offset(row, c);
@@ -245,7 +247,8 @@ gram_kernel(const float* __restrict__ X, int32_t n, int32_t k, int64_t ld, int32
         if (whole) {
             emit4(a, cc, x);
         } else {
-            // a tile on the diagonal keeps its upper half and mirrors it, so that F is symmetric to the bit
+            // a tile on the diagonal keeps its upper half and mirrors it, so that F is symmetric to the bit (where one cluster has the
+            // tile: what several add into it arrives in any order)
             const float y[4] = {x.x, x.y, x.z, x.w};
 #pragma unroll
             for (int u = 0; u < 4; ++u)
@@ -288,8 +291,9 @@ grass_status launch_fim(const float* X, int64_t n, int64_t k, int64_t ld, float 
     int64_t want = std::max<int64_t>(1, slots / ntiles);
     want = std::min<int64_t>(want, std::max<int64_t>(1, n / (4 * STEP)));
     want = std::max<int64_t>(want, (n + 8191) / 8192);
-    // With many tiles, pairs: wide clusters leave SMs of a partition idle (36 tiles: 58 us with pairs and 75 with eights
-    // at n = 4,656, k = 1,024); with few tiles, eights save global reductions (3 tiles: 18 against 30 us at n = 512).
+    // With many tiles, pairs: wide clusters leave SMs of a partition idle (36 tiles: 46 us with pairs, 66 with fours and 67 with
+    // eights at n = 4,656, k = 1,024; 21 tiles, k = 768: 36, 38 and 42); with few tiles, eights save global reductions (10 tiles:
+    // 12.5 us, 14.6 with fours and 19.7 with pairs at n = 512, k = 512).
     int64_t cs = 1;
     // (eight also where there are too few samples for them: each stores an eighth of the tile)
     while (cs < (ntiles >= 16 ? 2 : 8) && (cs * 2 <= want || ntiles < 16)) cs *= 2;
