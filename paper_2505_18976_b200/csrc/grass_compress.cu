@@ -48,15 +48,16 @@ __device__ __forceinline__ void load4(const __nv_bfloat16* p, float (&v)[4])
 // streamed with vector loads, four consecutive positions per thread, and S > 1 samples share each hash.
 // NT: threads per CTA (the gather path runs with 256, 512 or 1,024; the streamed path always with kThreads).
 // FORM: which of its launches an instance of the gather is for.  2,048 threads per SM leave a thread 32 registers, and what one
-// launch needs (global reductions, positions of 64 bits, the ways to store a row) costs the loads of another.  In us, one instance for
-// all and these: 256 rows of k' = 8,192, p = 65,536, stored one by one (odd row stride) and four at a time, k = 2,048 19.6 and 19.4,
-// 19.1 and 18.8; k = 16,384 29.5 and 24.2, 21.0 and 20.4; k = 32,768 41.7 and 29.3, 28.7 and 27.1; clusters: one row of k' = 8,192,
-// k = 2,048 4.85, 4.23; 61 rows of bf16, k' = 32,768, k = 8,192 32.9, 30.8; 512 rows of k' = 65,536, k = 4,096 199, 173.  Slower: 888
-// rows of k' = 8,192, k = 2,048 48.9, 50.2; 17 of k = 20,000 13.4, 13.5.
+// launch needs (stores of a row, global reductions, positions of 64 bits) costs the loads of another.  In us, one instance for all and
+// these: 256 rows of k' = 8,192, p = 65,536, stored one by one (odd row stride) and four at a time, k = 2,048 19.6 and 19.4, 19.4 and
+// 18.8; k = 16,384 29.6 and 24.2, 21.1 and 20.5; k = 32,768 41.6 and 29.2, 29.1 and 27.7; 888 rows, k = 2,048 49.1, 47.1; clusters:
+// one row of k' = 8,192, k = 2,048 4.86, 4.26; 61 rows of bf16, k' = 32,768, k = 8,192 32.9, 30.7; 512 rows of k' = 65,536, k = 4,096
+// 198, 171; wide: 7 rows of k' = 1.3 M, k = 2,268 57.2, 52.
 constexpr int kAny = 0;         // every launch
 constexpr int kRows = 1;        // one block owns a row (bins in shared memory, plain stores)
 constexpr int kRows4 = 2;       // the same, rows stored four at a time: k, their stride and their address allow it
 constexpr int kCluster = 3;     // a cluster owns a row
+constexpr int kWide = 4;        // more blocks than a cluster has add into a zeroed row
 template <typename T, int S, int U, bool S1, bool DENSE, int NT, int FORM = kAny>
 __global__ void __launch_bounds__(NT, DENSE ? 4 : (U >= 16 ? 1024 : 2048) / NT)
 grass_compress_kernel(const T* __restrict__ g, int64_t n, int64_t p, int64_t ld,
@@ -69,7 +70,7 @@ grass_compress_kernel(const T* __restrict__ g, int64_t n, int64_t p, int64_t ld,
     constexpr bool whole = FORM == kRows || FORM == kRows4;
     if (FORM != kAny) {
         use_smem = 1;
-        accumulate = whole ? 0 : 2;
+        accumulate = whole ? 0 : (FORM == kCluster ? 2 : 1);
         if (!whole) idx_smem_bytes = 0;
     }
     using pos_t = std::conditional_t<FORM == kAny, int64_t, uint32_t>;      // positions of the gather
@@ -78,8 +79,8 @@ grass_compress_kernel(const T* __restrict__ g, int64_t n, int64_t p, int64_t ld,
     static_assert(!DENSE || NT == kThreads, "the streamed path is written for kThreads threads");
     const int64_t i0 = (int64_t)blockIdx.x * S;
     const int ns = (int)((n - i0) < (int64_t)S ? (n - i0) : (int64_t)S);
-    const int64_t j0 = whole ? 0 : (int64_t)blockIdx.y * j_per_cta;
-    const int64_t j1 = whole || (j0 + j_per_cta) >= kprime ? kprime : (j0 + j_per_cta);
+    const int64_t j0 = (int64_t)blockIdx.y * j_per_cta;
+    const int64_t j1 = (j0 + j_per_cta) < kprime ? (j0 + j_per_cta) : kprime;
 
     // Whole-row thread blocks keep the index list in shared memory (idx_smem_bytes > 0: one bulk copy, started
     // before anything else): every thread block of the launch reads the whole list, and hundreds of them asking L2
@@ -103,7 +104,6 @@ grass_compress_kernel(const T* __restrict__ g, int64_t n, int64_t p, int64_t ld,
         }
     }
     if (use_smem)
-#pragma unroll 1
         for (uint32_t i = 4 * tid; i < (uint32_t)S * k; i += 4 * nthr) *reinterpret_cast<float4*>(bins + i) = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
     if (idx_smem_bytes)
         for (int64_t j = idx_bulk / 4 + tid; j < kprime; j += nthr) sidx[j] = __ldg(idx + j);   // at most 3 entries
@@ -246,7 +246,8 @@ grass_compress_kernel(const T* __restrict__ g, int64_t n, int64_t p, int64_t ld,
             ok[u] = j < (pos_t)j1;
             uint32_t c = 0;
             if (ok[u]) c = idx_in_smem ? sidx[j] : (idx ? __ldg(idx + j) : (uint32_t)j);
-            if ((int64_t)c >= p) { bad = bad || ok[u]; ok[u] = false; c = 0; }
+            // (p fits 32 bits; the forms that add into global memory are faster with the wider comparison)
+            if (whole || FORM == kCluster ? c >= (uint32_t)p : (int64_t)c >= p) { bad = bad || ok[u]; ok[u] = false; c = 0; }
             col[u] = c;
         }
         float v[U][S];
@@ -339,7 +340,6 @@ grass_compress_kernel(const T* __restrict__ g, int64_t n, int64_t p, int64_t ld,
                     if (x != 0.0f) atomicAdd(dst + i, x);
                 }
             } else if (FORM == kRows4) {
-#pragma unroll 1
                 for (uint32_t i = 4 * tid; i < k; i += 4 * nthr)
                     store_out4(out, (i0 + si) * ld_out + i, *reinterpret_cast<const float4*>(src + i), out_bf16, true);
             } else {
@@ -528,6 +528,7 @@ static grass_status launch_compress(const T* g, int64_t n, int64_t p, int64_t ld
     };
     if constexpr (S == 1 && U == 8) {
         if (pl.use_smem && kprime < 0x7FFF0000) {          // (a block's last round of positions ends within 32 bits)
+            if (accumulate == 1) return gather(std::integral_constant<int, kWide>{});
             if (accumulate == 2) return gather(std::integral_constant<int, kCluster>{});
             if (accumulate == 0) {
                 const bool four = sp.k % 4 == 0 && ld_out % 4 == 0 && (uintptr_t)out % (pl.out_bf16 ? 8 : 16) == 0;

@@ -1,4 +1,4 @@
-"""grass_compress by its forms of launch (a block per row, stored four at a time or one by one; a cluster per row): remainders of rows and
+"""grass_compress by its forms of launch (a block per row, stored four at a time or one by one; a cluster per row; many blocks): remainders of rows and
 masks, several draws, no mask, and what rows that rule out 16-byte stores cost."""
 import pytest
 import torch
@@ -54,10 +54,17 @@ def _time(pad, k, g, idx):
 
 
 # A row of odd stride is stored by lanes on consecutive elements.  (Lanes four elements apart, as they once were: 22 and 49 % slower than
-# rows that take 16-byte stores, where this is 3 and 6 %.)
+# rows that take 16-byte stores, where this is 3 and 7 %.)
 @pytest.mark.parametrize("k", [16_384, 40_000])
 def test_cost_of_rows_off_a_boundary(k):
     g = [torch.randn((256, 65_536), device="cuda") for _ in range(5)]
     idx = G.mask_to_device(G.grass_random_mask_host(65_536, 8_192, 3))
     _time(0, k, g, idx)
     assert _time(1, k, g, idx) < 1.15 * _time(0, k, g, idx)
+
+
+# few rows under long masks: more blocks than a cluster has, adding into a zeroed row (fp32 only: a bf16 row is rounded once)
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("n,p,kprime,k,s,off,pad", [(2, 300_001, 209_525, 752, 1, 3, 1), (7, 200_000, 131_073, 2_267, 1, 4, 4), (3, 150_000, 0, 3_000, 2, 0, 1)])
+def test_wide_splits(n, p, kprime, k, s, off, pad, dtype):
+    _check(n, p, kprime, k, s, off, pad, dtype, torch.float32)
